@@ -35,11 +35,18 @@ __global__ void chi_weights_kernel(const double* __restrict__ ev, const double* 
 namespace {
 constexpr int TB = 64;   // tile edge (G)
 constexpr int KB = 16;   // pairs per shared-memory slice
+// Real products of one 16-pair slice stay with the FMA kernel (device time per
+// call, N_G 300 / 2120: 27 / 82 us against 44 / 115 us on the tensor cores; with
+// a second slice 43 / 147 against 45 / 117).  Complex products are faster on the
+// tensor cores from the first pair on (76 / 283 against 57 / 171).
+constexpr long long kFmaRealPairs = 16;
 }
 
 __global__ void __launch_bounds__(256) chi_f64_kernel(const double2* __restrict__ M, long long K, int ng,
                                                       const double* __restrict__ w, double scale,
-                                                      int accumulate, double2* __restrict__ chi) {
+                                                      int accumulate, const int* __restrict__ guard,
+                                                      double2* __restrict__ chi) {
+  if (guard && !*guard) return;   // the tensor cores did this frequency
   __shared__ double2 As[KB][TB];
   __shared__ double2 Bs[KB][TB];
   // lower-triangle tile (I >= J) from the linear block index
@@ -123,7 +130,9 @@ __global__ void __launch_bounds__(256) chi_f64_kernel(const double2* __restrict_
 // mirrored; 4x4 register blocking as the complex kernel.
 __global__ void __launch_bounds__(256) chi_f64_real_kernel(const double* __restrict__ M, long long K, int ng,
                                                            const double* __restrict__ w, double scale,
-                                                           int accumulate, double* __restrict__ chi) {
+                                                           int accumulate, const int* __restrict__ guard,
+                                                           double* __restrict__ chi) {
+  if (guard && !*guard) return;
   __shared__ double As[KB][TB];
   __shared__ double Bs[KB][TB];
   const long long t = blockIdx.x;
@@ -184,6 +193,23 @@ __global__ void __launch_bounds__(256) chi_f64_real_kernel(const double* __restr
   }
 }
 
+// The FP64 product on the tensor cores where it is the faster one: *flags
+// then holds one device word per frequency, set where the FMA kernel must do
+// it after all (operands that are not finite).  Real products of a few pairs,
+// and calls whose scratch does not fit, leave *flags empty: the FMA kernels do
+// them.
+static int chi_f64_on_tensor_cores(Ctx* c, long long K, int ng, const void* M, const double* wr, const double2* wc,
+                                   int nrow, double scale, int accumulate, void* chi, bool real, Scratch* flags,
+                                   cudaStream_t st) {
+  if (real && K <= kFmaRealPairs) return BGW_OK;
+  void* p = nullptr;
+  if (c->pool.alloc((size_t)nrow * sizeof(int), &p) != BGW_OK) return BGW_OK;
+  const int rc = chi_oz_run(c, K, ng, M, wr, wc, nrow, scale, accumulate, chi, real, static_cast<int*>(p), st);
+  if (rc != BGW_OK) c->pool.release(p);
+  else flags->ptr = p;
+  return rc == BGW_ENOMEM ? BGW_OK : rc;
+}
+
 int chi_mixed_run(Ctx* c, int prec, long long K, int ng, const void* M, const double* w, int nrow,
                   double scale, int accumulate, void* chi, cudaStream_t st, bool real);
 
@@ -207,6 +233,12 @@ int chi_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const doubl
     if (hp && hp->g0 >= 0) return head_wings(c, hp, K, ng, M, h, w.as<double>(), nrow, scale, chi, st);
     return BGW_OK;
   }
+  Scratch flags;
+  flags.pool = &c->pool;
+  if ((rc = chi_f64_on_tensor_cores(c, K, ng, M, w.as<double>(), nullptr, nrow, scale, accumulate, chi, real, &flags,
+                                    st)) != BGW_OK)
+    return rc;
+  const int* guard = flags.as<int>();   // set: the FMA kernels below do the frequencies flagged there
   const int nt = (ng + TB - 1) / TB;
   const long long ntiles = (long long)nt * (nt + 1) / 2;
   if (real) {
@@ -214,7 +246,7 @@ int chi_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const doubl
       TimedScope ts(c, kTChiF64, st);
       chi_f64_real_kernel<<<(unsigned)ntiles, 256, 0, st>>>(static_cast<const double*>(M), K, ng,
                                                              w.as<double>() + (size_t)f * K, scale, accumulate,
-                                                             static_cast<double*>(chi) + (size_t)f * ng * ng);
+                                                             guard ? guard + f : nullptr, static_cast<double*>(chi) + (size_t)f * ng * ng);
       BGW_CUDA(c, cudaGetLastError());
       c->launches += 1;
     }
@@ -224,7 +256,7 @@ int chi_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const doubl
     TimedScope ts(c, kTChiF64, st);
     chi_f64_kernel<<<(unsigned)ntiles, 256, 0, st>>>(static_cast<const double2*>(M), K, ng,
                                                       w.as<double>() + (size_t)f * K, scale, accumulate,
-                                                      static_cast<double2*>(chi) + (size_t)f * ng * ng);
+                                                      guard ? guard + f : nullptr, static_cast<double2*>(chi) + (size_t)f * ng * ng);
     BGW_CUDA(c, cudaGetLastError());
     c->launches += 1;
   }
@@ -263,7 +295,9 @@ __global__ void chi_weights_real_kernel(const double* __restrict__ ev, const dou
 // (grid = nt^2), same register blocking as the Hermitian kernel.
 __global__ void __launch_bounds__(256) chi_f64_general_kernel(const double2* __restrict__ M, long long K, int ng,
                                                               const double2* __restrict__ w, double scale,
-                                                              int accumulate, double2* __restrict__ chi) {
+                                                              int accumulate, const int* __restrict__ guard,
+                                                              double2* __restrict__ chi) {
+  if (guard && !*guard) return;
   __shared__ double2 As[KB][TB];
   __shared__ double2 Bs[KB][TB];
   const int nt = (ng + TB - 1) / TB;
@@ -350,12 +384,18 @@ int chi_real_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const 
   c->launches += 1;
   if (prec != BGW_PREC_FP64)
     return chi_real_mixed_run(c, prec, K, ng, M, w.as<double2>(), nfreq, scale, accumulate, chi, st);
+  Scratch flags;
+  flags.pool = &c->pool;
+  if ((rc = chi_f64_on_tensor_cores(c, K, ng, M, nullptr, w.as<double2>(), nfreq, scale, accumulate, chi, false,
+                                    &flags, st)) != BGW_OK)
+    return rc;
+  const int* guard = flags.as<int>();
   const int nt = (ng + TB - 1) / TB;
   for (int f = 0; f < nfreq; ++f) {
     TimedScope ts(c, kTChiF64, st);
     chi_f64_general_kernel<<<(unsigned)(nt * nt), 256, 0, st>>>(static_cast<const double2*>(M), K, ng,
                                                                  w.as<double2>() + (size_t)f * K, scale,
-                                                                 accumulate,
+                                                                 accumulate, guard ? guard + f : nullptr,
                                                                  static_cast<double2*>(chi) + (size_t)f * ng * ng);
     BGW_CUDA(c, cudaGetLastError());
     c->launches += 1;

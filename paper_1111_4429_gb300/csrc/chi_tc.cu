@@ -31,111 +31,21 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 #include <vector>
 
 #include "runtime.h"
 #include "sweep_common.cuh"
+#include "tc_common.cuh"
 
 namespace bgw {
 
 namespace tc {
 
-constexpr int BM = 128;          // tile rows (G)
 constexpr int BK = 32;           // pairs per TMA box / stage (64 B of 16-bit values)
 constexpr int kEpiWarps = 8;     // epilogue warps of the GEMM kernel (two per tensor-memory lane quadrant)
 constexpr int kThreads = 32 * (kEpiWarps + 2);   // + TMA producer + MMA issuer
-constexpr unsigned long long kWaitNs = 1000000000ull;  // 1 s: default limit of every wait
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait: false when the barrier did not complete within limit_ns or
-// (watch_abort) the CTA is aborting.  A limit of 0 gives up at the first
-// failed try.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                          unsigned long long limit_ns = kWaitNs, bool watch_abort = true) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  while (!mbar_try_wait(bar, parity)) {
-    if (watch_abort && *abort_flag) return false;
-    if (globaltimer() - t0 >= limit_ns) return false;
-  }
-  return true;
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::
-          "r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
-      : "memory");
-}
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor: K-major operand, 64-byte swizzle, rows of
-// 64 bytes, 8-row groups 512 bytes apart.
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);          // start address
-  d |= (uint64_t)1u << 16;                            // leading byte offset (unused here)
-  d |= (uint64_t)((512u >> 4) & 0x3FFFu) << 32;       // stride byte offset: 8 rows x 64 B
-  d |= (uint64_t)1u << 46;                            // descriptor version
-  d |= (uint64_t)4u << 61;                            // SWIZZLE_64B
-  return d;
-}
-
-// Instruction descriptor, kind::f16: FP32 accumulator, A/B FP16 or BF16,
-// K-major A and B, optional negation of A.
-__host__ __device__ constexpr uint32_t idesc(int n, bool bf16, bool neg_a) {
-  return (1u << 4) | ((bf16 ? 1u : 0u) << 7) | ((bf16 ? 1u : 0u) << 10) | ((neg_a ? 1u : 0u) << 13) |
-         ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(id), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 template <int BN, int NP = 4>
 struct Layout {
@@ -788,23 +698,21 @@ __global__ void reduce_rows_kernel(const float* __restrict__ work, int nseg, int
 
 }  // namespace tc
 
-namespace {
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode = nullptr;
-
-int get_encode(Ctx* c) {
-  if (g_encode) return BGW_OK;
-  void* fn = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
-  if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn)
-    return fail(c, BGW_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
-  g_encode = reinterpret_cast<EncodeTiledFn>(fn);
+int tensor_map_encode(Ctx* c, TensorMapEncode* out) {
+  static std::atomic<TensorMapEncode> cached{nullptr};
+  if (!cached.load(std::memory_order_acquire)) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
+    if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn)
+      return fail(c, BGW_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    cached.store(reinterpret_cast<TensorMapEncode>(fn), std::memory_order_release);
+  }
+  *out = cached.load(std::memory_order_acquire);
   return BGW_OK;
 }
 
+namespace {
 constexpr int kBN = 128;
 constexpr int kStages = 3;
 // Default pairs per K segment (FP32 accumulation span before the FP64 sum).
@@ -815,8 +723,6 @@ constexpr int kSegPairsDefault = 512;
 // complex64 M); larger calls are processed chunk by chunk, each chunk's FP64
 // sum added into chi.
 constexpr size_t kChunkBytes = size_t(4) << 30;
-
-namespace {
 
 // Segments per CTA for nseg segments over ntiles tiles: the fewest groups of
 // segments (one FP32 partial per tile and group) whose grid of groups x
@@ -840,6 +746,8 @@ int segs_per_cta(long long nseg, int ntiles, int nsm) {
   return best;
 }
 
+namespace {
+
 // Both products: the Hermitian one (wr: real weights, X = Y = M sqrt|w|,
 // lower tiles, mirrored) and the general one (wc: complex weights, X = M,
 // Y = w M, all tiles).
@@ -848,7 +756,8 @@ int chi_tc_run(Ctx* c, int prec, long long K, int ng, const void* M, const doubl
   using namespace tc;
   const bool general = wc != nullptr;
   int rc;
-  if ((rc = get_encode(c)) != BGW_OK) return rc;
+  TensorMapEncode encode;
+  if ((rc = tensor_map_encode(c, &encode)) != BGW_OK) return rc;
   const int bf16 = prec == BGW_PREC_MIX_BF16;
   const int ntr = (ng + BM - 1) / BM, ntc = (ng + kBN - 1) / kBN;
   const int ngpad = std::max(ntr * BM, ntc * kBN);
@@ -895,7 +804,7 @@ int chi_tc_run(Ctx* c, int prec, long long K, int ng, const void* M, const doubl
   // One map serves both operands: the B box has kBN rows; with kBN == BM the
   // same box height applies.
   static_assert(kBN == BM, "one tensor map per operand height");
-  CUresult cr = g_encode(&tmap, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
+  CUresult cr = encode(&tmap, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
                          planes.ptr, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                          CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -1013,7 +922,8 @@ int chi_mixed_run(Ctx* c, int prec, long long K, int ng, const void* M, const do
 int tc_rows_gemm(Ctx* c, int prec, int R1, int R2, int K, const void* X, const void* Y, void* C, cudaStream_t st) {
   using namespace tc;
   int rc;
-  if ((rc = get_encode(c)) != BGW_OK) return rc;
+  TensorMapEncode encode;
+  if ((rc = tensor_map_encode(c, &encode)) != BGW_OK) return rc;
   const int bf16 = prec == BGW_PREC_MIX_BF16;
   const int rpad = (std::max(R1, R2) + BM - 1) / BM * BM;
   const int kpad = (K + BK - 1) / BK * BK;
@@ -1041,7 +951,7 @@ int tc_rows_gemm(Ctx* c, int prec, int R1, int R2, int K, const void* X, const v
   cuuint64_t gstride[1] = {(cuuint64_t)kpad * 2};
   cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)BM};
   cuuint32_t estr[2] = {1, 1};
-  CUresult cr = g_encode(&tmap, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
+  CUresult cr = encode(&tmap, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
                          planes.ptr, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                          CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

@@ -252,6 +252,13 @@ int chi_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const doubl
             const double* d_ec, int nfreq, const double* d_omega, double scale, int accumulate,
             void* chi, cudaStream_t st, const HeadPlan* hp = nullptr, const double2* h = nullptr,
             bool real = false);
+// FP64 chi on the tensor cores (chi_oz.cu): BGW_ENOMEM when its scratch does
+// not fit (nothing launched), flags[f] set on the device where the FP64 FMA
+// kernel must do frequency f (operands that are not finite).
+int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, const double2* wc, int nrow,
+               double scale, int accumulate, void* chi, bool real, int* flags, cudaStream_t st);
+// Segments of work per CTA for nseg segments over ntiles tiles (chi_tc.cu).
+int segs_per_cta(long long nseg, int ntiles, int nsm);
 // eps~ and its inverse for nmat matrices (per-matrix size, cell and q).
 // tc_update: the sweep's trailing updates run on the tensor cores with
 // FP64-level accuracy (sweep_tc.cu) instead of FP64 FMA.

@@ -240,6 +240,29 @@ __device__ __forceinline__ float2 ff_from_int(double x) {
   return make_float2(hi, sgn ? -lo : lo);
 }
 
+// rint(v 2^(56 - e)) for |v| < 2^e, rounded half to even, from v's own
+// fields in the integer pipe (the FP64 scaling and conversion it replaces run
+// on the SM's slow FP64 pipe): v = m 2^(E - 1075) with the 53-bit mantissa m
+// (no implicit bit below the normal range), so the result is m shifted by
+// E - 1019 - e (at most 3 to the left).
+__device__ __forceinline__ long long fixed56(double v, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int E = (int)((b >> 52) & 0x7FFull);
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (E ? (1ull << 52) : 0ull);
+  const int sh = (E ? E : 1) - 1019 - e;
+  unsigned long long X;
+  if (sh >= 0) {
+    X = m << sh;
+  } else if (sh > -64) {
+    const int k = -sh;
+    const unsigned long long q = m >> k, r = m & ((1ull << k) - 1ull), half = 1ull << (k - 1);
+    X = q + ((r > half || (r == half && (q & 1ull))) ? 1ull : 0ull);
+  } else {
+    X = 0ull;
+  }
+  return (b >> 63) ? -(long long)X : (long long)X;
+}
+
 // -x by the sign bit (no FP64 instruction)
 __device__ __forceinline__ double neg_bits(double x) {
   return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);

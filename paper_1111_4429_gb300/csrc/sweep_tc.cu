@@ -27,6 +27,7 @@
 #include "runtime.h"
 #include "sweep_common.cuh"
 #include "sweep_items.cuh"
+#include "tc_common.cuh"
 
 namespace bgw {
 
@@ -183,29 +184,6 @@ __device__ __forceinline__ void digits7(long long X, __half* out, size_t stride)
 #pragma unroll
   for (int a = 0; a < S; ++a)
     out[a * stride] = __hsub(__ushort_as_half((unsigned short)(0x6600 + d[a])), __ushort_as_half(0x6600));
-}
-
-// rint(v 2^(56 - e)) for |v| < 2^e, rounded half to even, from v's own
-// fields in the integer pipe (the FP64 scaling and conversion it replaces run
-// on the SM's slow FP64 pipe): v = m 2^(E - 1075) with the 53-bit mantissa m
-// (no implicit bit below the normal range), so the result is m shifted by
-// E - 1019 - e (at most 3 to the left).
-__device__ __forceinline__ long long fixed56(double v, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int E = (int)((b >> 52) & 0x7FFull);
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (E ? (1ull << 52) : 0ull);
-  const int sh = (E ? E : 1) - 1019 - e;
-  unsigned long long X;
-  if (sh >= 0) {
-    X = m << sh;
-  } else if (sh > -64) {
-    const int k = -sh;
-    const unsigned long long q = m >> k, r = m & ((1ull << k) - 1ull), half = 1ull << (k - 1);
-    X = q + ((r > half || (r == half && (q & 1ull))) ? 1ull : 0ull);
-  } else {
-    X = 0ull;
-  }
-  return (b >> 63) ? -(long long)X : (long long)X;
 }
 
 // Slices and exponent of one 64-value row held by a warp (lane: value k and
@@ -793,13 +771,6 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
 
 }  // namespace oz
 
-namespace {
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode_oz = nullptr;
-}  // namespace
-
 // Dynamic shared memory of update_pipe_kernel with SL slices: U, two V
 // buffers, alignment slack and the barriers.
 size_t pipe_smem(int slices) { return (size_t)slices * (oz::kUTile + 2 * oz::kVTile) + 1024 + 128; }
@@ -826,14 +797,8 @@ int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2
   plan->slices = slices;
   plan->ff_chain = ff_chain || slices < 7;   // five slices always use the double-FP32 chain
   if (nmat > kBatch) return fail(c, BGW_EUNSUPPORTED, "tensor-core inverse: at most %d matrices per batch", kBatch);
-  if (!g_encode_oz) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess || !fn)
-      return fail(c, BGW_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    g_encode_oz = reinterpret_cast<EncodeTiledFn>(fn);
-  }
+  TensorMapEncode encode;
+  if (int erc = tensor_map_encode(c, &encode)) return erc;
   plan->nmat = nmat;
   plan->general = general;
   plan->real_values = real_values;
@@ -873,10 +838,10 @@ int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2
   cuuint32_t estr[2] = {1, 1};
   cuuint32_t ubox[2] = {(cuuint32_t)KR, (cuuint32_t)BM};
   cuuint32_t vbox[2] = {(cuuint32_t)KR, (cuuint32_t)BN};
-  if (g_encode_oz(&plan->umap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plan->U.ptr, gdim, gstride, ubox, estr,
+  if (encode(&plan->umap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plan->U.ptr, gdim, gstride, ubox, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-      g_encode_oz(&plan->vmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plan->V.ptr, gdim, gstride, vbox, estr,
+      encode(&plan->vmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plan->V.ptr, gdim, gstride, vbox, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return fail(c, BGW_ECUDA, "tensor-core inverse: tensor map encoding failed");

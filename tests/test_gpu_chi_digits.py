@@ -1,0 +1,91 @@
+"""The FP64 polarizability by digit products on the tensor cores: tile edges,
+short and ragged pair counts, accumulation, chunked calls under a small HBM
+budget, and operands that are not finite (the FP64 FMA kernel's)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+CELL = (np.eye(3) * 0.3, 8641.0, (0.1, 0.0, 0.0), 40)
+
+
+def _case(ng, nv, nc, seed, real=False):
+    r = np.random.default_rng(seed)
+    m = r.standard_normal((nv * nc, ng)) + (0 if real else 1j * r.standard_normal((nv * nc, ng)))
+    m = m * np.exp2(r.integers(-20, 20, ng))          # columns of very different sizes
+    return m, np.sort(r.uniform(-0.5, 0.0, nv)), np.sort(r.uniform(0.04, 1.5, nc))
+
+
+def _ref(m, ev, ec, omega):
+    d = np.subtract.outer(ev, ec).ravel()
+    w = 1.0 / d if omega is None else d / (d * d + omega * omega)
+    return (m.conj().T * w) @ m * (4.0 / CELL[1])
+
+
+def _err(x, ref):
+    # per element, against the columns' norms: |chi_GG'| <= (chi_GG chi_G'G')^1/2, so a sum of K terms in FP64
+    # is within K 2^-53 of it (NumPy's reference included), the digit products within 2^-58 (6 K)^1/2 2^2
+    s = np.sqrt(np.abs(np.diagonal(ref)))
+    return np.abs((x - ref) / np.outer(s, s)).max()
+
+
+@pytest.mark.parametrize("real", [False, True])
+@pytest.mark.parametrize("ng,nv,nc", [(1, 1, 8), (31, 2, 4), (32, 3, 5), (33, 1, 16), (127, 1, 17), (128, 4, 48),
+                                      (129, 1, 193), (160, 5, 77), (257, 3, 9), (300, 2, 500)])
+def test_edges_against_numpy(ng, nv, nc, real):
+    from paper_1111_4429_gb300 import bgw
+    ctx, cell = bgw.Context(0), bgw.make_cell(*CELL)
+    m, ev, ec = _case(ng, nv, nc, 17 * ng + nc, real)
+    M = torch.from_numpy(m).cuda()
+    om = np.array([0.0, 0.7])
+    chi = torch.zeros((2, ng, ng), dtype=M.dtype, device="cuda")
+    prec = bgw.BGW_FLAVOR_REAL if real else 0
+    for acc in (False, True):
+        ctx.chi_sum(cell, nv, nc, ng, M, ev, ec, om, prec, acc, chi)
+    ctx.sync()
+    for f in range(2):
+        ref = 2 * _ref(m, ev, ec, om[f])
+        x = chi[f].cpu().numpy()
+        assert _err(x, ref) <= 4 * nv * nc * 2.0 ** -53
+        assert np.array_equal(x, x.conj().T)
+
+
+def test_general_product_and_small_budget():
+    from paper_1111_4429_gb300 import bgw
+    ng, nv, nc = 140, 6, 400
+    m, ev, ec = _case(ng, nv, nc, 5)
+    M = torch.from_numpy(m).cuda()
+    e = np.array([0.3])
+    d = np.subtract.outer(ev, ec).ravel()
+    w = 0.5 * (1 / (d - 0.3 - 0.05j) + 1 / (d + 0.3 + 0.05j))
+    ref = (m.conj().T * w) @ m * (4.0 / CELL[1])
+    s = np.sqrt((np.abs(m) ** 2).sum(0))
+    # whole, in chunks of pairs, and with no room for the digits (FMA kernel)
+    for budget in (0, 24 << 20, 1 << 20):
+        ctx, cell = bgw.Context(0, budget), bgw.make_cell(*CELL)
+        x = torch.zeros((1, ng, ng), dtype=torch.complex128, device="cuda")
+        ctx.chi_sum_real(cell, nv, nc, ng, M, ev, ec, e, 0.05, False, 0, False, x)
+        ctx.sync()
+        got = (x[0].cpu().numpy() - ref) / np.outer(s, s)
+        assert np.abs(got).max() <= nv * nc * 2.0 ** -53 * np.abs(w).max() * 4 / CELL[1]
+        h = torch.zeros((1, ng, ng), dtype=torch.complex128, device="cuda")
+        ctx.chi_sum(cell, nv, nc, ng, M, ev, ec, None, 0, False, h)
+        ctx.sync()
+        assert _err(h[0].cpu().numpy(), _ref(m, ev, ec, None)) <= 2 * nv * nc * 2.0 ** -53
+
+
+def test_values_that_are_not_finite_take_the_fma_kernel():
+    from paper_1111_4429_gb300 import bgw
+    ctx, cell = bgw.Context(0), bgw.make_cell(*CELL)
+    ng, nv, nc = 70, 2, 20
+    m, ev, ec = _case(ng, nv, nc, 9)
+    m[3, 17] = complex(np.inf, 0.0)
+    m[9, 40] = complex(np.nan, 1.0)
+    chi = torch.zeros((1, ng, ng), dtype=torch.complex128, device="cuda")
+    ctx.chi_sum(cell, nv, nc, ng, torch.from_numpy(m).cuda(), ev, ec, None, 0, False, chi)
+    ctx.sync()
+    bad = ~np.isfinite(chi[0].cpu().numpy())
+    rows = np.zeros(ng, bool)
+    rows[[17, 40]] = True
+    assert np.array_equal(bad, rows[:, None] | rows[None, :])
