@@ -131,10 +131,12 @@ bool is_device_ptr(const void* p) {
 // Largest epsilon sphere the gather kernel can hold in shared memory.
 int max_ng(int prec) { return (int)((227 * 1024) / (prec == BGW_PREC_FP64 ? 16 : 8)); }
 
+// Checks the arguments of a matrix-element evaluation; *n_out is the grid its
+// transforms run on.
 int validate_mtxel(Ctx* c, const bgw_cell* cell, int nv, int npw_v, const int32_t* gv, const void* cv, int nc,
                    int npw_c, const int32_t* gc, const void* cc, int ng, const int32_t* geps, int prec, void* M,
                    int* n_out) {
-  int n, rc;
+  int n, rc, need = 0;
   if ((rc = check_cell(c, cell, &n)) != BGW_OK) return rc;
   if ((rc = check_prec(c, prec)) != BGW_OK) return rc;
   if (nv <= 0 || nc <= 0) return fail(c, BGW_EINVAL, "nv and nc must be >= 1");
@@ -146,12 +148,14 @@ int validate_mtxel(Ctx* c, const bgw_cell* cell, int nv, int npw_v, const int32_
   if ((rc = check_glist(c, "gv", npw_v, gv, n, mv)) != BGW_OK) return rc;
   if ((rc = check_glist(c, "gc", npw_c, gc, n, mc)) != BGW_OK) return rc;
   if ((rc = check_glist(c, "geps", ng, geps, n, me)) != BGW_OK) return rc;
-  for (int d = 0; d < 3; ++d)
+  for (int d = 0; d < 3; ++d) {
     if (n <= mv[d] + mc[d] + me[d])
       return fail(c, BGW_EINVAL,
                   "FFT grid %d aliases on axis %d: need n > max|Gv| + max|Gc| + max|Geps| = %d + %d + %d", n, d,
                   mv[d], mc[d], me[d]);
-  *n_out = n;
+    need = std::max(need, mv[d] + mc[d] + me[d] + 1);
+  }
+  *n_out = transform_grid(n, need, ng, geps);
   return BGW_OK;
 }
 
@@ -621,8 +625,8 @@ namespace {
 
 // The whole batch, in stream order on st (no host synchronization once the
 // plans and uploads of its arguments are cached).
-int run_batch(Ctx* c, int nq, const bgw_problem* pr, int nfreq, const double* dev_om, int prec,
-              void* const* epsinv, const std::vector<const void*>& dev_ev, const std::vector<const void*>& dev_ec,
+int run_batch(Ctx* c, int nq, const bgw_problem* pr, const std::vector<int>& grids, int nfreq, const double* dev_om,
+              int prec, void* const* epsinv, const std::vector<const void*>& dev_ev, const std::vector<const void*>& dev_ec,
               const std::vector<const void*>& dev_geps, cudaStream_t st) {
   const int nrow = nfreq > 0 ? nfreq : 1;
   const size_t cs = prec == BGW_PREC_FP64 ? 16 : 8;
@@ -638,7 +642,7 @@ int run_batch(Ctx* c, int nq, const bgw_problem* pr, int nfreq, const double* de
     return fail(c, rc, "bgw_epsilon_batch: scratch allocation failed (M %zu B, chi %zu B)", mbytes, cbytes);
   for (int q = 0; q < nq; ++q) {
     const bgw_problem& p = pr[q];
-    const int n = p.cell.fft[0];
+    const int n = grids[q];
     const BandPlan *bpv, *bpc;
     const PairPlan* pp;
     if ((rc = get_band_plan(c, n, p.npw_v, p.gv, st, &bpv)) != BGW_OK) return rc;
@@ -689,11 +693,12 @@ extern "C" int bgw_epsilon_batch(bgw_ctx* ctx, int nq, const bgw_problem* proble
   if (nfreq < 0 || (nfreq > 0 && !omega)) return fail(c, BGW_EINVAL, "bad frequency list");
   for (int f = 0; f < nfreq; ++f)
     if (!isfinite(omega[f])) return fail(c, BGW_EINVAL, "omega[%d] is not finite", f);
-  int rc, n;
+  int rc;
+  std::vector<int> grids(nq);
   for (int q = 0; q < nq; ++q) {
     const bgw_problem& p = problems[q];
     if ((rc = validate_mtxel(c, &p.cell, p.nv, p.npw_v, p.gv, p.cv, p.nc, p.npw_c, p.gc, p.cc, p.ng, p.geps, prec,
-                             epsinv[q], &n)) != BGW_OK)
+                             epsinv[q], &grids[q])) != BGW_OK)
       return fail(c, rc, "problem %d: %s", q, c->err.c_str());
     if ((rc = check_energies(c, p.nv, p.ev, p.nc, p.ec)) != BGW_OK) return fail(c, rc, "problem %d: %s", q, c->err.c_str());
     if ((rc = check_q(c, &p.cell, p.ng, p.geps)) != BGW_OK) return fail(c, rc, "problem %d: %s", q, c->err.c_str());
@@ -742,7 +747,7 @@ extern "C" int bgw_epsilon_batch(bgw_ctx* ctx, int nq, const bgw_problem* proble
   }
   // Direct run: produces this call's results, creates the plans, tunes and
   // fills the pool with the blocks the capture below will reuse.
-  if ((rc = run_batch(c, nq, problems, nfreq, static_cast<const double*>(dev_om), prec, epsinv, dev_ev, dev_ec,
+  if ((rc = run_batch(c, nq, problems, grids, nfreq, static_cast<const double*>(dev_om), prec, epsinv, dev_ev, dev_ec,
                       dev_geps, st)) != BGW_OK)
     return rc;
   if (st == nullptr || st == cudaStreamLegacy) return BGW_OK;  // the legacy stream cannot be captured
@@ -754,7 +759,7 @@ extern "C" int bgw_epsilon_batch(bgw_ctx* ctx, int nq, const bgw_problem* proble
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    rc = run_batch(c, nq, problems, nfreq, static_cast<const double*>(dev_om), prec, epsinv, dev_ev, dev_ec,
+    rc = run_batch(c, nq, problems, grids, nfreq, static_cast<const double*>(dev_om), prec, epsinv, dev_ev, dev_ec,
                    dev_geps, st);
     e = cudaStreamEndCapture(st, &graph);
   }
@@ -1032,9 +1037,12 @@ int bgw_sigma_cohsex(bgw_ctx* ctx, const bgw_cell* cell, int no, int npw_o, cons
   if ((rc = check_glist(c, "go", npw_o, go, n, mo)) != BGW_OK) return rc;
   if ((rc = check_glist(c, "gi", npw_i, gi, n, mi)) != BGW_OK) return rc;
   if ((rc = check_glist(c, "geps", ng, geps, n, me)) != BGW_OK) return rc;
-  for (int d = 0; d < 3; ++d)
+  int need = 0;
+  for (int d = 0; d < 3; ++d) {
     if (n <= mo[d] + mi[d] + me[d])
       return fail(c, BGW_EINVAL, "FFT grid %d aliases on axis %d: need n > max|Gi| + max|Go| + max|Geps|", n, d);
+    need = std::max(need, mo[d] + mi[d] + me[d] + 1);
+  }
   if ((rc = check_q(c, cell, ng, geps)) != BGW_OK) return rc;
   DeviceGuard g(c->device);
   if (!g.ok) return fail(c, BGW_ECUDA, "cudaSetDevice failed");
@@ -1045,6 +1053,7 @@ int bgw_sigma_cohsex(bgw_ctx* ctx, const bgw_cell* cell, int no, int npw_o, cons
     int tmp[3];
     if ((rc = check_glist(c, "-geps", ng, neg.data(), n, tmp)) != BGW_OK) return rc;
   }
+  n = transform_grid(n, need, ng, neg.data());
   const BandPlan *bpo, *bpi;
   const PairPlan* pp;
   if ((rc = get_band_plan(c, n, npw_o, go, st, &bpo)) != BGW_OK) return rc;

@@ -351,7 +351,7 @@ int sigma_run(Ctx* c, const bgw_cell* cell, int n, int no, const BandPlan* bpo, 
     // product's spectrum (extent of the outer sphere's differences) nor the
     // box aliases.  Where no grid qualifies, the direct sum over the sphere.
     int nr = 0;
-    for (int cand = n; cand <= 64 && nr == 0 && c->sigma_density != 0; ++cand) {
+    for (int cand = 8; cand <= 64 && nr == 0 && c->sigma_density != 0; ++cand) {
       if (!fft_size_supported(cand)) continue;
       bool ok = true;
       for (int d = 0; d < 3; ++d) {
