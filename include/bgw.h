@@ -62,7 +62,9 @@ enum {
 };
 
 /* Precision of a call.
- *  BGW_PREC_FP64     : every step in FP64 / complex128 (the plain path).
+ *  BGW_PREC_FP64     : every step to FP64 accuracy / complex128 (the plain
+ *                      path; chi and the inverse's updates as exact digit
+ *                      products on the tensor cores).
  *  BGW_PREC_MIX_FP16 : M in complex64 (FP32 FFTs); chi on the tensor cores
  *                      as split FP16 (hi*hi + hi*lo + lo*hi) products with
  *                      FP32 accumulation, flushed into an FP64 chi per call;
@@ -164,15 +166,15 @@ int bgw_graph_stats(bgw_ctx* ctx, uint64_t* graphs, uint64_t* replays);
  *    in chunks of this many pairs (rounded down to a multiple of 32), each
  *    chunk's FP64 sum added into chi; 0 (default) sizes chunks so that their
  *    operand planes (as large as the chunk's complex64 M) stay within 4 GiB. */
-/*  BGW_OPT_INVERSE: how the sweep's trailing updates run.  -1 (default):
- *    bgw_epsilon, bgw_epsilon_batch and the server use the tensor cores for
- *    the mixed precisions and FP64 FMA for BGW_PREC_FP64, bgw_epsinv uses
- *    FP64 FMA; 0: FP64 FMA everywhere; 1: the tensor cores everywhere.  The
- *    tensor-core update splits P and C into 8-bit slices held exactly in
- *    FP16 (seven or five, BGW_OPT_UPDATE_SLICES), accumulates every slice
- *    product exactly in FP32 and combines them in double-FP32 before the
- *    FP64 subtraction: with seven its error is near 2^-48 of the update's
- *    scale (FP64 FMA: 2^-53).                                              */
+/*  BGW_OPT_INVERSE: how the sweep's trailing updates run.  -1 (default) and 1:
+ *    on the tensor cores; 0: FP64 FMA.  The tensor-core update splits P and C
+ *    into 8-bit slices held exactly in FP16 (seven or five,
+ *    BGW_OPT_UPDATE_SLICES) and accumulates every slice product exactly in
+ *    FP32.  FP64 inputs (BGW_PREC_FP64, bgw_epsinv*) join the exact sums in
+ *    integers and round once, with errors below those of FP64 FMA; the mixed
+ *    precisions combine them in double-FP32 (with seven slices near 2^-48 of
+ *    the update's scale).  -1 falls back to FP64 FMA for FP64 inputs whose
+ *    slice buffers do not fit the budget.                                  */
 /*  BGW_OPT_HEAD: the q0 head of the mixed precisions.  At a small q0 the
  *    head column M_vc(G = 0) is O(|q0|) while v(q0) = 4 pi / |q0|^2, so the
  *    FP32 FFTs' absolute error on it (near 2^-24 |M|) becomes a relative

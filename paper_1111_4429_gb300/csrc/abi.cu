@@ -208,18 +208,15 @@ int run_graphed(Ctx* c, uint64_t key, cudaStream_t st, const std::function<int()
   return BGW_OK;
 }
 
-// The mixed precisions invert with the tensor-core trailing update unless
-// BGW_OPT_INVERSE selects otherwise; the plain FP64 path uses FP64 FMA.
-bool use_tc_inverse(Ctx* c, int prec) {
-  if (c->inverse_mode == 0) return false;
-  if (c->inverse_mode == 1) return true;
-  return prec != BGW_PREC_FP64;
-}
+// The inverses run their trailing updates on the tensor cores unless
+// BGW_OPT_INVERSE asks for FP64 FMA.
+bool use_tc_inverse(Ctx* c) { return c->inverse_mode != 0; }
 
 // Precision of the tensor-core inverse for a call of precision prec: seven
-// slices (FP64-level updates, near 2^-48) unless the option asks for five
-// (near 2^-34); the mixed precisions take the next diagonal block and the
-// panel product in double FP32 (about 2^-46), FP64 inputs in FP64.
+// slices unless the option asks for five (near 2^-34); the mixed precisions
+// take the level sums (near 2^-48), the next diagonal block and the panel
+// product in double FP32 (about 2^-46), FP64 inputs join the level sums in
+// integers (below the roundings of the FMA sweep) and stay FP64 elsewhere.
 // Recorded in the context for the inverse that follows.
 void set_run_slices(Ctx* c, int prec) {
   c->run_slices = c->update_slices ? c->update_slices : 7;
@@ -517,7 +514,7 @@ int bgw_epsinv_general(bgw_ctx* ctx, int nmat, const bgw_cell* cells, const int*
     cp[m] = &cells[m];
   }
   set_run_slices(c, BGW_PREC_FP64);
-  return epsinv_general_run(c, nmat, ng, cp.data(), dgeps.data(), chi, eps, epsinv, st, c->inverse_mode == 1);
+  return epsinv_general_run(c, nmat, ng, cp.data(), dgeps.data(), chi, eps, epsinv, st, use_tc_inverse(c));
 }
 
 int bgw_epsinv_rflavor(bgw_ctx* ctx, int nmat, const bgw_cell* cells, const int* ng, const int32_t* const* geps,
@@ -543,7 +540,7 @@ int bgw_epsinv_rflavor(bgw_ctx* ctx, int nmat, const bgw_cell* cells, const int*
     cp[m] = &cells[m];
   }
   set_run_slices(c, BGW_PREC_FP64);
-  return epsinv_rflavor_run(c, nmat, ng, cp.data(), dgeps.data(), chi, eps, epsinv, st, c->inverse_mode == 1);
+  return epsinv_rflavor_run(c, nmat, ng, cp.data(), dgeps.data(), chi, eps, epsinv, st, use_tc_inverse(c));
 }
 
 int bgw_epsinv(bgw_ctx* ctx, int nmat, const bgw_cell* cells, const int* ng, const int32_t* const* geps,
@@ -570,7 +567,7 @@ int bgw_epsinv(bgw_ctx* ctx, int nmat, const bgw_cell* cells, const int* ng, con
   }
   set_run_slices(c, BGW_PREC_FP64);
   auto body = [&]() {
-    return epsinv_batch_run(c, nmat, ng, cp.data(), dgeps.data(), chi, eps, epsinv, st, c->inverse_mode == 1);
+    return epsinv_batch_run(c, nmat, ng, cp.data(), dgeps.data(), chi, eps, epsinv, st, use_tc_inverse(c));
   };
   // Repeated calls with the same arguments replay a CUDA graph of the
   // sweep (about five launches per 32-column step on three streams): the
@@ -676,7 +673,7 @@ int run_batch(Ctx* c, int nq, const bgw_problem* pr, const std::vector<int>& gri
     }
     set_run_slices(c, prec);
     if ((rc = epsinv_batch_run(c, nrow, ngv.data(), cp.data(), gv.data(), chis.data(), nullptr,
-                               invs.data(), st, use_tc_inverse(c, prec))) != BGW_OK)
+                               invs.data(), st, use_tc_inverse(c))) != BGW_OK)
       return rc;
   }
   return BGW_OK;
@@ -936,13 +933,13 @@ int epsilon_run(bgw_ctx* ctx, const bgw_cell* cell, int nv, int npw_v, const int
       set_run_slices(c, prec);
       if (fa.real)
         rc = epsinv_general_run(c, nrow, ngv.data(), cp.data(), gv2.data(), chis.data(), nullptr, invs.data(), st,
-                                use_tc_inverse(c, prec));
+                                use_tc_inverse(c));
       else if (rf)
         rc = epsinv_rflavor_run(c, nrow, ngv.data(), cp.data(), gv2.data(), chis.data(), nullptr, invs.data(), st,
-                                use_tc_inverse(c, prec));
+                                use_tc_inverse(c));
       else
         rc = epsinv_batch_run(c, nrow, ngv.data(), cp.data(), gv2.data(), chis.data(), nullptr, invs.data(), st,
-                              use_tc_inverse(c, prec));
+                              use_tc_inverse(c));
       if (rc != BGW_OK) return rc;
     }
     if (chi && !chi_dev) BGW_CUDA(c, cudaMemcpyAsync(chi, d_chi, nrow * n2, cudaMemcpyDeviceToHost, st));

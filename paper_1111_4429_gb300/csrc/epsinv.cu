@@ -477,6 +477,19 @@ __global__ void sw_finish_kernel(const __grid_constant__ SweepBatch b) {
   }
 }
 
+// FP64 inputs under the default option: the FMA sweep takes matrices of one
+// block (no trailing update: N_G 20, 44 us against 46) and batches whose slice
+// buffers do not fit.  Everything larger is faster on the tensor cores (one
+// matrix, N_G 40 / 85 / 400 / 1185 / 2120 / 4096: 0.11 / 0.21 / 1.0 / 2.9 / 5.9 /
+// 21 ms against 0.26 / 0.53 / 2.5 / 12.4 / 40 / 247).
+static bool plain_default(Ctx* c) { return c->inverse_mode == -1 && !c->run_ff_chain; }
+static bool one_step(Ctx* c, int ngmax) { return plain_default(c) && ngmax <= NB; }
+bool fma_fallback(Ctx* c, int rc) {
+  if (!plain_default(c) || (rc != BGW_ENOMEM && rc != BGW_EBUSY)) return false;
+  c->err.clear();
+  return true;
+}
+
 // eps~ formation for every matrix of the batch, then the batched sweep.
 int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cells,
                      const int32_t* const* d_geps, const void* const* chi, void* const* eps, void* const* epsinv,
@@ -528,7 +541,7 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
     const size_t upd_smem = sizeof(double2) * 2 * TU * (NB + 1);
     BGW_CUDA(c, cudaFuncSetAttribute(sw_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)upd_smem));
     std::unique_ptr<OzPlan, void (*)(OzPlan*)> oz(nullptr, oz_plan_delete);
-    if (tc_update) {
+    if (tc_update && !one_step(c, ngmax)) {
       oz.reset(oz_plan_new());
       std::vector<int> ngs(nb);
       std::vector<double2*> As(nb);
@@ -541,12 +554,16 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
         Ps[k] = sb.m[k].P;
         Ds[k] = sb.m[k].Dinv;
       }
-      if ((rc = oz_prepare(c, nb, ngs.data(), As.data(), Cs.data(), Ps.data(), Ds.data(), oz.get(), false,
-                           real_values, c->run_slices, c->run_ff_chain)) != BGW_OK)
+      rc = oz_prepare(c, nb, ngs.data(), As.data(), Cs.data(), Ps.data(), Ds.data(), oz.get(), false, real_values,
+                      c->run_slices, c->run_ff_chain);
+      if (rc == BGW_OK)
+        oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
+      else if (fma_fallback(c, rc))
+        oz.reset();
+      else
         return rc;
-      oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
     }
-    if (!tc_update) {
+    if (!oz) {
       for (int k0 = 0; k0 < ngmax; k0 += NB) {
         sw_diag_kernel<<<nb, kDiagThreads, 0, st>>>(sb, k0, c->d_status);
         sw_panel_kernel<<<dim3((ngmax + 7) / 8, nb), 256, 0, st>>>(sb, k0);

@@ -411,10 +411,14 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
         Rs[k] = R.as<double2>() + (size_t)k * kPB * n;
         Cs[k] = Cp.as<double2>() + (size_t)k * kPB * n;
       }
-      if ((rc = oz_prepare(c, nb, ngs.data(), As.data(), Rs.data(), Cs.data(), nullptr, oz.get(), true, false,
-                           c->run_slices, c->run_ff_chain)) != BGW_OK)
+      rc = oz_prepare(c, nb, ngs.data(), As.data(), Rs.data(), Cs.data(), nullptr, oz.get(), true, false,
+                      c->run_slices, c->run_ff_chain);
+      if (rc == BGW_OK)
+        oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
+      else if (fma_fallback(c, rc))
+        oz.reset();
+      else
         return rc;
-      oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
     }
     int* piv = ipiv.as<int>();
     int* src = piv + (size_t)kGB * ngmax;
@@ -447,7 +451,7 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
         c->launches += 1;
         BGW_CUDA(c, cudaGetLastError());
       }
-      if (!tc_update) {
+      if (!oz) {
         for (int k = 0; k < nb; ++k)
           if ((rc = gj_update_run(c, P.A[k], n, k0, kb, R.as<double2>() + (size_t)k * kPB * n,
                                   Cp.as<double2>() + (size_t)k * kPB * n, st)) != BGW_OK)

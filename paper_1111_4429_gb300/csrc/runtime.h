@@ -135,7 +135,7 @@ struct Ctx {
   cudaEvent_t la_ev[4] = {};       // look-ahead dependencies (fork, slice, rest x2)
   cudaStream_t copy_st = nullptr;  // host-to-device copies of bgw_epsilon's conduction chunks
   cudaEvent_t copy_ev[3] = {};     // fork, and the chunk copies (ping-pong)
-  int inverse_mode = -1;     // -1: tensor-core update for the mixed precisions; 0: FP64 FMA; 1: tensor cores
+  int inverse_mode = -1;     // sweep updates: -1, 1 tensor cores (-1: FMA where FP64 buffers do not fit); 0: FP64 FMA
   int head_mode = -1;        // mixed chi head/wings in FP64: -1 automatic at small q, 0 off, 1 on
   int sigma_density = -1;    // Sigma band densities: -1/1 product transform where alias-free, 0 direct sum
   int update_slices = 0;     // tensor-core update slices: 0 automatic (7), 5 or 7
@@ -269,6 +269,9 @@ int segs_per_cta(long long nseg, int ntiles, int nsm);
 int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cells,
                      const int32_t* const* d_geps, const void* const* chi, void* const* eps, void* const* epsinv,
                      cudaStream_t st, bool tc_update, bool real_values = false);
+// Whether the FMA sweep takes over an FP64 inverse whose tensor-core buffers
+// could not be had (rc from oz_prepare): under the default option only.
+bool fma_fallback(Ctx* c, int rc);
 // eps~ = I - sv chi sv of one matrix into A (and eps when non-NULL), sv from
 // the cell's Coulomb model (epsinv.cu).
 int eps_form_run(Ctx* c, const bgw_cell* cell, const int32_t* d_geps, int ng, const void* chi, double* sv,

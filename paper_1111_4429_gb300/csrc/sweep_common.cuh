@@ -194,6 +194,25 @@ __device__ __forceinline__ double ff2d_pair(float s, float t, int ex) {
       (long long)(((unsigned long long)hi << 32) | lo) + (lowers ? -(long long)d : (long long)d);
   return __longlong_as_double(b);
 }
+// X 2^ex rounded to FP64 (half away from zero) for |X| < 2^63, in the integer
+// pipe: the magnitude is shifted up to its leading bit, rounded at the 53rd
+// and the carry runs into the exponent.  Results below the normal range are
+// zero, above it NaN: ex = kBadExp marks operands that are not finite.
+constexpr int kBadExp = 1 << 20;
+__device__ __forceinline__ double i64_to_scaled(long long X, int ex) {
+  const long long s = X >> 63;
+  const unsigned long long m0 = (unsigned long long)((X ^ s) - s);
+  const int c = __clzll((long long)m0) & 63;
+  const unsigned long long m = (m0 << c) + 0x400ull;   // a carry out of bit 63 is the next power of two
+  const bool carry = m < 0x400ull;
+  const unsigned long long mant = carry ? 0ull : (m << 1) >> 12;
+  const int e = 1023 + 63 - c + ex + (carry ? 1 : 0);
+  unsigned long long b =
+      ((unsigned long long)s & 0x8000000000000000ull) | ((unsigned long long)(unsigned)e << 52) | mant;
+  if (m0 == 0ull || e <= 0) b = 0ull;
+  if (e >= 2047) b = 0x7FF8000000000000ull;
+  return __longlong_as_double((long long)b);
+}
 // The rare FP64 forms, out of line: a short slow path inline would be
 // predicated and its FP64 instructions issued on every call.
 static __device__ __noinline__ double ff_to_slow(float hi, float lo) { return (double)hi + (double)lo; }

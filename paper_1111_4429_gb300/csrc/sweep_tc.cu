@@ -18,6 +18,12 @@
 // double-FP32 (two-sum); the pair, scaled by the power of two
 // sigma_i tau_j 2^-16, is subtracted from A in FP64.  The dropped levels and the double-FP32 sum
 // bound the error near 2^-48 of |u_i| |v_j| 64.
+//
+// FP64 inputs (the plain path) join the seven exact level sums in integers
+// instead: a 64-bit integer of unit 2^-55 sigma_i tau_j holds the sum but for
+// its last nine bits, and is rounded to FP64 once.  What is left of the error
+// is the dropped levels' (near 2^-55 sigma_i tau_j), below the roundings of 32
+// complex FMAs and their subtraction.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -187,8 +193,10 @@ __device__ __forceinline__ void digits7(long long X, __half* out, size_t stride)
 }
 
 // Slices and exponent of one 64-value row held by a warp (lane: value k and
-// k + 32); all lanes call it.
-__device__ __forceinline__ void slice_row(double re, double im, int lane, __half* base, size_t stride, int* exp_out) {
+// k + 32); all lanes call it.  mark: a row that holds an infinity or NaN gets
+// the exponent kBadExp, which makes NaN of every element it updates.
+__device__ __forceinline__ void slice_row(double re, double im, int lane, __half* base, size_t stride, int* exp_out,
+                                          bool mark) {
   // e = frexp exponent of the row's largest magnitude, from the biased
   // exponent fields (integer max over the warp; 0 for a zero row, and rows
   // of subnormals alone are cut to zero)
@@ -198,7 +206,7 @@ __device__ __forceinline__ void slice_row(double re, double im, int lane, __half
   const long long Xr = fixed56(re, e), Xi = fixed56(im, e);
   digits7(Xr, base + lane, stride);
   digits7(Xi, base + lane + 32, stride);
-  if (lane == 0) *exp_out = e;
+  if (lane == 0) *exp_out = (mark && emax == 0x7FFu) ? kBadExp : e;
 }
 
 // The Hermitian sweep's panel and its slices in one launch (the look-ahead
@@ -302,8 +310,10 @@ __global__ void __launch_bounds__(256) panel_slice_kernel(const __grid_constant_
   if (lane >= kb) pv = cv = make_double2(0.0, 0.0);
   const size_t row = (size_t)M.row_off + i;
   const size_t base = (size_t)buf * S * rows_total * KR + row * KR;
-  slice_row(pv.x, pv.y, lane, U + base, (size_t)rows_total * KR, sig + (size_t)buf * rows_total + row);
-  slice_row(cv.x, cv.y, lane, V + base, (size_t)rows_total * KR, tau + (size_t)buf * rows_total + row);
+  slice_row(pv.x, pv.y, lane, U + base, (size_t)rows_total * KR, sig + (size_t)buf * rows_total + row,
+            !FF);
+  slice_row(cv.x, cv.y, lane, V + base, (size_t)rows_total * KR, tau + (size_t)buf * rows_total + row,
+            !FF);
 }
 
 // Slices for the general (Gauss-Jordan) update A -= Cp R of the pivoted
@@ -312,9 +322,9 @@ __global__ void __launch_bounds__(256) panel_slice_kernel(const __grid_constant_
 // transposed from R [NB][ng] (every row live: the block's columns receive
 // -Cp D^-1).  M.P holds Cp, M.C holds R.
 __global__ void __launch_bounds__(256) slice_general_kernel(const __grid_constant__ OzBatch b, int k0,
-                                                            int rows_total, int buf, __half* __restrict__ U,
-                                                            __half* __restrict__ V, int* __restrict__ sig,
-                                                            int* __restrict__ tau) {
+                                                            int rows_total, int buf, int mark,
+                                                            __half* __restrict__ U, __half* __restrict__ V,
+                                                            int* __restrict__ sig, int* __restrict__ tau) {
   const OzMat& M = b.m[blockIdx.y];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * 8 + warp;
@@ -336,7 +346,7 @@ __global__ void __launch_bounds__(256) slice_general_kernel(const __grid_constan
   const size_t row = (size_t)M.row_off + i;
   __half* out = (blockIdx.z == 0 ? U : V) + (size_t)buf * S * rows_total * KR + row * KR;
   slice_row(re, im, lane, out, (size_t)rows_total * KR,
-            (blockIdx.z == 0 ? sig : tau) + (size_t)buf * rows_total + row);
+            (blockIdx.z == 0 ? sig : tau) + (size_t)buf * rows_total + row, mark != 0);
 }
 
 // Rows of the block K after the general update: A[k0 + r][j] = R[r][j].
@@ -373,10 +383,20 @@ __device__ __forceinline__ bool mbar_wait_ab(uint64_t* bar, uint32_t parity, vol
   return true;
 }
 
+// A segment's seven level sums (integers below 2^23.2 in FP32) joined in units
+// of 2^-55: adjacent levels in 32 bits, the rest in 64.
+__device__ __forceinline__ long long join_levels(const uint32_t (&x)[7][4], int q) {
+  auto f = [&](int L) { return __float2int_rn(__uint_as_float(x[L][q])); };
+  const int p01 = f(0) * 256 + f(1), p23 = f(2) * 256 + f(3), p45 = f(4) * 256 + f(5);
+  const long long hi = (long long)p01 * 65536 + p23, lo = (long long)p45 * 256 + f(6);   // units 2^-40, 2^-64
+  return (hi << 15) + ((lo + 256) >> 9);
+}
+
 // SL: slices used per value (the most significant SL of the S stored): 7
 // gives an update error near 2^-48 of its scale, 5 near 2^-34.  FFC: the
 // look-ahead CTA sweeps the next diagonal block in double FP32 (about 2^-46
-// per operation, on the FP32 pipe) instead of FP64.
+// per operation, on the FP32 pipe) instead of FP64; without it (FP64 inputs)
+// the level sums are joined in integers and rounded to FP64 once.
 template <bool realv, int SL, bool FFC, bool NARROW>
 __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per sub-partition, 96 registers
     update_pipe_kernel(const __grid_constant__ CUtensorMap umap, const __grid_constant__ CUtensorMap vmap,
@@ -609,7 +629,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
         load_tau(k + 1, tnext);
         bool have = mbar_wait_ab(t_full, tt & 1, abort_flag);
         have = __all_sync(0xffffffffu, have) != 0;
-        float hr[8], lr[8], hm[8], lm[8];
+        float hr[8], lr[8], hm[8], lm[8];      // FFC: level sums as double-FP32 pairs
+        long long xr[8], xm[8];                // FP64 inputs: as integers
         if (have) {
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           // Four rounds (two 16-row halves, real then imaginary parts):
@@ -650,14 +671,21 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
 #pragma unroll
               for (int L = 0; L < SL; ++L) tmem_ld16x256(tl + 32 * (part * SL + L), x[L]);
               asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-              if (part == 0)
+              if constexpr (!FFC) {
+#pragma unroll
+                for (int qq = 0; qq < 4; ++qq) (part == 0 ? xr : xm)[4 * hb + qq] = join_levels(x, qq);
+              } else if (part == 0) {
                 combine(x, hb, hr, lr);
-              else
+              } else {
                 combine(x, hb, hm, lm);
+              }
             }
             if constexpr (realv) {
 #pragma unroll
-              for (int qq = 0; qq < 4; ++qq) hm[4 * hb + qq] = lm[4 * hb + qq] = 0.f;
+              for (int qq = 0; qq < 4; ++qq) {
+                hm[4 * hb + qq] = lm[4 * hb + qq] = 0.f;
+                xm[4 * hb + qq] = 0;
+              }
             }
           }
         } else if (lane == 0) {
@@ -698,8 +726,13 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
             const int e2 = ei[m] + tv[n] - 2 * BETA;
             // scale 2^e2 (sigma_i tau_j 2^-16) applied in the conversion; one
             // FP64 add per word
-            o[n].x = v.x - ff2d_scaled(hr[e], lr[e], e2);
-            o[n].y = realv ? v.y : v.y - ff2d_scaled(hm[e], lm[e], e2);
+            if constexpr (FFC) {
+              o[n].x = v.x - ff2d_scaled(hr[e], lr[e], e2);
+              o[n].y = realv ? v.y : v.y - ff2d_scaled(hm[e], lm[e], e2);
+            } else {   // unit 2^-55 against the pairs' 2^-16
+              o[n].x = v.x - i64_to_scaled(xr[e], e2 - 39);
+              o[n].y = realv ? v.y : v.y - i64_to_scaled(xm[e], e2 - 39);
+            }
           }
           const unsigned wr = (mask >> (2 * m)) & 3u;
           if (wr == 3u && !(reinterpret_cast<uintptr_t>(M.A + off) & 31u)) {
@@ -872,8 +905,9 @@ int oz_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, cudaStream_t st) 
   const int rpad = (ngmax + BM - 1) / BM * BM;
   if (!plan->general) return fail(c, BGW_EINVAL, "oz_slice: the Hermitian sweep slices in oz_panel_slice");
   slice_general_kernel<<<dim3(rpad / 8, plan->nmat, 2), 256, 0, st>>>(plan->batch, k0, plan->rows_total, buf,
-                                                                      plan->U.as<__half>(), plan->V.as<__half>(),
-                                                                      plan->sig.as<int>(), plan->tau.as<int>());
+                                                                      plan->ff_chain ? 0 : 1, plan->U.as<__half>(),
+                                                                      plan->V.as<__half>(), plan->sig.as<int>(),
+                                                                      plan->tau.as<int>());
   BGW_CUDA(c, cudaGetLastError());
   return BGW_OK;
 }
