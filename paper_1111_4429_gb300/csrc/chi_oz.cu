@@ -488,6 +488,43 @@ __global__ void reduce_kernel(const double2* __restrict__ work, int ngroups, int
   }
 }
 
+// The Sigma forms of pair p = p0 + i, one warp per pair: C = W m from the
+// product's partial tiles, qW = Re sum_G conj(m_p(G)) C(G), qV = sum_G |m_p(G)|^2 v_G.
+__global__ void __launch_bounds__(256) sigma_forms_kernel(const double2* __restrict__ M, long long p0, int R, int ng,
+                                                          const double* __restrict__ sv,
+                                                          const double2* __restrict__ work, int ngroups, int ntiles,
+                                                          const int* __restrict__ flag, double* __restrict__ qW,
+                                                          double* __restrict__ qV) {
+  if (*flag) return;
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= R) return;
+  const int nJ = (ng + BN - 1) / BN;
+  const double2* m = M + (p0 + i) * ng;
+  double w = 0.0, s = 0.0;
+  for (int J = 0; J < nJ; ++J) {
+    const int g = J * BN + lane;
+    if (g >= ng) break;
+    const double2* t = work + ((size_t)(i / BM) * nJ + J) * kTileElems + (size_t)(i % BM) * BN + lane;
+    double2 c = *t;
+    for (int q = 1; q < ngroups; ++q) {
+      const double2 x = t[(size_t)q * ntiles * kTileElems];
+      c.x += x.x;
+      c.y += x.y;
+    }
+    const double2 v = m[g];
+    w = fma(v.x, c.x, fma(v.y, c.y, w));
+    s = fma(fma(v.x, v.x, v.y * v.y), sv[g] * sv[g], s);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    w += __shfl_xor_sync(0xffffffffu, w, o);
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
+  if (lane == 0) {
+    qW[p0 + i] = w;
+    qV[p0 + i] = s;
+  }
+}
+
 }  // namespace oz64
 
 namespace {
@@ -700,6 +737,66 @@ int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, con
       }
     }
   }
+  return BGW_OK;
+}
+
+// The FP64 Sigma forms qW_p = m_p^H W m_p and qV_p = sum_G |m_p(G)|^2 v_G of K
+// pairs on the tensor cores: C = W m by digit products (rows of conj(m) against
+// rows of W, inner index G'), block by block of pairs.  *flag (device, zeroed
+// here) is set where an operand is not finite: the FMA kernels must then do the
+// call.  Returns BGW_ENOMEM when the scratch does not fit (nothing launched).
+int sigma_oz_forms(Ctx* c, long long K, int ng, const void* M, const void* W, const double* sv, double* qW, double* qV,
+                   int* flag, cudaStream_t st) {
+  using namespace oz64;
+  const int nsm = sm_count(c);
+  const int nJ = (ng + BN - 1) / BN;
+  const long long nst = (ng + SK / 2 - 1) / (SK / 2);
+  OzGemm g(&c->pool);
+  g.kpad = nst * (SK / 2);
+  g.vrows = nJ * BN;
+  Scratch meta;
+  meta.pool = &c->pool;
+  const size_t row_bytes = (size_t)S * g.kpad * 2 * 2;
+  long long rows = std::min<long long>((K + BM - 1) / BM * BM,
+                                       std::max<long long>(BM, (long long)(kOzChunkBytes / 2 / row_bytes) / BM * BM));
+  int rc;
+  if ((rc = c->pool.alloc((size_t)(rows + g.vrows) * sizeof(int), &meta.ptr)) != BGW_OK) return BGW_ENOMEM;
+  for (;;) {
+    g.urows = (int)rows;
+    rc = oz_alloc(c, &g, true, (int)(rows / BM) * nJ, nsm, g.kpad, false);
+    if (rc == BGW_OK) break;
+    oz_release(c, &g);
+    if (rc == BGW_ECUDA || rows == BM) return rc == BGW_ECUDA ? rc : BGW_ENOMEM;
+    rows = std::max<long long>(BM, rows / 2 / BM * BM);
+  }
+  std::vector<int2> tl;
+  for (int I = 0; I < (int)(rows / BM); ++I)
+    for (int J = 0; J < nJ; ++J) tl.push_back(make_int2(I, J));
+  const void* d_tiles;
+  if ((rc = upload_cached(c, tl.data(), tl.size() * sizeof(int2), st, &d_tiles)) != BGW_OK) return rc;
+  if ((rc = oz_maps(c, &g)) != BGW_OK) return rc;
+  int* ufield = meta.as<int>();
+  int* vfield = ufield + rows;
+  BGW_CUDA(c, cudaMemsetAsync(flag, 0, sizeof(int), st));
+  row_digits_kernel<<<(g.vrows + 7) / 8, 256, 0, st>>>(static_cast<const double2*>(W), ng, ng, g.vrows, g.rowlen, 0,
+                                                       vfield, flag, g.v.as<__half>());
+  for (long long p0 = 0; p0 < K; p0 += rows) {
+    const int R = (int)std::min<long long>(rows, K - p0), nI = (R + BM - 1) / BM, ntiles = nI * nJ;
+    row_digits_kernel<<<nI * BM / 8, 256, 0, st>>>(static_cast<const double2*>(M) + (size_t)p0 * ng, R, ng, g.urows,
+                                                   g.rowlen, 1, ufield, flag, g.u.as<__half>());
+    BGW_CUDA(c, cudaGetLastError());
+    OzSplit s = oz_split(nst, ntiles, nsm);
+    s.groups = std::min(s.groups, g.ngroups_max * (int)(rows / BM) * nJ / ntiles);   // fits the partial sums' space
+    s.per = (int)((((nst + s.seg - 1) / s.seg) + s.groups - 1) / s.groups);
+    if ((rc = oz_launch<false>(c, g, nst, s, ntiles, static_cast<const int2*>(d_tiles), ufield, vfield, flag, st)) !=
+        BGW_OK)
+      return rc;
+    sigma_forms_kernel<<<(R + 7) / 8, 256, 0, st>>>(static_cast<const double2*>(M), p0, R, ng, sv,
+                                                    g.work.as<double2>(), s.groups, ntiles, flag, qW, qV);
+    BGW_CUDA(c, cudaGetLastError());
+    c->launches += 2;
+  }
+  c->launches += 1;
   return BGW_OK;
 }
 

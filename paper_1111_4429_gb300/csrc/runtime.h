@@ -261,6 +261,10 @@ int chi_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const doubl
 // kernel must do frequency f (operands that are not finite).
 int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, const double2* wc, int nrow,
                double scale, int accumulate, void* chi, bool real, int* flags, cudaStream_t st);
+// The FP64 Sigma forms of K pairs (M [K][ng], W [ng][ng], sv = v^1/2) on the
+// tensor cores; *flag and the return value as chi_oz_run's.
+int sigma_oz_forms(Ctx* c, long long K, int ng, const void* M, const void* W, const double* sv, double* qW, double* qV,
+                   int* flag, cudaStream_t st);
 // Segments of work per CTA for nseg segments over ntiles tiles (chi_tc.cu).
 int segs_per_cta(long long nseg, int ntiles, int nsm);
 // eps~ and its inverse for nmat matrices (per-matrix size, cell and q).

@@ -89,3 +89,22 @@ def test_values_that_are_not_finite_take_the_fma_kernel():
     rows = np.zeros(ng, bool)
     rows[[17, 40]] = True
     assert np.array_equal(bad, rows[:, None] | rows[None, :])
+
+
+@pytest.mark.parametrize("no,ni,nocc", [(1, 1, 1), (1, 127, 9), (2, 64, 5), (3, 43, 4), (5, 77, 7)])
+def test_sigma_forms_at_tile_edges(no, ni, nocc):
+    """K = no ni pairs around the 128-row tile, whole and in blocks of pairs
+    under a budget, against the oracle (the FP64 bar of the Sigma tests)."""
+    import oracle
+    from paper_1111_4429_gb300 import bgw, synth
+    s = synth.make_system("sd", a=14.0, fft=24, ecut_wfn=6.0, ecut_eps=2.5, nv=3, nc=20, seed=61)
+    r = oracle.solve(s)
+    sb = synth.sigma_bands(s, no, ni, nocc, seed=ni)
+    ref = oracle.sigma_cohsex(sb.gi, sb.ci, nocc, sb.go, sb.co, s.geps, r["epsinv"], r["v"], s.omega)
+    for budget in (0, 48 << 20):
+        ctx = bgw.Context(0, budget)
+        got = ctx.sigma_cohsex(bgw.system_cell(s), sb.go, torch.from_numpy(sb.co).cuda(), sb.gi,
+                               torch.from_numpy(sb.ci).cuda(), nocc, s.geps, torch.from_numpy(r["epsinv"]).cuda())
+        for k, key in enumerate(("X", "SX", "CH")):
+            want = np.real(ref[key])
+            assert np.abs(got[k] - want).max() <= 1e-12 * np.abs(want).max()
