@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kDiagThreads) sw_diag_kernel(const __grid_cons
   bool low;
   diag_thread_element(t, kb, i, j, low);
   if (low) sm.L[i][j] = A[(size_t)(k0 + i) * ng + k0 + j];
-  diag_sweep_smem(sm, kb, t, i, j, low, status);
+  diag_sweep_f64(sm, kb, t, status);
   for (int e2 = threadIdx.x; e2 < NB * NB; e2 += blockDim.x) {
     const int r = e2 / NB, c = e2 % NB;
     if (r >= kb || c >= kb) continue;

@@ -5,16 +5,19 @@
 // L[i][j], i >= j.  Pivot s: every lower element outside row/column s loses
 // col_i conj(col_j) / d (col = column s of the full matrix, d = L[s][s]), the
 // pivot column is divided by d and the pivot becomes -1/d.  After kb pivots
-// L holds -D^-1.  The 528 lower elements are packed into 17 full warps: the
-// FP64 pipe of the SM this runs on is the limit, and idle lanes of a warp
-// still occupy it.
+// L holds -D^-1.
 #pragma once
 #include "runtime.h"
 
 namespace bgw {
 
+// -x by the sign bit (no FP64 instruction)
+__device__ __forceinline__ double neg_bits(double x) {
+  return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);
+}
+
 constexpr int kSwNB = 32;
-constexpr int kDiagThreads = (kSwNB * (kSwNB + 1) / 2 + 31) / 32 * 32;  // 544
+constexpr int kDiagThreads = 17 * 32;   // a thread per lower element, and the pivot's warp
 
 struct DiagSmem {
   double2 L[kSwNB][kSwNB + 1];
@@ -32,119 +35,8 @@ __device__ __forceinline__ void diag_thread_element(int t, int kb, int& i, int& 
   low = t < kSwNB * (kSwNB + 1) / 2 && i < kb;
 }
 
-// Called by all kDiagThreads threads after L (lower) is loaded; ends with a
-// __syncthreads().  A non-positive or non-finite pivot sets *status.
-__device__ __forceinline__ void diag_sweep_smem(DiagSmem& sm, int kb, int t, int i, int j, bool low,
-                                                int* status) {
-  for (int s = 0; s < kb; ++s) {
-    __syncthreads();
-    if (t < kb) {
-      const int r = t;
-      double2 cv;
-      if (r > s) {
-        cv = sm.L[r][s];
-      } else if (r < s) {
-        const double2 x = sm.L[s][r];
-        cv = make_double2(x.x, -x.y);
-      } else {
-        cv = sm.L[s][s];
-      }
-      sm.col[r] = cv;
-      const double d = sm.L[s][s].x;
-      double rr;
-      if (!(d > 0.0) || !isfinite(d)) {
-        if (r == 0) atomicExch(status, (int)kDevZeroPivot);
-        rr = 0.0;
-      } else {
-        rr = 1.0 / d;
-      }
-      sm.ncolr[r] = make_double2(-cv.x * rr, cv.y * rr);
-      if (r == s) sm.rpiv = rr;
-    }
-    __syncthreads();
-    if (low) {
-      if (i != s && j != s) {
-        const double2 a = sm.col[i], c = sm.ncolr[j];
-        double2 v = sm.L[i][j];
-        v.x = fma(a.x, c.x, fma(-a.y, c.y, v.x));
-        v.y = fma(a.x, c.y, fma(a.y, c.x, v.y));
-        sm.L[i][j] = v;
-      } else if (i == s && j == s) {
-        sm.L[s][s] = make_double2(-sm.rpiv, 0.0);
-      } else if (j == s) {  // i > s: A_is / d
-        const double2 a = sm.col[i];
-        sm.L[i][s] = make_double2(a.x * sm.rpiv, a.y * sm.rpiv);
-      } else {              // i == s, j < s: A_sj / d = conj(col_j) / d
-        const double2 c = sm.ncolr[j];
-        sm.L[s][j] = make_double2(-c.x, -c.y);
-      }
-    }
-  }
-  __syncthreads();
-}
-
-// The same sweep with NT threads (NT < 528): each thread owns the lower
-// elements t, t + NT, ...  Called by all NT threads after L (lower) is
-// loaded; ends with a __syncthreads().
-template <int NT>
-__device__ __forceinline__ void diag_sweep_smem_n(DiagSmem& sm, int kb, int t, int* status) {
-  constexpr int NE = (kSwNB * (kSwNB + 1) / 2 + NT - 1) / NT;
-  int ei[NE], ej[NE];
-  bool el[NE];
-#pragma unroll
-  for (int q = 0; q < NE; ++q) diag_thread_element(t + q * NT, kb, ei[q], ej[q], el[q]);
-  for (int s = 0; s < kb; ++s) {
-    __syncthreads();
-    if (t < kb) {
-      const int r = t;
-      double2 cv;
-      if (r > s) {
-        cv = sm.L[r][s];
-      } else if (r < s) {
-        const double2 x = sm.L[s][r];
-        cv = make_double2(x.x, -x.y);
-      } else {
-        cv = sm.L[s][s];
-      }
-      sm.col[r] = cv;
-      const double d = sm.L[s][s].x;
-      double rr;
-      if (!(d > 0.0) || !isfinite(d)) {
-        if (r == 0) atomicExch(status, (int)kDevZeroPivot);
-        rr = 0.0;
-      } else {
-        rr = 1.0 / d;
-      }
-      sm.ncolr[r] = make_double2(-cv.x * rr, cv.y * rr);
-      if (r == s) sm.rpiv = rr;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < NE; ++q) {
-      if (!el[q]) continue;
-      const int i = ei[q], j = ej[q];
-      if (i != s && j != s) {
-        const double2 a = sm.col[i], c = sm.ncolr[j];
-        double2 v = sm.L[i][j];
-        v.x = fma(a.x, c.x, fma(-a.y, c.y, v.x));
-        v.y = fma(a.x, c.y, fma(a.y, c.x, v.y));
-        sm.L[i][j] = v;
-      } else if (i == s && j == s) {
-        sm.L[s][s] = make_double2(-sm.rpiv, 0.0);
-      } else if (j == s) {
-        const double2 a = sm.col[i];
-        sm.L[i][s] = make_double2(a.x * sm.rpiv, a.y * sm.rpiv);
-      } else {
-        const double2 c = sm.ncolr[j];
-        sm.L[s][j] = make_double2(-c.x, -c.y);
-      }
-    }
-  }
-  __syncthreads();
-}
-
 // ---------------------------------------------------------------------------
-// The same sweep in double-FP32 arithmetic (a value is hi + lo, two floats,
+// Double-FP32 arithmetic for the same sweep (a value is hi + lo, two floats,
 // about 2^-46 relative per operation) for updates whose target precision is
 // far coarser than FP64 (the five-slice tensor-core update, near 2^-34).
 // GB300's FP32 pipe issues 64 times the FP64 pipe's operations, so the
@@ -217,6 +109,7 @@ __device__ __forceinline__ double i64_to_scaled(long long X, int ex) {
 // predicated and its FP64 instructions issued on every call.
 static __device__ __noinline__ double ff_to_slow(float hi, float lo) { return (double)hi + (double)lo; }
 static __device__ __noinline__ float2 ff_from_slow(double x) { return ff_from(x); }
+static __device__ __noinline__ double rcp_slow(double x) { return 1.0 / x; }
 
 // hi + lo as a double for any finite pair: the integer form above where the
 // sum lies in [2^-66, 2^123), else the FP64 pipe.
@@ -282,10 +175,6 @@ __device__ __forceinline__ long long fixed56(double v, int e) {
   return (b >> 63) ? -(long long)X : (long long)X;
 }
 
-// -x by the sign bit (no FP64 instruction)
-__device__ __forceinline__ double neg_bits(double x) {
-  return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);
-}
 __device__ __forceinline__ float2 ff_neg(float2 a) { return make_float2(-a.x, -a.y); }
 // a b
 __device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
@@ -323,27 +212,102 @@ __device__ __forceinline__ float2 ff_dot2(float2 v, float2 a1, float2 b1, float2
   return make_float2(s2.x, __fadd_rn(__fadd_rn(v.y, __fadd_rn(e1, e2)), __fadd_rn(s1.y, s2.y)));
 }
 
-// Double-FP32 form of diag_sweep_smem_n with one barrier per pivot: the
-// matrix ping-pongs between sm.L (as float4: re hi, re lo, im hi, im lo) and
-// the scratch buffer (32 x 33 float4, 16.9 KiB of shared memory the caller
-// does not need meanwhile).  Pivot s reads buffer s & 1 and writes every
-// lower element into the other; each thread forms the column entries it
-// needs itself, and the thread that writes the next pivot element forms its
-// reciprocal, so no step has a serial phase.  Converts sm.L from and back to
-// double2, so callers read and write sm.L as double2 before and after.
-// Called by all NT threads after L (lower) is loaded; ends with a
-// __syncthreads().  A non-positive or non-finite pivot sets *status.
-template <int NT>
-__device__ __forceinline__ void diag_sweep_ff_n(DiagSmem& sm, float4* scratch, int kb, int t, int* status,
-                                                float4* dff = nullptr) {
-  constexpr int NE = (kSwNB * (kSwNB + 1) / 2 + NT - 1) / NT;
+// The sweep, by 17 warps.  Pivot s, two barriers: warp 16
+// (lane r: index r) copies the pivot's column and its scaled form
+// -conj(col) / d and writes the pivot's row and column, which are multiples of
+// them; then warps 0 .. 15 update the other lower elements, one per thread
+// (thread q: element (x, y) of the 31 x 31 triangle, indices from s on moved up
+// by one), without divergence, while the lane of the next pivot forms that
+// pivot's reciprocal from its own registers.  Called by all 544 threads after
+// L (lower) is loaded; ends with a __syncthreads().  A non-positive or
+// non-finite pivot sets *status.
+//
+// Bound by the two phases' latencies (double FP32) and by the FP64 pipe (496
+// elements x 4 operations at 2 a clock: 0.5 us of 1.0 us a pivot).  A 32 x 32
+// block takes 15.3 us in double FP32 and 31.7 us in FP64; with every lower
+// element at a fixed thread (the pivot's row and column as divergent branches)
+// and the reciprocal by the thread that also updates, 17.3 and 38.7 us; with
+// one barrier a pivot and no shared scaled column, 21 us in double FP32.
+// Element (i, j) of thread q in step s, kb x kb block; live = it owns one.
+__device__ __forceinline__ void sweep_element(int x, int y, int s, int& i, int& j) {
+  i = x + (x >= s ? 1 : 0);
+  j = y + (y >= s ? 1 : 0);
+}
+
+__device__ __forceinline__ void diag_sweep_f64(DiagSmem& sm, int kb, int t, int* status) {
+  const int lane = t & 31;
+  const bool head = t >= 16 * 32;
+  int x, y;
+  bool low;
+  diag_thread_element(t, kb - 1, x, y, low);
+  // 1 / d: the double-FP32 reciprocal (2^-46) and one Newton step with a fused
+  // residual, two FP64 operations instead of a division's chain of them, each
+  // of which would queue behind the update's at the FP64 pipe
+  auto rcp_checked = [&](double d) {
+    if (!(d > 0.0) || !isfinite(d)) {
+      atomicExch(status, (int)kDevZeroPivot);
+      return 0.0;
+    }
+    const int ex = (int)((unsigned)__double2hiint(d) >> 20) - 1023;
+    if (ex < -60 || ex > 60) return rcp_slow(d);   // outside double FP32's safe range
+    const float2 r = ff_rcp(ff_from_int(d));
+    const double r0 = ff_to_any(r.x, r.y);
+    return fma(r0, fma(-d, r0, 1.0), r0);
+  };
+  __syncthreads();
+  if (head && lane == 0) sm.rpiv = rcp_checked(sm.L[0][0].x);
+  for (int s = 0; s < kb; ++s) {
+    double2 cv = make_double2(0.0, 0.0), nc = cv;
+    double v = 0.0;
+    __syncthreads();
+    if (head && lane < kb) {
+      const double rr = sm.rpiv;
+      const double2 z = lane < s ? sm.L[s][lane] : sm.L[lane][s];
+      v = sm.L[lane][lane].x;
+      cv = lane < s ? make_double2(z.x, neg_bits(z.y)) : z;
+      nc = make_double2(neg_bits(cv.x * rr), cv.y * rr);
+      sm.col[lane] = cv;
+      sm.ncolr[lane] = nc;
+      if (lane == s)
+        sm.L[s][s] = make_double2(neg_bits(rr), 0.0);
+      else if (lane > s)                                            // A_is / d
+        sm.L[lane][s] = make_double2(neg_bits(nc.x), nc.y);
+      else                                                          // conj(col_j) / d
+        sm.L[s][lane] = make_double2(neg_bits(nc.x), neg_bits(nc.y));
+    }
+    __syncthreads();
+    if (head) {
+      if (lane == s + 1 && lane < kb) sm.rpiv = rcp_checked(fma(cv.x, nc.x, fma(-cv.y, nc.y, v)));
+    } else if (low) {
+      int i, j;
+      sweep_element(x, y, s, i, j);
+      const double2 a = sm.col[i], c = sm.ncolr[j];
+      double2 e = sm.L[i][j];
+      e.x = fma(a.x, c.x, fma(-a.y, c.y, e.x));
+      e.y = fma(a.x, c.y, fma(a.y, c.x, e.y));
+      sm.L[i][j] = e;
+    }
+  }
+  __syncthreads();
+}
+
+// The same in double FP32.  The elements are held in sm.L as float4 (re hi, re
+// lo, im hi, im lo), the pivot's column and its scaled form in scratch (64
+// float4 the caller does not need meanwhile).  Converts sm.L from and back to
+// double2; dff gets -(the result) = D^-1 as normalized pairs, both triangles
+// (ld kSwNB): the next panel product reads it without FP64 conversions.
+__device__ __forceinline__ void diag_sweep_ff(DiagSmem& sm, float4* scratch, int kb, int t, int* status, float4* dff) {
   typedef float4 Row[kSwNB + 1];
-  Row* const B0 = reinterpret_cast<Row*>(sm.L);
-  Row* const B1 = reinterpret_cast<Row*>(scratch);
-  float2* rps = reinterpret_cast<float2*>(sm.col);   // reciprocal of the pivot of step s in rps[s & 1]
-  int ei[NE], ej[NE];
-  bool el[NE];
-  __syncthreads();   // the caller's loads of L are visible before the conversion
+  Row* const B = reinterpret_cast<Row*>(sm.L);
+  float4* const col = scratch;
+  float4* const ncol = scratch + kSwNB;
+  float2* const rpiv = reinterpret_cast<float2*>(&sm.rpiv);
+  const int lane = t & 31;
+  const bool head = t >= 16 * 32;
+  int i, j, x, y;
+  bool low, all;
+  diag_thread_element(t, kb, i, j, all);        // conversions: every lower element
+  diag_thread_element(t, kb - 1, x, y, low);    // updates: the 31 x 31 triangle
   auto rcp_checked = [&](float2 d) {
     d = ff_two_sum(d.x, d.y);   // leading word first (the pair may be unnormalized)
     if (!(d.x > 0.f) || !isfinite(d.x)) {
@@ -352,72 +316,56 @@ __device__ __forceinline__ void diag_sweep_ff_n(DiagSmem& sm, float4* scratch, i
     }
     return ff_rcp(d);
   };
-#pragma unroll
-  for (int q = 0; q < NE; ++q) {
-    diag_thread_element(t + q * NT, kb, ei[q], ej[q], el[q]);
-    if (el[q]) {
-      const double2 x = sm.L[ei[q]][ej[q]];
-      const float2 re = ff_from_int(x.x), im = ff_from_int(x.y);
-      B0[ei[q]][ej[q]] = make_float4(re.x, re.y, im.x, im.y);
-      if (ei[q] == 0 && ej[q] == 0) rps[0] = rcp_checked(re);
-    }
+  __syncthreads();   // the caller's loads of L are visible before the conversion
+  if (all) {
+    const double2 z = sm.L[i][j];
+    const float2 re = ff_from_int(z.x), im = ff_from_int(z.y);
+    B[i][j] = make_float4(re.x, re.y, im.x, im.y);
+    if (i == 0) *rpiv = rcp_checked(re);
   }
   for (int s = 0; s < kb; ++s) {
+    float4 cv = make_float4(0.f, 0.f, 0.f, 0.f), nc = cv, v = cv;
     __syncthreads();
-    Row* const R = (s & 1) ? B1 : B0;   // selects, not an indexed array (kept out of local memory)
-    Row* const W = (s & 1) ? B0 : B1;
-    const float2 rp = rps[s & 1];
-    // column s of the full (Hermitian) matrix at index x: R[x][s] below the
-    // pivot, conj(R[s][x]) above it
-    auto col = [&](int x) {
-      const bool up = x < s;
-      const float4 v = up ? R[s][x] : R[x][s];
-      const float g = up ? -1.f : 1.f;
-      return make_float4(v.x, v.y, g * v.z, g * v.w);
-    };
-#pragma unroll
-    for (int q = 0; q < NE; ++q) {
-      if (!el[q]) continue;
-      const int i = ei[q], j = ej[q];
-      float4 out;
-      if (i != s && j != s) {
-        const float4 a4 = col(i), c4 = col(j), v4 = R[i][j];
-        // ncolr_j = -conj(col_j) / d
-        const float2 cr = ff_mul(ff_neg(make_float2(c4.x, c4.y)), rp), ci = ff_mul(make_float2(c4.z, c4.w), rp);
-        const float2 ar = make_float2(a4.x, a4.y), ai = make_float2(a4.z, a4.w);
-        const float2 vr = ff_dot2(make_float2(v4.x, v4.y), ar, cr, ff_neg(ai), ci);   // + a_r c_r - a_i c_i
-        const float2 vi = ff_dot2(make_float2(v4.z, v4.w), ar, ci, ai, cr);           // + a_r c_i + a_i c_r
-        out = make_float4(vr.x, vr.y, vi.x, vi.y);
-        if (i == s + 1 && j == s + 1) rps[(s + 1) & 1] = rcp_checked(vr);
-      } else if (i == s && j == s) {
-        out = make_float4(-rp.x, -rp.y, 0.f, 0.f);
-      } else if (j == s) {  // i > s: A_is / d
-        const float4 a4 = R[i][s];
-        const float2 xr = ff_mul(make_float2(a4.x, a4.y), rp), xi = ff_mul(make_float2(a4.z, a4.w), rp);
-        out = make_float4(xr.x, xr.y, xi.x, xi.y);
-      } else {              // i == s, j < s: conj(col_j) / d
-        const float4 c4 = R[s][j];   // col_j = conj(R[s][j]); conj(col_j) = R[s][j]
-        const float2 xr = ff_mul(make_float2(c4.x, c4.y), rp), xi = ff_mul(make_float2(c4.z, c4.w), rp);
-        out = make_float4(xr.x, xr.y, xi.x, xi.y);
-      }
-      W[i][j] = out;
+    if (head && lane < kb) {
+      const float2 rp = *rpiv;
+      const float4 z = lane < s ? B[s][lane] : B[lane][s];
+      const float g = lane < s ? -1.f : 1.f;
+      v = B[lane][lane];
+      const float2 cr = ff_mul(make_float2(z.x, z.y), rp), ci = ff_mul(make_float2(g * z.z, g * z.w), rp);
+      cv = make_float4(z.x, z.y, g * z.z, g * z.w);
+      nc = make_float4(-cr.x, -cr.y, ci.x, ci.y);
+      col[lane] = cv;
+      ncol[lane] = nc;
+      if (lane == s)
+        B[s][s] = make_float4(-rp.x, -rp.y, 0.f, 0.f);
+      else if (lane > s)                                       // A_is / d
+        B[lane][s] = make_float4(cr.x, cr.y, ci.x, ci.y);
+      else                                                     // conj(col_j) / d
+        B[s][lane] = make_float4(cr.x, cr.y, -ci.x, -ci.y);
+    }
+    __syncthreads();
+    if (head) {
+      if (lane == s + 1 && lane < kb)
+        *rpiv = rcp_checked(ff_dot2(make_float2(v.x, v.y), make_float2(cv.x, cv.y), make_float2(nc.x, nc.y),
+                                    make_float2(-cv.z, -cv.w), make_float2(nc.z, nc.w)));
+    } else if (low) {
+      int ii, jj;
+      sweep_element(x, y, s, ii, jj);
+      const float4 a = col[ii], c = ncol[jj], e = B[ii][jj];
+      const float2 ar = make_float2(a.x, a.y), ai = make_float2(a.z, a.w);
+      const float2 cr = make_float2(c.x, c.y), ci = make_float2(c.z, c.w);
+      const float2 vr = ff_dot2(make_float2(e.x, e.y), ar, cr, ff_neg(ai), ci);   // + a_r c_r - a_i c_i
+      const float2 vi = ff_dot2(make_float2(e.z, e.w), ar, ci, ai, cr);           // + a_r c_i + a_i c_r
+      B[ii][jj] = make_float4(vr.x, vr.y, vi.x, vi.y);
     }
   }
   __syncthreads();
-  Row* const F = (kb & 1) ? B1 : B0;
-#pragma unroll
-  for (int q = 0; q < NE; ++q) {
-    if (!el[q]) continue;
-    const float4 x = F[ei[q]][ej[q]];
-    sm.L[ei[q]][ej[q]] = make_double2(ff_to_any(x.x, x.y), ff_to_any(x.z, x.w));
-    if (dff) {
-      // -D^-1 as normalized double-FP32 pairs, both triangles (ld kSwNB):
-      // the next panel product reads them without FP64 conversions
-      const float2 re = ff_two_sum(x.x, x.y), im = ff_two_sum(x.z, x.w);
-      const int i = ei[q], j = ej[q];
-      dff[i * kSwNB + j] = make_float4(-re.x, -re.y, -im.x, -im.y);
-      if (i != j) dff[j * kSwNB + i] = make_float4(-re.x, -re.y, im.x, im.y);
-    }
+  if (all) {
+    const float4 z = B[i][j];
+    sm.L[i][j] = make_double2(ff_to_any(z.x, z.y), ff_to_any(z.z, z.w));
+    const float2 re = ff_two_sum(z.x, z.y), im = ff_two_sum(z.z, z.w);
+    dff[i * kSwNB + j] = make_float4(-re.x, -re.y, -im.x, -im.y);
+    if (i != j) dff[j * kSwNB + i] = make_float4(-re.x, -re.y, im.x, im.y);
   }
   __syncthreads();
 }

@@ -370,6 +370,7 @@ __global__ void rows_from_r_kernel(const __grid_constant__ OzBatch b, int k0) {
 // MMAs start -- and apply the FP64 subtraction while they run.
 constexpr int kPipeEpiWarps = 16;
 constexpr int kPipeThreads = (kPipeEpiWarps + 1) * 32;
+static_assert(kPipeThreads == kDiagThreads, "the look-ahead CTA sweeps the next diagonal block");
 
 
 // Bounded wait that also gives up when the CTA aborts.
@@ -767,9 +768,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
       // double-FP32 chain: the block's sweep in double FP32 (about 2^-46),
       // off the SM's slow FP64 pipe; else FP64
       if constexpr (FFC)
-        diag_sweep_ff_n<kPipeThreads>(dsm, reinterpret_cast<float4*>(us), kb1, threadIdx.x, status, M.Dff);
+        diag_sweep_ff(dsm, reinterpret_cast<float4*>(us), kb1, threadIdx.x, status, M.Dff);
       else
-        diag_sweep_smem_n<kPipeThreads>(dsm, kb1, threadIdx.x, status);
+        diag_sweep_f64(dsm, kb1, threadIdx.x, status);
       for (int e = threadIdx.x; e < NB * NB; e += kPipeThreads) {
         const int rr = e / NB, c2 = e % NB;
         if (rr >= kb1 || c2 >= kb1) continue;
