@@ -218,8 +218,8 @@ __device__ __forceinline__ float2 ff_dot2(float2 v, float2 a1, float2 b1, float2
 // them; then warps 0 .. 15 update the other lower elements, one per thread
 // (thread q: element (x, y) of the 31 x 31 triangle, indices from s on moved up
 // by one), without divergence, while the lane of the next pivot forms that
-// pivot's reciprocal from its own registers.  Called by all 544 threads after
-// L (lower) is loaded; ends with a __syncthreads().  A non-positive or
+// pivot's reciprocal from its own registers.  Called by all the block's threads
+// (kDiagThreads or more) after L (lower) is loaded; ends with a __syncthreads().  A non-positive or
 // non-finite pivot sets *status.
 //
 // Bound by the two phases' latencies (double FP32) and by the FP64 pipe (496
@@ -236,7 +236,7 @@ __device__ __forceinline__ void sweep_element(int x, int y, int s, int& i, int& 
 
 __device__ __forceinline__ void diag_sweep_f64(DiagSmem& sm, int kb, int t, int* status) {
   const int lane = t & 31;
-  const bool head = t >= 16 * 32;
+  const bool head = (t >> 5) == 16;
   int x, y;
   bool low;
   diag_thread_element(t, kb - 1, x, y, low);
@@ -303,7 +303,7 @@ __device__ __forceinline__ void diag_sweep_ff(DiagSmem& sm, float4* scratch, int
   float4* const ncol = scratch + kSwNB;
   float2* const rpiv = reinterpret_cast<float2*>(&sm.rpiv);
   const int lane = t & 31;
-  const bool head = t >= 16 * 32;
+  const bool head = (t >> 5) == 16;
   int i, j, x, y;
   bool low, all;
   diag_thread_element(t, kb, i, j, all);        // conversions: every lower element

@@ -192,9 +192,13 @@ __device__ __forceinline__ void digits7(long long X, __half* out, size_t stride)
     out[a * stride] = __hsub(__ushort_as_half((unsigned short)(0x6600 + d[a])), __ushort_as_half(0x6600));
 }
 
-// Slices and exponent of one 64-value row held by a warp (lane: value k and
-// k + 32); all lanes call it.  mark: a row that holds an infinity or NaN gets
-// the exponent kBadExp, which makes NaN of every element it updates.
+// Slices of one row of 64 values held by a warp (lane: value k and k + 32);
+// all lanes call it.  VROW false: a row of U, re | im.  VROW true: the two
+// rows a column of the product reads (vrow): re | im for the real part of
+// P C^H and -im | re for the imaginary part, so that one MMA makes both.
+// *exp_out: the row's exponent; mark: a row that holds an infinity or NaN
+// gets kBadExp, which makes NaN of every element it updates.
+template <bool VROW>
 __device__ __forceinline__ void slice_row(double re, double im, int lane, __half* base, size_t stride, int* exp_out,
                                           bool mark) {
   // e = frexp exponent of the row's largest magnitude, from the biased
@@ -206,8 +210,17 @@ __device__ __forceinline__ void slice_row(double re, double im, int lane, __half
   const long long Xr = fixed56(re, e), Xi = fixed56(im, e);
   digits7(Xr, base + lane, stride);
   digits7(Xi, base + lane + 32, stride);
+  if constexpr (VROW) {
+    __half* second = base + 16 * KR;   // the imaginary part's row of the same column
+    digits7(-Xi, second + lane, stride);
+    digits7(Xr, second + lane + 32, stride);
+  }
   if (lane == 0) *exp_out = (mark && emax == 0x7FFu) ? kBadExp : e;
 }
+
+// Row of V planes that holds column j's real-part row (its imaginary-part row
+// lies 16 further): 16 columns' pairs of rows are contiguous, one TMA box.
+__device__ __forceinline__ size_t vrow(size_t j) { return (j >> 4) * 32 + (j & 15); }
 
 // The Hermitian sweep's panel and its slices in one launch (the look-ahead
 // chain's critical path): for every row i outside the block K (warp per
@@ -221,8 +234,9 @@ __device__ __forceinline__ void slice_row(double re, double im, int lane, __half
 // gathered in the low word; the FP64 pipe keeps only the conversions.
 template <bool FF, bool FFD>
 __global__ void __launch_bounds__(256) panel_slice_kernel(const __grid_constant__ OzBatch b, int k0, int rows_total,
-                                                          int buf, __half* __restrict__ U, __half* __restrict__ V,
-                                                          int* __restrict__ sig, int* __restrict__ tau) {
+                                                          int buf, int vpair, __half* __restrict__ U,
+                                                          __half* __restrict__ V, int* __restrict__ sig,
+                                                          int* __restrict__ tau) {
   __shared__ double2 Ds[NB][NB];   // FF: float4 (re hi, re lo, im hi, im lo)
   __shared__ double2 Cs[8][NB];
   const OzMat& M = b.m[blockIdx.y];
@@ -309,11 +323,14 @@ __global__ void __launch_bounds__(256) panel_slice_kernel(const __grid_constant_
   }
   if (lane >= kb) pv = cv = make_double2(0.0, 0.0);
   const size_t row = (size_t)M.row_off + i;
-  const size_t base = (size_t)buf * S * rows_total * KR + row * KR;
-  slice_row(pv.x, pv.y, lane, U + base, (size_t)rows_total * KR, sig + (size_t)buf * rows_total + row,
-            !FF);
-  slice_row(cv.x, cv.y, lane, V + base, (size_t)rows_total * KR, tau + (size_t)buf * rows_total + row,
-            !FF);
+  slice_row<false>(pv.x, pv.y, lane, U + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
+                   sig + (size_t)buf * rows_total + row, !FF);
+  if (vpair)
+    slice_row<true>(cv.x, cv.y, lane, V + ((size_t)buf * S * 2 * rows_total + vrow(row)) * KR,
+                    (size_t)2 * rows_total * KR, tau + (size_t)buf * rows_total + row, !FF);
+  else   // real values: the real part's rows alone
+    slice_row<false>(cv.x, cv.y, lane, V + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
+                     tau + (size_t)buf * rows_total + row, !FF);
 }
 
 // Slices for the general (Gauss-Jordan) update A -= Cp R of the pivoted
@@ -344,9 +361,12 @@ __global__ void __launch_bounds__(256) slice_general_kernel(const __grid_constan
     im = -v.y;
   }
   const size_t row = (size_t)M.row_off + i;
-  __half* out = (blockIdx.z == 0 ? U : V) + (size_t)buf * S * rows_total * KR + row * KR;
-  slice_row(re, im, lane, out, (size_t)rows_total * KR,
-            (blockIdx.z == 0 ? sig : tau) + (size_t)buf * rows_total + row, mark != 0);
+  if (blockIdx.z == 0)
+    slice_row<false>(re, im, lane, U + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
+                     sig + (size_t)buf * rows_total + row, mark != 0);
+  else
+    slice_row<true>(re, im, lane, V + ((size_t)buf * S * 2 * rows_total + vrow(row)) * KR,
+                    (size_t)2 * rows_total * KR, tau + (size_t)buf * rows_total + row, mark != 0);
 }
 
 // Rows of the block K after the general update: A[k0 + r][j] = R[r][j].
@@ -362,15 +382,32 @@ __global__ void rows_from_r_kernel(const __grid_constant__ OzBatch b, int k0) {
 
 // ---------------------------------------------------------------------------
 // Persistent, pipelined form of the update.  A CTA takes work items of up to
-// kJPI column tiles of one row tile I: the row's U slices are loaded once per item, the V slices of
-// consecutive tiles are double-buffered, and one control thread (warp 16)
-// issues the TMA copies and the MMAs.  The 16 epilogue warps first read the
-// tile's 14 accumulators out of tensor memory and combine the levels in
-// double FP32 (registers), then release tensor memory -- the next tile's
-// MMAs start -- and apply the FP64 subtraction while they run.
+// kJPI column tiles of one row tile I: the row's U slices are loaded once per
+// item.  A complex tile is worked on as two halves of 16 columns, each with its
+// own accumulators in tensor memory (SL levels x 16 columns, real and imaginary
+// parts side by side: 224 of 512 columns) and its own group of 8 epilogue
+// warps, so the tensor cores fill one half's sums while the other half's are
+// used; tiles of real values alternate between the two sets and groups.  One
+// control thread (warp 16) issues the TMA copies (V double-buffered) and the
+// MMAs.  An epilogue thread reads its old values of A while the MMAs run, joins
+// the levels as it reads them out of tensor memory and subtracts at once.
+//
+// Per 128 x 32 tile and SM: 1.9 us of MMAs (4 KB of U from shared memory per MMA),
+// 2.0 us of FP64 adds (one per word), 1.9 us of instruction issue (level sums and
+// conversions); 2.9 us of HBM where the matrix exceeds L2.  Measured 4.6 us:
+// stamps show the control thread (2.3 us a half: MMA issue 1.1, the wait for the
+// half before and its copies 0.7) and the reads of tensor memory (1.9 us, slower
+// beside MMAs) in turn.  Bulk launch at N_G 7180 254 -> 232 us, six matrices of
+// 2120 157 -> 142 us, with FP64 inputs 308 -> 261 and 193 -> 162 us, against one
+// set of accumulators drained before the FP64 part.  Separate warps for copies
+// and MMAs with lists of tiles in shared memory (MMAs of one half always beside
+// reads of the other, both twice as slow) measured 240 and 148 us; a third V
+// buffer leaves less shared memory to other streams' kernels (three concurrent
+// solves 1 to 8% slower).
 constexpr int kPipeEpiWarps = 16;
 constexpr int kPipeThreads = (kPipeEpiWarps + 1) * 32;
 static_assert(kPipeThreads == kDiagThreads, "the look-ahead CTA sweeps the next diagonal block");
+constexpr int kVRing = 2;              // V units in flight
 
 
 // Bounded wait that also gives up when the CTA aborts.
@@ -393,6 +430,31 @@ __device__ __forceinline__ long long join_levels(const uint32_t (&x)[7][4], int 
   return (hi << 15) + ((lo + 256) >> 9);
 }
 
+// The level sums of accumulator q as a double-FP32 pair: level L enters scaled
+// by 2^-8L (exact), folded into fused multiply-adds (the roundings of scaling
+// first).  Levels 1 .. two_sum that reach the running sum's last bits are
+// two-summed into the high word (with seven slices the target is near 2^-48:
+// levels 1 and 2; with five near 2^-34: level 1); deeper levels lie below
+// the sum's last bit at the target precision and go to the low word.
+template <int SL>
+__device__ __forceinline__ void sum_levels(const uint32_t (&x)[SL][4], int q, float& h, float& l) {
+  constexpr int two_sum = SL >= 7 ? 2 : 1;
+  h = __uint_as_float(x[0][q]);
+  l = 0.f;
+#pragma unroll
+  for (int L = 1; L < SL; ++L) {
+    const float w = ldexpf(1.f, -BETA * L), v = __uint_as_float(x[L][q]);
+    if (L <= two_sum) {
+      float sm, e;
+      two_sum_scaled(h, v, w, sm, e);
+      h = sm;
+      l = __fadd_rn(l, e);
+    } else {
+      l = __fmaf_rn(v, w, l);
+    }
+  }
+}
+
 // SL: slices used per value (the most significant SL of the S stored): 7
 // gives an update error near 2^-48 of its scale, 5 near 2^-34.  FFC: the
 // look-ahead CTA sweeps the next diagonal block in double FP32 (about 2^-46
@@ -406,10 +468,10 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
   // column tiles per bulk work item, a compile-time constant (a runtime
   // width costs 2% in the item decode)
   constexpr int wide = NARROW ? 2 : (SL < 7 ? 3 : kJPI);
-  // Levels 1 .. kTwoSumLevels are summed exactly (two-sum) into the high
-  // word: with 7 slices the target is near 2^-48, so levels 1 and 2 (2^-8,
-  // 2^-16 of the sum) need it; with 5 slices (near 2^-34) only level 1.
-  constexpr int kTwoSumLevels = SL >= 7 ? 2 : 1;
+  // Units of a tile: its two halves (16 columns, real and imaginary parts: 32
+  // accumulator columns a level; accumulators h), or for real values the tile
+  // itself (32 columns; accumulators of the tile's parity).
+  constexpr int UN = realv ? 1 : 2, UC = BN / UN;
   const OzMat& M = b.m[blockIdx.y];
   const int ng = M.ng;
   if (k0 >= ng) return;
@@ -425,13 +487,13 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* us = smem;                          // SL x 16 KiB
-  unsigned char* vs = smem + SL * kUTile;            // 2 x SL x 4 KiB
-  uint64_t* u_full = reinterpret_cast<uint64_t*>(vs + 2 * SL * kVTile);
-  uint64_t* v_full = u_full + 1;                     // [2]
-  uint64_t* v_empty = v_full + 2;                    // [2]
-  uint64_t* t_full = v_empty + 2;
-  uint64_t* t_empty = t_full + 1;
-  uint64_t* u_empty = t_empty + 1;                   // an item's MMAs are complete
+  unsigned char* vs = smem + SL * kUTile;            // kVRing x SL x 4 KiB
+  uint64_t* u_full = reinterpret_cast<uint64_t*>(vs + kVRing * SL * kVTile);
+  uint64_t* v_full = u_full + 1;                     // [kVRing]
+  uint64_t* v_empty = v_full + kVRing;               // [kVRing]
+  uint64_t* t_full = v_empty + kVRing;               // [2] a half's sums are complete
+  uint64_t* t_empty = t_full + 2;                    // [2] a half's sums have been read
+  uint64_t* u_empty = t_empty + 2;                   // an item's MMAs are complete
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(u_empty + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   __shared__ DiagSmem dsm;
@@ -440,12 +502,15 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
   const bool control = warp == kPipeEpiWarps;
   if (threadIdx.x == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(u_full)) : "memory");
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < kVRing; ++q) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(v_full + q)) : "memory");
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(v_empty + q)) : "memory");
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(t_full)) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(t_empty)), "r"(kPipeEpiWarps) : "memory");
+    for (int q = 0; q < 2; ++q) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(t_full + q)) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(t_empty + q)), "r"(kPipeEpiWarps / 2)
+                   : "memory");
+    }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(u_empty)) : "memory");
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -463,7 +528,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
   int t = 0;           // tiles processed by this CTA (buffer and phase bookkeeping)
   int items_done = 0;  // items processed
   int u_loads = 0;     // U loads issued (control; phase of u_full)
-  int vissued = 0;     // V loads issued (control)
+  int vissued = 0;     // V units issued (control)
   PipeCursor cursor;
   for (int item = blockIdx.x; item < nitems; item += gridDim.x, ++items_done) {
     int I, J0, J1;
@@ -487,69 +552,60 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
             tma_load_2d(us + a * kUTile, &umap, u_full, 0, slice_base + a * rows_total + M.row_off + i0);
           ++u_loads;
         }
-        auto issue_v = [&](int tt, int J) {
-          const int bq = tt & 1;
-          if (tt >= 2 && !mbar_wait_ab(&v_empty[bq], ((tt - 2) >> 1) & 1, abort_flag)) return false;
+        // unit uu (counted over the CTA's life) of the item: columns UC (uu % UN) .. of tile Js[(uu - uu0) / UN]
+        const int uu0 = UN * t, uu1 = UN * (t + nt);
+        auto issue_v = [&](int uu) {
+          const int bq = uu % kVRing;
+          if (uu >= kVRing && !mbar_wait_ab(&v_empty[bq], (uu / kVRing - 1) & 1, abort_flag)) return false;
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(v_full + bq)),
                        "r"((uint32_t)(SL * kVTile))
                        : "memory");
+          const int j = Js[(uu - uu0) / UN] * BN + (uu % UN) * UC;
           for (int a = 0; a < SL; ++a)
             tma_load_2d(vs + (bq * SL + a) * kVTile, &vmap, v_full + bq, 0,
-                        slice_base + a * rows_total + M.row_off + J * BN);
+                        UN * (slice_base + a * rows_total + M.row_off + j));
+          vissued = uu + 1;
           return true;
         };
-        ok = ok && issue_v(t, Js[0]);
-        if (ok) vissued = t + 1;
-        for (int k = 0; k < nt && ok; ++k) {
-          const int tt = t + k;
-          if (k + 1 < nt) {
-            ok = issue_v(tt + 1, Js[k + 1]);
-            vissued = tt + 2;
-            if (!ok) break;
+        ok = ok && issue_v(uu0);
+        for (int uu = uu0; uu < uu1 && ok; ++uu) {
+          if (uu + 1 < uu1 && !issue_v(uu + 1)) {
+            ok = false;
+            break;
           }
-          if ((k == 0 && !mbar_wait_ab(u_full, u_phase, abort_flag)) ||
-              !mbar_wait_ab(&v_full[tt & 1], (tt >> 1) & 1, abort_flag) ||
-              (tt > 0 && !mbar_wait_ab(t_empty, (tt - 1) & 1, abort_flag))) {
+          const int tt = uu / UN, bq = uu % kVRing;
+          const int acc = realv ? tt & 1 : uu & 1, use = realv ? tt >> 1 : tt;   // accumulators, and how often used before
+          if ((uu == uu0 && !mbar_wait_ab(u_full, u_phase, abort_flag)) ||
+              !mbar_wait_ab(&v_full[bq], (uu / kVRing) & 1, abort_flag) ||
+              (use > 0 && !mbar_wait_ab(&t_empty[acc], (use - 1) & 1, abort_flag))) {
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          // Tensor memory holds the real parts of the SL level sums in columns
-          // 32 L and their imaginary parts in 32 (SL + L).  The V slices lie
-          // one after the other in shared memory, so for one U slice a the
-          // products with V slices 0 .. SL-1-a are one MMA of N = 32 (SL - a)
-          // columns into levels a .. SL-1: each U chunk is read once per
-          // slice instead of once per slice pair (shared-memory traffic per
-          // tile 2.5x lower at seven slices).  A descriptor's start address
-          // is its low 14 bits (address / 16, no carry below 256 KiB), so
-          // every operand descriptor is the base's plus a constant; level L
-          // is first written by slice a = 0.
-          const uint64_t du = sdesc(smem_u32(us)), dv = sdesc(smem_u32(vs + (tt & 1) * SL * kVTile));
+          // Level L of the unit's sums lies in columns 32 L (16 of the real
+          // parts, then 16 of the imaginary parts; real values: 32).  The V
+          // slices lie one after the other in shared memory, so for one U slice
+          // a the products with V slices 0 .. SL-1-a are one MMA of N = 32
+          // (SL - a) columns into levels a .. SL-1, and the two rows of a column
+          // (vrow) make both parts: each U chunk is read once per slice.  A
+          // descriptor's start address is its low 14 bits (address / 16, no
+          // carry below 256 KiB), so every operand descriptor is the base's plus
+          // a constant; slice a = 0 writes every level first.
+          const uint64_t du = sdesc(smem_u32(us)), dv = sdesc(smem_u32(vs + bq * SL * kVTile));
 #pragma unroll
           for (int a = 0; a < SL; ++a) {
-            const uint32_t dre = tmem + 32 * a, dim = tmem + 32 * (SL + a);
+            const uint32_t d = tmem + (acc * SL + a) * 32;
             const uint64_t ua = du + (uint64_t)((a * kUTile) >> 4);
-            const uint32_t ida = idesc(false, 32 * (SL - a)), idna = idesc(true, 32 * (SL - a));
-            const uint32_t acc0 = a == 0 ? 0u : 1u;
-            if constexpr (realv) {
-              mma(dre, ua, dv, ida, acc0);
-              mma(dre, ua + 2, dv + 2, ida, 1u);
-            } else {
-              mma(dre, ua, dv, ida, acc0);            // byte offsets 32 q along K: +2 q in the descriptor
-              mma(dre, ua + 2, dv + 2, ida, 1u);
-              mma(dre, ua + 4, dv + 4, ida, 1u);
-              mma(dre, ua + 6, dv + 6, ida, 1u);
-              mma(dim, ua + 4, dv + 0, ida, acc0);
-              mma(dim, ua + 6, dv + 2, ida, 1u);
-              mma(dim, ua + 0, dv + 4, idna, 1u);
-              mma(dim, ua + 2, dv + 6, idna, 1u);
-            }
+            const uint32_t id = idesc(false, 32 * (SL - a));
+            // byte offsets 32 q along K: +2 q in the descriptor; real values fill the first half of the row
+#pragma unroll
+            for (int q = 0; q < (realv ? 2 : 4); ++q) mma(d, ua + 2 * q, dv + 2 * q, id, a == 0 && q == 0 ? 0u : 1u);
           }
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_u32(v_empty + (tt & 1)))
+                           smem_u32(v_empty + bq))
                        : "memory");
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_u32(t_full))
+                           smem_u32(t_full + acc))
                        : "memory");
         }
         if (ok)
@@ -563,14 +619,16 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
       }
       __syncwarp();
     } else {
-      // ---------------- epilogue warps: rows 32 (warp % 4) .. + 31, columns 8 (warp / 4) .. + 7.
-      // The accumulators are read in the 16x256b shape: lane l holds rows
-      // g, g + 8, g + 16, g + 24 (g = l / 4) and columns 2 (l % 4), + 1, so one
-      // warp-wide access of A touches 8 rows of 128 contiguous bytes instead
-      // of 32 rows of 16 (four times fewer cache lines per instruction).
-      const int quad = warp & 3, part = warp >> 2;
+      // ---------------- epilogue warps: group warp / 8 takes one half of every tile (real values: every other tile),
+      // its warps rows 32 (warp % 4) .. + 31 and eight columns (real values:
+      // sixteen, eight at a time).  The accumulators are read in the 16x256b
+      // shape: lane l holds rows g, g + 8, g + 16, g + 24 (g = l / 4) and
+      // columns 2 (l % 4), + 1, so one warp-wide access of A touches 8 rows of
+      // 128 contiguous bytes instead of 32 rows of 16 (four times fewer cache
+      // lines).
+      const int group = warp >> 3, quad = warp & 3, part = (warp >> 2) & 1;
       const int g = lane >> 2, cl = 2 * (lane & 3);
-      const int c0 = part * 8;
+      const int c0 = realv ? part * 16 : group * UC + part * 8;
       // rows r0 + 8 m (m = 0 .. 3) and their exponents sigma
       const int r0 = i0 + quad * 32 + g;
       auto row_ok = [&](int i) { return i < ng && !(i >= k0 && i < k0 + kb); };
@@ -588,27 +646,35 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
         const double2* row = M.A + (size_t)prow * ng;
         asm volatile("prefetch.global.L2 [%0];" ::"l"(row + j));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(row + min(j + 7, ng - 1)));
+        if constexpr (realv) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + min(j + 15, ng - 1)));
       };
-      // the column exponents of tile kk (read one tile ahead)
-      auto load_tau = [&](int kk, int (&tv)[2]) {
+      // the exponents of tile kk's columns from c (complex tiles: read one tile ahead)
+      auto load_tau = [&](int kk, int c, int (&tv)[2]) {
 #pragma unroll
         for (int n = 0; n < 2; ++n) {
-          const int j = kk < nt ? Js[kk] * BN + c0 + cl + n : ng;
+          const int j = kk < nt ? Js[kk] * BN + c + cl + n : ng;
           tv[n] = j < ng ? tau[buf * rows_total + M.row_off + j] : 0;
         }
       };
-      // element e = 2 m + n of tile kk: row r0 + 8 m, column Js[kk] BN + c0 + cl + n,
+      // element e = 2 m + n of tile kk from column c: row r0 + 8 m, column Js[kk] BN + c + cl + n,
       // scale exponent ei[m] + tv[n] - 16.  Bit e of the mask: the element is
       // updated; bit 8 + e: its old value is read (columns of the block K
       // start from zero in the Gauss-Jordan form).
       int tv[2];
+      // a lane's pair of columns starts at an even index: 32-byte aligned in every row
+      const bool paired = (ng & 1) == 0 && (reinterpret_cast<uintptr_t>(M.A) & 31u) == 0;
       unsigned mask = 0;
-      auto tile_mask = [&](int kk) {
+      auto tile_mask = [&](int kk, int c) {
         const int j0 = Js[kk] * BN;
+        // inside the matrix, below the diagonal and clear of the block's rows
+        // and columns: every element is live
+        if (i0 + BM <= ng && (mode == 3 ? j0 + BN <= ng : j0 + BN <= i0) && (i0 >= k0 + kb || i0 + BM <= k0) &&
+            (j0 >= k0 + kb || j0 + BN <= k0))
+          return 0xFFFFu;
         unsigned mk = 0;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const int i = r0 + 8 * (e >> 1), j = j0 + c0 + cl + (e & 1);
+          const int i = r0 + 8 * (e >> 1), j = j0 + c + cl + (e & 1);
           const bool jblock = j >= k0 && j < k0 + kb;
           const bool live = row_ok(i) && j < ng && (mode == 3 ? true : (j <= i && !jblock));
           mk |= (live ? 1u : 0u) << e;
@@ -616,76 +682,82 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
         }
         return mk;
       };
-      if (nt > 0) {
-        load_tau(0, tv);
-        mask = tile_mask(0);
+      if (nt > 0 && !realv) {
+        load_tau(0, c0, tv);
+        mask = tile_mask(0, c0);
       }
       prefetch_a(0);
       for (int k = 0; k < nt; ++k) {
         const int tt = t + k;
         const int j0 = Js[k] * BN;
-        prefetch_a(k + 1);
-        // the next tile's column exponents, used after this tile's FP64 part
+        if constexpr (realv) {
+          prefetch_a(k + 2);
+          if ((tt & 1) != group) continue;
+        } else {
+          prefetch_a(k + 1);
+        }
+        bool have = true;
+#pragma unroll 1
+        for (int ch = 0; ch < (realv ? 2 : 1) && have; ++ch) {
+        const int c = c0 + 8 * ch;
+        if constexpr (realv) {
+          load_tau(k, c, tv);
+          mask = tile_mask(k, c);
+        }
+        // the tile's old values, read while its MMAs run: a lane's two columns
+        // are adjacent, one 256-bit access per row where both are read
+        // (written) and the pair is 32-byte aligned (every row for an even N_G
+        // and an aligned matrix), else one 128-bit access per element
+        double2 av[8];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const size_t off = (size_t)(r0 + 8 * m) * ng + j0 + c + cl;
+          const unsigned rd = (mask >> (8 + 2 * m)) & 3u;
+          av[2 * m] = av[2 * m + 1] = make_double2(0.0, 0.0);
+          if (rd == 3u && paired) {
+            ld_pair(M.A + off, av[2 * m], av[2 * m + 1]);
+          } else {
+            if (rd & 1u) av[2 * m] = M.A[off];
+            if (rd & 2u) av[2 * m + 1] = M.A[off + 1];
+          }
+        }
+        // the next tile's column exponents, used after this tile
         int tnext[2];
-        load_tau(k + 1, tnext);
-        bool have = mbar_wait_ab(t_full, tt & 1, abort_flag);
+        if constexpr (!realv) load_tau(k + 1, c0, tnext);
+        have = mbar_wait_ab(&t_full[group], (realv ? tt >> 1 : tt) & 1, abort_flag);
         have = __all_sync(0xffffffffu, have) != 0;
-        float hr[8], lr[8], hm[8], lm[8];      // FFC: level sums as double-FP32 pairs
-        long long xr[8], xm[8];                // FP64 inputs: as integers
         if (have) {
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          // Four rounds (two 16-row halves, real then imaginary parts):
-          // each issues the loads of all SL levels before one wait.
-          // level L enters scaled by w = 2^-8L (exact), folded into fused
-          // multiply-adds: the same roundings as scaling first
-          auto combine = [&](const uint32_t (&x)[SL][4], int hb, float (&h)[8], float (&l)[8]) {
+          // Four rounds (two 16-row halves, real then imaginary parts): each
+          // issues the loads of all SL levels before one wait, joins the
+          // levels, applies the scale 2^e2 (sigma_i tau_j 2^-16) in the
+          // conversion and subtracts: one FP64 add per word.
 #pragma unroll
-            for (int L = 0; L < SL; ++L) {
-              const float w = ldexpf(1.f, -BETA * L);
+          for (int rb = 0; rb < (realv ? 2 : 4); ++rb) {
+            const int hb = realv ? rb : rb >> 1, im = realv ? 0 : rb & 1;
+            const uint32_t tl = tmem + ((uint32_t)(quad * 32 + 16 * hb) << 16) + group * SL * 32 + im * UC + (realv ? c : part * 8);
+            uint32_t x[SL][4];
 #pragma unroll
-              for (int qq = 0; qq < 4; ++qq) {
-                const int q = 4 * hb + qq;
-                const float v = __uint_as_float(x[L][qq]);
-                if (L == 0) {
-                  h[q] = v;
-                  l[q] = 0.f;
-                } else if (L <= kTwoSumLevels) {
-                  // levels that can reach the running sum's last bits: exact two-sum
-                  float sm, e;
-                  two_sum_scaled(h[q], v, w, sm, e);
-                  h[q] = sm;
-                  l[q] = __fadd_rn(l[q], e);
-                } else {
-                  // deeper levels lie below the sum's last bit at the target
-                  // precision: they go to the low word
-                  l[q] = __fmaf_rn(v, w, l[q]);
-                }
-              }
+            for (int L = 0; L < SL; ++L) tmem_ld16x256(tl + 32 * L, x[L]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (realv ? (ch == 1 && rb == 1) : rb == 3) {
+              // every sum is read: the accumulators are free for the next MMAs
+              asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+              __syncwarp();
+              if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(t_empty + group)) : "memory");
             }
-          };
 #pragma unroll
-          for (int hb = 0; hb < 2; ++hb) {
-            const uint32_t tl = tmem + ((uint32_t)(quad * 32 + 16 * hb) << 16) + c0;
-#pragma unroll
-            for (int part = 0; part < (realv ? 1 : 2); ++part) {
-              uint32_t x[SL][4];
-#pragma unroll
-              for (int L = 0; L < SL; ++L) tmem_ld16x256(tl + 32 * (part * SL + L), x[L]);
-              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-              if constexpr (!FFC) {
-#pragma unroll
-                for (int qq = 0; qq < 4; ++qq) (part == 0 ? xr : xm)[4 * hb + qq] = join_levels(x, qq);
-              } else if (part == 0) {
-                combine(x, hb, hr, lr);
-              } else {
-                combine(x, hb, hm, lm);
-              }
-            }
-            if constexpr (realv) {
-#pragma unroll
-              for (int qq = 0; qq < 4; ++qq) {
-                hm[4 * hb + qq] = lm[4 * hb + qq] = 0.f;
-                xm[4 * hb + qq] = 0;
+            for (int qq = 0; qq < 4; ++qq) {
+              const int e = 4 * hb + qq, m = e >> 1;
+              const int e2 = ei[m] + tv[e & 1] - 2 * BETA;
+              double& dst = im ? av[e].y : av[e].x;
+              if constexpr (FFC) {
+                float hs, ls;
+                sum_levels<SL>(x, qq, hs, ls);
+                dst -= ff2d_scaled(hs, ls, e2);
+              } else {   // unit 2^-55 against the pairs' 2^-16
+                dst -= i64_to_scaled(join_levels(x, qq), e2 - 39);
               }
             }
           }
@@ -693,60 +765,23 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
           *abort_flag = 1;
           atomicExch(status, (int)kDevTimeout);
         }
-        // tensor memory is free for the next tile's MMAs
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(t_empty)) : "memory");
-        if (!have) continue;
-        // the tile's FP64 values, read while the next tile's MMAs run
-        // a lane's two columns are adjacent: one 256-bit access per row
-        // where both are read (written) and the pair is 32-byte aligned
-        // (every row for an even N_G and an aligned matrix), else one
-        // 128-bit access per element
-        double2 av[8];
+        if (!have) break;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-          const size_t off = (size_t)(r0 + 8 * m) * ng + j0 + c0 + cl;
-          const unsigned rd = (mask >> (8 + 2 * m)) & 3u;
-          av[2 * m] = av[2 * m + 1] = make_double2(0.0, 0.0);
-          if (rd == 3u && !(reinterpret_cast<uintptr_t>(M.A + off) & 31u)) {
-            ld_pair(M.A + off, av[2 * m], av[2 * m + 1]);
-          } else {
-            if (rd & 1u) av[2 * m] = M.A[off];
-            if (rd & 2u) av[2 * m + 1] = M.A[off + 1];
-          }
-        }
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          const size_t off = (size_t)(r0 + 8 * m) * ng + j0 + c0 + cl;
-          double2 o[2];
-#pragma unroll
-          for (int n = 0; n < 2; ++n) {
-            const int e = 2 * m + n;
-            const double2 v = av[e];
-            const int e2 = ei[m] + tv[n] - 2 * BETA;
-            // scale 2^e2 (sigma_i tau_j 2^-16) applied in the conversion; one
-            // FP64 add per word
-            if constexpr (FFC) {
-              o[n].x = v.x - ff2d_scaled(hr[e], lr[e], e2);
-              o[n].y = realv ? v.y : v.y - ff2d_scaled(hm[e], lm[e], e2);
-            } else {   // unit 2^-55 against the pairs' 2^-16
-              o[n].x = v.x - i64_to_scaled(xr[e], e2 - 39);
-              o[n].y = realv ? v.y : v.y - i64_to_scaled(xm[e], e2 - 39);
-            }
-          }
+          const size_t off = (size_t)(r0 + 8 * m) * ng + j0 + c + cl;
           const unsigned wr = (mask >> (2 * m)) & 3u;
-          if (wr == 3u && !(reinterpret_cast<uintptr_t>(M.A + off) & 31u)) {
-            st_pair(M.A + off, o[0], o[1]);
+          if (wr == 3u && paired) {
+            st_pair(M.A + off, av[2 * m], av[2 * m + 1]);
           } else {
-            if (wr & 1u) M.A[off] = o[0];
-            if (wr & 2u) M.A[off + 1] = o[1];
+            if (wr & 1u) M.A[off] = av[2 * m];
+            if (wr & 2u) M.A[off + 1] = av[2 * m + 1];
           }
         }
-        if (k + 1 < nt) {
+        if (!realv && k + 1 < nt) {
           tv[0] = tnext[0];
           tv[1] = tnext[1];
-          mask = tile_mask(k + 1);
+          mask = tile_mask(k + 1, c0);
+        }
         }
       }
     }
@@ -789,9 +824,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
     const uint64_t t2 = globaltimer();
     while (!*abort_flag && !mbar_try_wait(u_empty, (u_loads - 1) & 1) && globaltimer() - t2 < kWaitNs) {
     }
-    for (int tt = max(0, vissued - 2); tt < vissued; ++tt) {
+    for (int uu = max(0, vissued - kVRing); uu < vissued; ++uu) {
       const uint64_t t1 = globaltimer();
-      while (!mbar_try_wait(&v_full[tt & 1], (tt >> 1) & 1) && globaltimer() - t1 < kWaitNs) {
+      while (!mbar_try_wait(&v_full[uu % kVRing], (uu / kVRing) & 1) && globaltimer() - t1 < kWaitNs) {
       }
     }
   }
@@ -805,9 +840,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
 
 }  // namespace oz
 
-// Dynamic shared memory of update_pipe_kernel with SL slices: U, two V
-// buffers, alignment slack and the barriers.
-size_t pipe_smem(int slices) { return (size_t)slices * (oz::kUTile + 2 * oz::kVTile) + 1024 + 128; }
+// Dynamic shared memory of update_pipe_kernel with SL slices: U, the ring of
+// V halves, alignment slack and the barriers.
+size_t pipe_smem(int slices) { return (size_t)slices * (oz::kUTile + oz::kVRing * oz::kVTile) + 1024 + 128; }
 
 // State of one batched sweep that uses the tensor-core update.
 struct OzPlan {
@@ -861,25 +896,27 @@ int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2
   // two slice buffers: a step may slice while the previous step's update
   // still reads its own
   const size_t sb = (size_t)2 * S * rows * KR * sizeof(__half);
-  if ((rc = c->pool.alloc(sb, &plan->U.ptr)) != BGW_OK || (rc = c->pool.alloc(sb, &plan->V.ptr)) != BGW_OK ||
+  if ((rc = c->pool.alloc(sb, &plan->U.ptr)) != BGW_OK || (rc = c->pool.alloc(real_values ? sb : 2 * sb, &plan->V.ptr)) != BGW_OK ||
       (rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &plan->sig.ptr)) != BGW_OK ||
       (rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &plan->tau.ptr)) != BGW_OK ||
       (rc = c->pool.alloc((size_t)nmat * NB * NB * sizeof(float4), &plan->dff.ptr)) != BGW_OK)
-    return fail(c, rc, "tensor-core inverse: slice buffers (%zu B each) could not be allocated", sb);
+    return fail(c, rc, "tensor-core inverse: slice buffers (%zu B) could not be allocated", 3 * sb);
   for (int m = 0; m < nmat; ++m) plan->batch.m[m].Dff = plan->dff.as<float4>() + (size_t)m * NB * NB;
   cuuint64_t gdim[2] = {(cuuint64_t)KR, (cuuint64_t)2 * S * rows};
   cuuint64_t gstride[1] = {(cuuint64_t)KR * sizeof(__half)};
   cuuint32_t estr[2] = {1, 1};
   cuuint32_t ubox[2] = {(cuuint32_t)KR, (cuuint32_t)BM};
+  // 16 columns of two rows each (vrow); real values: 32 of one
   cuuint32_t vbox[2] = {(cuuint32_t)KR, (cuuint32_t)BN};
+  cuuint64_t vdim[2] = {(cuuint64_t)KR, (cuuint64_t)(real_values ? 2 : 4) * S * rows};
   if (encode(&plan->umap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plan->U.ptr, gdim, gstride, ubox, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-      encode(&plan->vmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plan->V.ptr, gdim, gstride, vbox, estr,
+      encode(&plan->vmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plan->V.ptr, vdim, gstride, vbox, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return fail(c, BGW_ECUDA, "tensor-core inverse: tensor map encoding failed");
-  // U slices, two V buffers, alignment and barriers: about 170 KiB dynamic (7 slices)
+  // U slices, V ring, alignment and barriers: about 170 KiB dynamic (7 slices)
   const size_t psmem = pipe_smem(slices);
 #define BGW_PIPE_ATTR(RV, SLC, FF)                                                                        \
   BGW_CUDA(c, cudaFuncSetAttribute(update_pipe_kernel<RV, SLC, FF, false>,                                       \
@@ -921,16 +958,16 @@ int oz_panel_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, cudaStream_
   // for every step after the first
   if (plan->ff_chain && k0 > 0)
     panel_slice_kernel<true, true><<<dim3(rpad / 8, plan->nmat), 256, 0, st>>>(
-        plan->batch, k0, plan->rows_total, buf, plan->U.as<__half>(), plan->V.as<__half>(), plan->sig.as<int>(),
-        plan->tau.as<int>());
+        plan->batch, k0, plan->rows_total, buf, plan->real_values ? 0 : 1, plan->U.as<__half>(), plan->V.as<__half>(),
+        plan->sig.as<int>(), plan->tau.as<int>());
   else if (plan->ff_chain)
     panel_slice_kernel<true, false><<<dim3(rpad / 8, plan->nmat), 256, 0, st>>>(
-        plan->batch, k0, plan->rows_total, buf, plan->U.as<__half>(), plan->V.as<__half>(), plan->sig.as<int>(),
-        plan->tau.as<int>());
+        plan->batch, k0, plan->rows_total, buf, plan->real_values ? 0 : 1, plan->U.as<__half>(), plan->V.as<__half>(),
+        plan->sig.as<int>(), plan->tau.as<int>());
   else
     panel_slice_kernel<false, false><<<dim3(rpad / 8, plan->nmat), 256, 0, st>>>(
-        plan->batch, k0, plan->rows_total, buf, plan->U.as<__half>(), plan->V.as<__half>(), plan->sig.as<int>(),
-        plan->tau.as<int>());
+        plan->batch, k0, plan->rows_total, buf, plan->real_values ? 0 : 1, plan->U.as<__half>(), plan->V.as<__half>(),
+        plan->sig.as<int>(), plan->tau.as<int>());
   BGW_CUDA(c, cudaGetLastError());
   return BGW_OK;
 }
