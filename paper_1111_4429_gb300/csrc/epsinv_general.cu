@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "runtime.h"
+#include "sweep_common.cuh"
 
 namespace bgw {
 
@@ -39,193 +40,287 @@ struct GenPtrs {
   double2* A[kGB];
 };
 
-__device__ __forceinline__ double cabs1(double2 z) { return fabs(z.x) + fabs(z.y); }
-
-// Partial-pivoting LU of nr (<= 256) rows x kb columns held in P; thread t
-// owns row t.  Picks, column by column, the active row of largest |Re|+|Im|
-// (ties: smallest global row), eliminates that column from the other active
-// rows.  Writes the global rows in selection order to sel and returns their
-// number (min(nr, kb)).  The selection runs in FP32: it only orders the rows
-// (the elimination itself is the FP64 Gauss-Jordan step that follows), and
-// FP32 runs at 64 times the FP64 rate of one SM.
-__device__ __forceinline__ float cabs1f(float2 z) { return fabsf(z.x) + fabsf(z.y); }
-
-__device__ int select_rows(float2 (*P)[kPB + 1], const int* gid, int nr, int kb, int* sel) {
-  __shared__ float wv[kTRows / 32];
-  __shared__ int wg[kTRows / 32], wl[kTRows / 32];
-  __shared__ int win;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  bool active = t < nr;
-  const int cnt = min(nr, kb);
-  for (int j = 0; j < cnt; ++j) {
-    float v = active ? cabs1f(P[t][j]) : -1.f;
-    int g = active ? gid[t] : 0x7fffffff, l = t;
-    for (int o = 16; o > 0; o >>= 1) {
-      const float v2 = __shfl_xor_sync(0xffffffffu, v, o);
-      const int g2 = __shfl_xor_sync(0xffffffffu, g, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
-      if (v2 > v || (v2 == v && g2 < g)) {
-        v = v2;
-        g = g2;
-        l = l2;
-      }
-    }
-    if (lane == 0) {
-      wv[warp] = v;
-      wg[warp] = g;
-      wl[warp] = l;
-    }
-    __syncthreads();
-    if (t == 0) {
-      float bv = wv[0];
-      int bg = wg[0], bl = wl[0];
-      for (int w = 1; w < kTRows / 32; ++w)
-        if (wv[w] > bv || (wv[w] == bv && wg[w] < bg)) {
-          bv = wv[w];
-          bg = wg[w];
-          bl = wl[w];
-        }
-      win = bl;
-      sel[j] = bg;
-    }
-    __syncthreads();
-    const int w = win;
-    if (t == w) active = false;
-    const float2 pv = P[w][j];
-    const float m2 = pv.x * pv.x + pv.y * pv.y;
-    if (active && m2 > 0.f) {
-      const float2 a = P[t][j];
-      const float2 l = make_float2((a.x * pv.x + a.y * pv.y) / m2, (a.y * pv.x - a.x * pv.y) / m2);
-      for (int c = j + 1; c < kb; ++c) {
-        const float2 u = P[w][c];
-        P[t][c] = make_float2(P[t][c].x - (l.x * u.x - l.y * u.y), P[t][c].y - (l.x * u.y + l.y * u.x));
-      }
-    }
-    __syncthreads();
-  }
-  return cnt;
+// z + a b
+__device__ __forceinline__ double2 cfma2(double2 a, double2 b, double2 z) {
+  z.x = fma(a.x, b.x, z.x);
+  z.y = fma(a.x, b.y, z.y);
+  z.x = fma(-a.y, b.y, z.x);
+  z.y = fma(a.y, b.x, z.y);
+  return z;
 }
-
-// FP32 copy of a panel entry.  The values are eps~ entries (finite, far
-// inside the FP32 range); a zero pivot column stays zero.
-__device__ __forceinline__ float2 to_f2(double2 z) { return make_float2((float)z.x, (float)z.y); }
 
 __device__ __forceinline__ double2 cmul2(double2 a, double2 b) {
   return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
 
-// FP64 LU (without further pivoting) of the block D = A[sel][K], the chosen
-// rows in selection order: lu[r][c] holds L below the diagonal (unit
-// diagonal implied) and U on and above it, lu[NB*NB + s] = 1/U_ss.  Run by
-// the CTA that makes the final choice, before the rows are swapped; the
-// buffer P (no longer needed) holds D.
-__device__ void factor_block(const double2* __restrict__ A, int ng, int k0, int kb, const int* sel, void* scratch,
-                             double2* __restrict__ lu, int* __restrict__ status) {
-  double2 (*D)[kPB + 1] = reinterpret_cast<double2 (*)[kPB + 1]>(scratch);
-  __shared__ double2 rinv[kPB];
-  const int tid = threadIdx.x;
-  for (int e = tid; e < kPB * kPB; e += blockDim.x) {
-    const int r = e / kPB, c = e % kPB;
-    D[r][c] = (r < kb && c < kb) ? A[(size_t)sel[r] * ng + k0 + c] : make_double2(r == c ? 1.0 : 0.0, 0.0);
-  }
-  for (int s = 0; s < kb; ++s) {
+// z - a b with one rounding of z
+__device__ __forceinline__ double2 csub2(double2 z, double2 a, double2 b) {
+  const double2 t = cmul2(a, b);
+  return make_double2(z.x - t.x, z.y - t.y);
+}
+
+__device__ __forceinline__ double2 shfl2(double2 v, int src, int width = 32) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, src, width), __shfl_sync(0xffffffffu, v.y, src, width));
+}
+
+// FP32 copy of a panel entry, rounded in the integer pipe (a conversion goes
+// through the FP64 pipe: 4 us of a CTA's 16384).  The values are eps~ entries
+// (finite, far inside the FP32 range); a zero pivot column stays zero.
+__device__ __forceinline__ float2 to_f2(double2 z) { return make_float2(ff_from_int(z.x).x, ff_from_int(z.y).x); }
+
+// Partial-pivoting LU of nr (<= 256) rows gid[] x kb columns of the panel at
+// column k0; thread t owns row t and keeps it in registers.  Picks, column by
+// column, the active row of largest |Re|+|Im| (ties: smallest global row),
+// eliminates that column from the other active rows.  Writes the global rows
+// in selection order to sel and returns their number (min(nr, kb)).  The
+// selection runs in FP32: it only orders the rows (the elimination itself is
+// the FP64 Gauss-Jordan step that follows), and FP32 runs at 64 times the
+// FP64 rate of one SM.
+//
+// A chain of kb dependent searches bounds it.  Each warp finds its own best
+// row with two redux instructions and lays that row down beside the key
+// before the one barrier of the column; after it every warp compares the
+// eight keys itself and reads the winner's row (two sets of rows, so the next
+// column may write while this one is read).  About 33 us a launch once the rows
+// are in L2, latencies of 32 columns with two warps a scheduler.
+struct SelectSmem {
+  float4 row[2][kTRows / 32][kPB / 2];
+  uint2 key[2][kTRows / 32];   // (|Re|+|Im| as ordered bits + 1, global row); 0: no active row
+};
+
+// Columns [j0, j0 + 8) of the panel and the ones after them; x[0] is column j0
+// of the thread's row.  The row moves down by one register with every column's
+// update, so that the loop needs one body a stage: 32 unrolled columns are code
+// that runs once, and with its fetches a launch took 50 us.
+template <int J0>
+__device__ __forceinline__ void select_stage(float2 (&x)[kPB], bool active, unsigned g, int cnt, SelectSmem& sm,
+                                             int* sel) {
+  constexpr int W = kPB - J0;   // columns left
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 1
+  for (int j = J0; j < min(J0 + 8, cnt); ++j) {
+    const float v = fabsf(x[0].x) + fabsf(x[0].y);
+    const unsigned key = active ? (v == v ? __float_as_uint(v) : 0u) + 1u : 0u;
+    const unsigned kmax = __reduce_max_sync(0xffffffffu, key);
+    const unsigned gmin = __reduce_min_sync(0xffffffffu, key == kmax ? g : 0xffffffffu);
+    if (kmax == 0 ? lane == 0 : (active && g == gmin)) {
+      sm.key[j & 1][warp] = make_uint2(kmax, gmin);
+#pragma unroll
+      for (int c = 0; c < W / 2; ++c)
+        sm.row[j & 1][warp][c] = make_float4(x[2 * c].x, x[2 * c].y, x[2 * c + 1].x, x[2 * c + 1].y);
+    }
     __syncthreads();
-    if (tid == 0) {
-      const double2 p = D[s][s];
-      const double m2 = p.x * p.x + p.y * p.y;
-      if (!(m2 > 0.0) || !isfinite(m2)) {
-        atomicExch(status, (int)kDevZeroPivot);
-        rinv[s] = make_double2(0.0, 0.0);
-      } else {
-        const double q = 1.0 / m2;
-        rinv[s] = make_double2(p.x * q, -p.y * q);
+    // the best of the eight: every warp by itself, lane = warp of the key
+    const uint2 k = sm.key[j & 1][lane & 7];
+    uint2 best;
+    best.x = __reduce_max_sync(0xffffffffu, k.x);
+    best.y = __reduce_min_sync(0xffffffffu, k.x == best.x ? k.y : 0xffffffffu);
+    const int bw = __ffs(__ballot_sync(0xffffffffu, k.x == best.x && k.y == best.y)) - 1;
+    if (threadIdx.x == 0) sel[j] = (int)best.y;
+    if (g == best.y) active = false;
+    const float4* row = sm.row[j & 1][bw];
+    float4 q = row[0];
+    const float m2 = q.x * q.x + q.y * q.y;
+    float2 l = make_float2(0.f, 0.f);
+    if (active && m2 > 0.f)
+      l = make_float2((x[0].x * q.x + x[0].y * q.y) / m2, (x[0].y * q.x - x[0].x * q.y) / m2);
+    auto sub = [&](float2 z, float ux, float uy) {
+      return make_float2(fmaf(-l.x, ux, fmaf(l.y, uy, z.x)), fmaf(-l.x, uy, fmaf(-l.y, ux, z.y)));
+    };
+    if (active) {
+      x[0] = sub(x[1], q.z, q.w);
+#pragma unroll
+      for (int c = 1; c < W / 2; ++c) {
+        q = row[c];
+        x[2 * c - 1] = sub(x[2 * c], q.x, q.y);
+        x[2 * c] = sub(x[2 * c + 1], q.z, q.w);
       }
-    }
-    __syncthreads();
-    for (int r = s + 1 + tid; r < kb; r += blockDim.x) D[r][s] = cmul2(D[r][s], rinv[s]);
-    __syncthreads();
-    const int w = kb - 1 - s;
-    for (int e = tid; e < w * w; e += blockDim.x) {
-      const int r = s + 1 + e / w, c = s + 1 + e % w;
-      const double2 t = cmul2(D[r][s], D[s][c]);
-      D[r][c] = make_double2(D[r][c].x - t.x, D[r][c].y - t.y);
+      x[W - 1] = make_float2(0.f, 0.f);
     }
   }
+  if constexpr (J0 + 8 < kPB) select_stage<J0 + 8>(x, active, g, cnt, sm, sel);
+}
+
+__device__ __forceinline__ int select_rows(const double2* __restrict__ A, int ng, int k0, const int* gid, int nr,
+                                           int kb, float2 (*P)[kPB + 1], SelectSmem& sm, int* sel) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  // coalesced: a warp reads its 32 rows, one row a load
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    const int r = 32 * warp + i;
+    P[r][lane] = (r < nr && lane < kb) ? to_f2(A[(size_t)gid[r] * ng + k0 + lane]) : make_float2(0.f, 0.f);
+  }
+  __syncwarp();
+  float2 x[kPB];
+#pragma unroll
+  for (int c = 0; c < kPB; ++c) x[c] = P[t][c];
+  const int cnt = min(nr, kb);
+  select_stage<0>(x, t < nr, t < nr ? (unsigned)gid[t] : 0xffffffffu, cnt, sm, sel);
   __syncthreads();
-  for (int e = tid; e < kPB * kPB; e += blockDim.x) lu[e] = D[e / kPB][e % kPB];
-  for (int e = tid; e < kPB; e += blockDim.x) lu[kPB * kPB + e] = e < kb ? rinv[e] : make_double2(1.0, 0.0);
+  return cnt;
+}
+
+// The CTA that makes the final choice leaves the block D = A[sel][K] (the
+// chosen rows in selection order, identity outside kb) before the rows are
+// swapped; the swap launch factors it beside the swaps.
+__device__ __forceinline__ void stash_block(const double2* __restrict__ A, int ng, int k0, int kb, const int* sel,
+                                            double2* __restrict__ lu) {
+  for (int e = threadIdx.x; e < kPB * kPB; e += blockDim.x) {
+    const int r = e / kPB, c = e % kPB;
+    lu[e] = (r < kb && c < kb) ? A[(size_t)sel[r] * ng + k0 + c] : make_double2(r == c ? 1.0 : 0.0, 0.0);
+  }
+}
+
+// FP64 LU (without further pivoting) of the stashed block, 256 threads: lu
+// comes in as D[r][c] and goes out by columns, lu[c * NB + r] = L below the
+// diagonal (unit diagonal implied) and U on and above it, lu[NB*NB + s] =
+// 1/U_ss.  Lane = row, warp w holds columns w, w + 8, ... in registers; the
+// row of U comes by shuffle, the column of L through shared memory, written
+// for the next column by its warp ahead of that warp's other columns (one
+// barrier a column).  50 us, bounded by that chain (its FP64 operations queue
+// behind the other warps') and by the pipe (25 us with idle lanes); it runs
+// beside the swaps (about 10 us).
+__device__ void factor_block(double2* __restrict__ lu, int kb, double2 (*Lb)[kPB], int* __restrict__ status) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double2 x[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = lu[lane * kPB + warp + 8 * i];
+  auto scale = [&](double2& v, int s) {   // column s: reciprocal pivot, L below it
+    const double2 p = shfl2(v, s);
+    const double m2 = p.x * p.x + p.y * p.y;
+    const double q = rcp_f64_checked(m2, status);   // the same in every lane; 0 sets the status
+    const double2 ri = make_double2(p.x * q, -p.y * q);
+    if (lane > s) v = cmul2(v, ri);
+    Lb[s & 1][lane] = v;
+    if (lane == 0) lu[kPB * kPB + s] = ri;
+  };
+  __syncthreads();   // every element read before any is written back
+  if (warp == 0) scale(x[0], 0);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    for (int q = 0; q < 8; ++q) {
+      const int s = 8 * i + q;
+      if (s >= kb) break;
+      __syncthreads();
+      const double2 l = Lb[s & 1][lane];
+      auto upd = [&](double2& v) {
+        const double2 u = shfl2(v, s);
+        if (lane > s) v = csub2(v, l, u);
+      };
+      if (q < 7) {
+        if (warp == q + 1 && s + 1 < kb) {
+          upd(x[i]);
+          scale(x[i], s + 1);
+        } else if (warp > q) {
+          upd(x[i]);
+        }
+        if (i < 3) upd(x[i < 3 ? i + 1 : 3]);
+      } else if (i < 3) {
+        upd(x[i < 3 ? i + 1 : 3]);
+        if (warp == 0 && s + 1 < kb) scale(x[i < 3 ? i + 1 : 3], s + 1);
+      }
+#pragma unroll
+      for (int h = 2; h < 4; ++h)
+        if (i + h < 4) upd(x[i + h < 4 ? i + h : 3]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) lu[(warp + 8 * i) * kPB + lane] = x[i];
+  if (threadIdx.x >= kb && threadIdx.x < kPB) lu[kPB * kPB + threadIdx.x] = make_double2(1.0, 0.0);
 }
 
 // Row panel R = D^-1 A_K,: from the factors (after the swap, row k0 + r is
-// the r-th chosen row): each CTA solves L U x = b for 16 columns of A_K,:,
-// the block's own columns replaced by identity columns (R = D^-1 there).
-// blockIdx.y >= 1 copies the column panel Cp = A_:,K (ld NB).  256 threads:
-// 16 columns x 16 row groups (rows g, g + 16).
-__global__ void __launch_bounds__(256) solve_panels_kernel(const __grid_constant__ GenPtrs P, int ng, int k0,
-                                                           int kb, const double2* __restrict__ lu_all,
-                                                           double2* __restrict__ R_all, double2* __restrict__ C_all) {
+// the r-th chosen row): L U x = b for every column of A_K,:, the block's own
+// columns replaced by identity columns (R = D^-1 there).  CTAs after the
+// first ceil(ng / 16) copy the column panel Cp = A_:,K (ld NB).
+//
+// The FP64 pipe (two FMAs a clock and SM) bounds it: 4600 operations a column.
+// Four lanes hold a column, rows l, l + 4, ... in registers, so the chain needs
+// shuffles and no barrier, and the triangles leave few lanes idle.  A row takes
+// four solved rows at a time and rounds once for them: with one FMA after the
+// other on the row itself the step takes 88 us but the inverse's error is 6 %
+// larger than with a product rounded apart from the row, this way 5 % smaller.
+// Five matrices of N_G 2064: 106 us a step (82 us of FP64 operations alone),
+// CTAs of one warp for the last wave's sake (of two: 17 us more); 209 us with
+// 16 columns by 16 row groups, shared memory and three barriers a row pair.
+constexpr int kCopyRows = 32;
+constexpr int kSolveThreads = 32, kSolveCols = kSolveThreads / 4;
+
+__global__ void __launch_bounds__(kSolveThreads) solve_panels_kernel(const __grid_constant__ GenPtrs P, int ng,
+                                                                     int k0, int kb,
+                                                                     const double2* __restrict__ lu_all,
+                                                                     double2* __restrict__ R_all,
+                                                                     double2* __restrict__ C_all) {
   const int tid = threadIdx.x;
-  const int m = blockIdx.z;
+  const int m = blockIdx.y;
   const double2* __restrict__ A = P.A[m];
   const double2* __restrict__ lu = lu_all + (size_t)m * kPB * (kPB + 1);
   double2* __restrict__ R = R_all + (size_t)m * kPB * ng;
   double2* __restrict__ C = C_all + (size_t)m * kPB * ng;
-  if (blockIdx.y > 0) {
-    const int i = (blockIdx.y - 1) * 256 + tid;
-    if (blockIdx.x != 0 || i >= ng) return;
-    for (int s = 0; s < kb; ++s) C[(size_t)i * kPB + s] = A[(size_t)i * ng + k0 + s];
+  const int ncol = (ng + kSolveCols - 1) / kSolveCols;
+  if ((int)blockIdx.x >= ncol) {   // kCopyRows rows of the column panel
+    const int r0 = (blockIdx.x - ncol) * kCopyRows, s = tid & 31;
+#pragma unroll 8
+    for (int r = tid >> 5; r < kCopyRows; r += kSolveThreads / 32)
+      if (s < kb && r0 + r < ng) C[(size_t)(r0 + r) * kPB + s] = A[(size_t)(r0 + r) * ng + k0 + s];
     return;
   }
-  __shared__ double2 D[kPB][kPB + 1];
-  __shared__ double2 B[kPB][17];
+  __shared__ double2 D[kPB][kPB];   // by columns
   __shared__ double2 rinv[kPB];
-  const int j0 = blockIdx.x * 16;
-  for (int e = tid; e < kPB * kPB; e += 256) D[e / kPB][e % kPB] = lu[e];
-  if (tid < kPB) rinv[tid] = lu[kPB * kPB + tid];
-  for (int e = tid; e < kPB * 16; e += 256) {
-    const int r = e / 16, jj = e % 16, j = j0 + jj;
-    double2 v = make_double2(0.0, 0.0);
+  const int l = tid & 3;
+  const int j = blockIdx.x * kSolveCols + (tid >> 2);
+  double2 x[8];
+#pragma unroll
+  for (int h = 0; h < 8; ++h) {
+    const int r = l + 4 * h;
+    x[h] = make_double2(0.0, 0.0);
     if (r < kb && j < ng)
-      v = (j >= k0 && j < k0 + kb) ? make_double2(j - k0 == r ? 1.0 : 0.0, 0.0) : A[(size_t)(k0 + r) * ng + j];
-    B[r][jj] = v;
+      x[h] = (j >= k0 && j < k0 + kb) ? make_double2(j - k0 == r ? 1.0 : 0.0, 0.0) : A[(size_t)(k0 + r) * ng + j];
   }
-  const int col = tid & 15, g = tid >> 4;
-  for (int s = 0; s < kb; ++s) {   // unit lower factor
-    __syncthreads();
-    const double2 y = B[s][col];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = g + 16 * h;
-      if (r > s && r < kb) {
-        const double2 t = cmul2(D[r][s], y);
-        B[r][col] = make_double2(B[r][col].x - t.x, B[r][col].y - t.y);
-      }
-    }
-  }
-  for (int s = kb - 1; s >= 0; --s) {   // upper factor
-    __syncthreads();
-    if (g == (s & 15)) B[s][col] = cmul2(B[s][col], rinv[s]);
-    __syncthreads();
-    const double2 x = B[s][col];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = g + 16 * h;
-      if (r < s) {
-        const double2 t = cmul2(D[r][s], x);
-        B[r][col] = make_double2(B[r][col].x - t.x, B[r][col].y - t.y);
-      }
-    }
-  }
+#pragma unroll 8
+  for (int e = tid; e < kPB * kPB; e += kSolveThreads) (&D[0][0])[e] = lu[e];
+  if (tid < kPB) rinv[tid] = lu[kPB * kPB + tid];
   __syncthreads();
-  for (int e = tid; e < kPB * 16; e += 256) {
-    const int r = e / 16, jj = e % 16, j = j0 + jj;
-    if (r < kb && j < ng) R[(size_t)r * ng + j] = B[r][jj];
+  // rows 4 i + l take four solved rows 4 h .. 4 h + 3 at a time, their sum rounded to x once
+  auto rest = [&](double2& xi, int h, int i, const double2 (&y)[4]) {
+    double2 t = cmul2(D[4 * h][l + 4 * i], y[0]);
+#pragma unroll
+    for (int q = 1; q < 4; ++q) t = cfma2(D[4 * h + q][l + 4 * i], y[q], t);
+    xi = make_double2(xi.x - t.x, xi.y - t.y);
+  };
+  double2 y[4];
+#pragma unroll
+  for (int h = 0; h < 8; ++h) {   // unit lower factor
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      y[q] = shfl2(x[h], q, 4);
+      if (l > q) x[h] = csub2(x[h], D[4 * h + q][l + 4 * h], y[q]);
+    }
+#pragma unroll
+    for (int i = h + 1; i < 8; ++i) rest(x[i], h, i, y);
+  }
+#pragma unroll
+  for (int h = 7; h >= 0; --h) {   // upper factor
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+      if (l == q) x[h] = cmul2(x[h], rinv[4 * h + q]);
+      y[q] = shfl2(x[h], q, 4);
+      if (l < q) x[h] = csub2(x[h], D[4 * h + q][l + 4 * h], y[q]);
+    }
+#pragma unroll
+    for (int i = h - 1; i >= 0; --i) rest(x[i], h, i, y);
+  }
+#pragma unroll
+  for (int h = 0; h < 8; ++h) {
+    const int r = l + 4 * h;
+    if (r < kb && j < ng) R[(size_t)r * ng + j] = x[h];
   }
 }
 
 // Leaf round: CTA b takes rows k0 + 256 b ... of the panel.
 __global__ void __launch_bounds__(kTRows) pivot_leaf_kernel(const __grid_constant__ GenPtrs Pm, int ng, int k0,
                                                             int kb, int* __restrict__ out_all, int cstride,
-                                                            double2* __restrict__ lu_all, int* __restrict__ status) {
+                                                            double2* __restrict__ lu_all) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int m = blockIdx.y;
   const double2* __restrict__ A = Pm.A[m];
@@ -235,25 +330,23 @@ __global__ void __launch_bounds__(kTRows) pivot_leaf_kernel(const __grid_constan
   float2 (*P)[kPB + 1] = reinterpret_cast<float2 (*)[kPB + 1]>(smem_raw);
   __shared__ int gid[kTRows];
   __shared__ int sel[kPB];
+  __shared__ SelectSmem sm;
   const int r0 = k0 + blockIdx.x * kTRows;
   const int nr = min(kTRows, ng - r0);
   const int t = threadIdx.x;
   gid[t] = r0 + t;
-  if (t < nr)
-    for (int c = 0; c < kb; ++c) P[t][c] = to_f2(A[(size_t)(r0 + t) * ng + k0 + c]);
   __syncthreads();
-  const int n = select_rows(P, gid, nr, kb, sel);
-  __syncthreads();
+  const int n = select_rows(A, ng, k0, gid, nr, kb, P, sm, sel);
   if (t < n) out[blockIdx.x * kPB + t] = sel[t];
   if (t == 0) cnt[blockIdx.x] = n;
-  if (gridDim.x == 1) factor_block(A, ng, k0, kb, sel, smem_raw, lu, status);   // the final choice
+  if (gridDim.x == 1) stash_block(A, ng, k0, kb, sel, lu);   // the final choice
 }
 
 // Merge round: CTA m takes candidate sets 8m .. 8m+7 (of ngroups).
 __global__ void __launch_bounds__(kTRows) pivot_merge_kernel(const __grid_constant__ GenPtrs Pm, int ng, int k0,
                                                              int kb, const int* __restrict__ in_all,
                                                              int ngroups, int* __restrict__ out_all, int cstride,
-                                                             double2* __restrict__ lu_all, int* __restrict__ status) {
+                                                             double2* __restrict__ lu_all) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int m = blockIdx.y;
   const double2* __restrict__ A = Pm.A[m];
@@ -265,68 +358,83 @@ __global__ void __launch_bounds__(kTRows) pivot_merge_kernel(const __grid_consta
   float2 (*P)[kPB + 1] = reinterpret_cast<float2 (*)[kPB + 1]>(smem_raw);
   __shared__ int gid[kTRows];
   __shared__ int sel[kPB];
-  __shared__ int nr_s;
-  const int t = threadIdx.x;
-  if (t == 0) {
-    int n = 0;
-    for (int g = blockIdx.x * 8; g < min(ngroups, blockIdx.x * 8 + 8); ++g)
-      for (int i = 0; i < cin[g]; ++i) gid[n++] = in[g * kPB + i];
-    nr_s = n;
+  __shared__ SelectSmem sm;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int g0 = blockIdx.x * 8;
+  int before = 0, nr = 0, mine = 0;   // rows of the sets before this warp's, of all, of its own
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = g0 + i < ngroups ? cin[g0 + i] : 0;
+    if (i < warp) before += k;
+    if (i == warp) mine = k;
+    nr += k;
   }
+  if (lane < mine) gid[before + lane] = in[(g0 + warp) * kPB + lane];
   __syncthreads();
-  const int nr = nr_s;
-  if (t < nr)
-    for (int c = 0; c < kb; ++c) P[t][c] = to_f2(A[(size_t)gid[t] * ng + k0 + c]);
-  __syncthreads();
-  const int n = select_rows(P, gid, nr, kb, sel);
-  __syncthreads();
+  const int n = select_rows(A, ng, k0, gid, nr, kb, P, sm, sel);
   if (t < n) out[blockIdx.x * kPB + t] = sel[t];
   if (t == 0) cout[blockIdx.x] = n;
-  if (gridDim.x == 1) factor_block(A, ng, k0, kb, sel, smem_raw, lu, status);   // the final choice
+  if (gridDim.x == 1) stash_block(A, ng, k0, kb, sel, lu);   // the final choice
 }
 
 // Brings row sel[j] to row k0 + j for j < kb by successive interchanges
-// (recorded in ipiv[k0 + j]).  Every CTA replays the interchanges on the set
-// of affected rows (at most 64) and moves its 64 columns of them.
+// (recorded in ipiv[k0 + j]).  Every CTA but the last replays the
+// interchanges on the set of affected rows (at most 64; one warp, two slots a
+// lane) and moves its 64 columns of them.  The last CTA factors the stashed
+// block meanwhile.
 __global__ void __launch_bounds__(256) pivot_swap_kernel(const __grid_constant__ GenPtrs Pm, int ng, int k0, int kb,
                                                          const int* __restrict__ sel_all, int cstride,
-                                                         int* __restrict__ ipiv_all) {
+                                                         int* __restrict__ ipiv_all, double2* __restrict__ lu_all,
+                                                         int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int m = blockIdx.y;
+  if (blockIdx.x == gridDim.x - 1) {
+    factor_block(lu_all + (size_t)m * kPB * (kPB + 1), kb, reinterpret_cast<double2 (*)[kPB]>(smem_raw), status);
+    return;
+  }
   double2* __restrict__ A = Pm.A[m];
   const int* __restrict__ sel = sel_all + (size_t)m * cstride;
   int* __restrict__ ipiv = ipiv_all + (size_t)m * ng;
   double2 (*buf)[kSwapCols] = reinterpret_cast<double2 (*)[kSwapCols]>(smem_raw);
-  __shared__ int pos[2 * kPB];   // positions of the affected rows
+  __shared__ int pos[2 * kPB];   // positions of the affected rows (-1: none)
   __shared__ int from[2 * kPB];  // original row that ends at pos[i]
-  __shared__ int ns;
   const int t = threadIdx.x;
-  if (t == 0) {
-    int n = 0;
-    for (int j = 0; j < kb; ++j) pos[n++] = k0 + j;
-    for (int j = 0; j < kb; ++j)
-      if (sel[j] >= k0 + kb) pos[n++] = sel[j];
-    for (int i = 0; i < n; ++i) from[i] = pos[i];
+  if (t < 32) {
+    const int sj = t < kb ? sel[t] : -1;
+    const bool far = sj >= k0 + kb;   // a row outside the block's own
+    const unsigned fm = __ballot_sync(0xffffffffu, far);
+    pos[t] = t < kb ? k0 + t : -1;
+    pos[kPB + t] = -1;
+    __syncwarp();
+    if (far) pos[kPB + __popc(fm & ((1u << t) - 1))] = sj;
+    __syncwarp();
+    int f0 = pos[t], f1 = pos[kPB + t];
     for (int j = 0; j < kb; ++j) {
-      int cur = -1;   // slot currently holding original row sel[j]
-      for (int i = 0; i < n; ++i)
-        if (from[i] == sel[j]) cur = i;
-      const int tmp = from[j];
-      from[j] = from[cur];
-      from[cur] = tmp;
-      if (blockIdx.x == 0) ipiv[k0 + j] = pos[cur];
+      const int want = __shfl_sync(0xffffffffu, sj, j);
+      const int old = __shfl_sync(0xffffffffu, f0, j);
+      const unsigned b0 = __ballot_sync(0xffffffffu, f0 == want), b1 = __ballot_sync(0xffffffffu, f1 == want);
+      const int cur = b0 ? __ffs(b0) - 1 : kPB + __ffs(b1) - 1;   // slot holding original row sel[j]
+      if (t == j) f0 = want;
+      if (cur < kPB) {
+        if (t == cur) f0 = old;
+      } else if (t == cur - kPB) {
+        f1 = old;
+      }
+      if (blockIdx.x == 0 && t == 0) ipiv[k0 + j] = pos[cur];
     }
-    ns = n;
+    from[t] = f0;
+    from[kPB + t] = f1;
   }
   __syncthreads();
-  const int n = ns;
   const int c0 = blockIdx.x * kSwapCols;
-  for (int e = t; e < n * kSwapCols; e += 256) {
+#pragma unroll 8
+  for (int e = t; e < 2 * kPB * kSwapCols; e += 256) {
     const int i = e / kSwapCols, cc = e % kSwapCols;
     if (c0 + cc < ng && from[i] != pos[i]) buf[i][cc] = A[(size_t)from[i] * ng + c0 + cc];
   }
   __syncthreads();
-  for (int e = t; e < n * kSwapCols; e += 256) {
+#pragma unroll 8
+  for (int e = t; e < 2 * kPB * kSwapCols; e += 256) {
     const int i = e / kSwapCols, cc = e % kSwapCols;
     if (c0 + cc < ng && from[i] != pos[i]) A[(size_t)pos[i] * ng + c0 + cc] = buf[i][cc];
   }
@@ -334,17 +442,26 @@ __global__ void __launch_bounds__(256) pivot_swap_kernel(const __grid_constant__
 
 // Column j of the inverse is column src[j] of the working matrix: the
 // interchanges undone on the columns, last first.
-__global__ void colperm_build_kernel(const int* __restrict__ ipiv_all, int ng, int* __restrict__ src_all) {
-  if (threadIdx.x != 0) return;
-  const int* __restrict__ ipiv = ipiv_all + (size_t)blockIdx.x * ng;
-  int* __restrict__ src = src_all + (size_t)blockIdx.x * ng;
-  for (int j = 0; j < ng; ++j) src[j] = j;
-  for (int j = ng - 1; j >= 0; --j) {
-    const int p = ipiv[j];
-    const int tmp = src[j];
-    src[j] = src[p];
-    src[p] = tmp;
+// The chain of interchanges runs in shared memory.
+__global__ void __launch_bounds__(256) colperm_build_kernel(const int* __restrict__ ipiv_all, int ng,
+                                                            int* __restrict__ src_all) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int* src = reinterpret_cast<int*>(smem_raw);
+  int* ipiv = src + ng;
+  for (int j = threadIdx.x; j < ng; j += 256) {
+    src[j] = j;
+    ipiv[j] = ipiv_all[(size_t)blockIdx.x * ng + j];
   }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int j = ng - 1; j >= 0; --j) {
+      const int p = ipiv[j];
+      const int tmp = src[j];
+      src[j] = src[p];
+      src[p] = tmp;
+    }
+  __syncthreads();
+  for (int j = threadIdx.x; j < ng; j += 256) src_all[(size_t)blockIdx.x * ng + j] = src[j];
 }
 
 __global__ void __launch_bounds__(256) colperm_apply_kernel(const __grid_constant__ GenPtrs Pm, int ng,
@@ -382,6 +499,8 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
   BGW_CUDA(c, cudaFuncSetAttribute(pivot_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
   BGW_CUDA(c, cudaFuncSetAttribute(pivot_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
   BGW_CUDA(c, cudaFuncSetAttribute(pivot_swap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
+  BGW_CUDA(c, cudaFuncSetAttribute(colperm_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)(2 * sizeof(int) * ngmax)));
   BGW_CUDA(c, cudaFuncSetAttribute(colperm_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)(sizeof(double2) * ngmax)));
   int* cbuf[2] = {cand.as<int>(), cand.as<int>() + (size_t)kGB * cstride};
@@ -428,25 +547,25 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
       int cur = 0;
       {
         TimedScope tp(c, kTPivot, st);
-        pivot_leaf_kernel<<<dim3(groups, nb), kTRows, psmem, st>>>(P, n, k0, kb, cbuf[0], cstride, lu.as<double2>(),
-                                                                   c->d_status);
+        pivot_leaf_kernel<<<dim3(groups, nb), kTRows, psmem, st>>>(P, n, k0, kb, cbuf[0], cstride, lu.as<double2>());
         c->launches += 1;
         while (groups > 1) {
           const int next = (groups + 7) / 8;
           pivot_merge_kernel<<<dim3(next, nb), kTRows, psmem, st>>>(P, n, k0, kb, cbuf[cur], groups, cbuf[1 - cur],
-                                                                    cstride, lu.as<double2>(), c->d_status);
+                                                                    cstride, lu.as<double2>());
           c->launches += 1;
           cur = 1 - cur;
           groups = next;
         }
-        pivot_swap_kernel<<<dim3((n + kSwapCols - 1) / kSwapCols, nb), 256, ssmem, st>>>(P, n, k0, kb, cbuf[cur],
-                                                                                         cstride, piv);
+        pivot_swap_kernel<<<dim3((n + kSwapCols - 1) / kSwapCols + 1, nb), 256, ssmem, st>>>(
+            P, n, k0, kb, cbuf[cur], cstride, piv, lu.as<double2>(), c->d_status);
         c->launches += 1;
         BGW_CUDA(c, cudaGetLastError());
       }
       {
         TimedScope tg(c, kTSweepChain, st);
-        solve_panels_kernel<<<dim3((n + 15) / 16, 1 + (n + 255) / 256, nb), 256, 0, st>>>(
+        solve_panels_kernel<<<dim3((n + kSolveCols - 1) / kSolveCols + (n + kCopyRows - 1) / kCopyRows, nb),
+                              kSolveThreads, 0, st>>>(
             P, n, k0, kb, lu.as<double2>(), R.as<double2>(), Cp.as<double2>());
         c->launches += 1;
         BGW_CUDA(c, cudaGetLastError());
@@ -463,7 +582,7 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
         c->launches += 3;
       }
     }
-    colperm_build_kernel<<<nb, 1, 0, st>>>(piv, n, src);
+    colperm_build_kernel<<<nb, 256, 2 * sizeof(int) * n, st>>>(piv, n, src);
     colperm_apply_kernel<<<dim3(n, nb), 256, sizeof(double2) * n, st>>>(P, n, src);
     BGW_CUDA(c, cudaGetLastError());
     c->launches += 2;

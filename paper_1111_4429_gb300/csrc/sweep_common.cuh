@@ -193,6 +193,22 @@ __device__ __forceinline__ float2 ff_rcp(float2 d) {
   return ff_fast(r0, __fmul_rn(r0, err));
 }
 
+// 1 / d for a pivot d > 0 (else 0 and *status): the double-FP32 reciprocal
+// (2^-46) and one Newton step with a fused residual, two FP64 operations
+// instead of a division's chain of them, each of which would queue behind the
+// update's at the FP64 pipe.
+__device__ __forceinline__ double rcp_f64_checked(double d, int* status) {
+  if (!(d > 0.0) || !isfinite(d)) {
+    atomicExch(status, (int)kDevZeroPivot);
+    return 0.0;
+  }
+  const int ex = (int)((unsigned)__double2hiint(d) >> 20) - 1023;
+  if (ex < -60 || ex > 60) return rcp_slow(d);   // outside double FP32's safe range
+  const float2 r = ff_rcp(ff_from_int(d));
+  const double r0 = ff_to_any(r.x, r.y);
+  return fma(r0, fma(-d, r0, 1.0), r0);
+}
+
 // v + a1 b1 + a2 b2 with both products as exact pairs and the high words
 // two-summed; the result is left unnormalized (hi, lo): lo gathers the
 // error terms, so hi + lo carries the sum to about 2^-43 of the largest
@@ -240,20 +256,7 @@ __device__ __forceinline__ void diag_sweep_f64(DiagSmem& sm, int kb, int t, int*
   int x, y;
   bool low;
   diag_thread_element(t, kb - 1, x, y, low);
-  // 1 / d: the double-FP32 reciprocal (2^-46) and one Newton step with a fused
-  // residual, two FP64 operations instead of a division's chain of them, each
-  // of which would queue behind the update's at the FP64 pipe
-  auto rcp_checked = [&](double d) {
-    if (!(d > 0.0) || !isfinite(d)) {
-      atomicExch(status, (int)kDevZeroPivot);
-      return 0.0;
-    }
-    const int ex = (int)((unsigned)__double2hiint(d) >> 20) - 1023;
-    if (ex < -60 || ex > 60) return rcp_slow(d);   // outside double FP32's safe range
-    const float2 r = ff_rcp(ff_from_int(d));
-    const double r0 = ff_to_any(r.x, r.y);
-    return fma(r0, fma(-d, r0, 1.0), r0);
-  };
+  auto rcp_checked = [&](double d) { return rcp_f64_checked(d, status); };
   __syncthreads();
   if (head && lane == 0) sm.rpiv = rcp_checked(sm.L[0][0].x);
   for (int s = 0; s < kb; ++s) {
