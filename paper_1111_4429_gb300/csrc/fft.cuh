@@ -15,6 +15,11 @@
 // Twiddles e^{2 pi i t/N} come from a table of cos/sin values filled by the
 // host in extended precision (upload_twiddles); inside a stage the table
 // index is a compile-time constant, so the loads are constant-bank operands.
+//
+// FP32 forms both parts of a complex number with packed instructions
+// (fma.rn.f32x2 and the like: the same roundings, half the instructions):
+// sums and differences always, rotations and twiddles, whose swapped operands
+// can cost moves, where it measured faster (pack_all).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -29,6 +34,10 @@ template <typename T> using cpx = typename cpx_t<T>::type;
 template <typename T> __device__ __forceinline__ cpx<T> mk(T x, T y) { cpx<T> r; r.x = x; r.y = y; return r; }
 template <typename T> __device__ __forceinline__ cpx<T> add(cpx<T> a, cpx<T> b) { return mk<T>(a.x + b.x, a.y + b.y); }
 template <typename T> __device__ __forceinline__ cpx<T> sub(cpx<T> a, cpx<T> b) { return mk<T>(a.x - b.x, a.y - b.y); }
+template <> __device__ __forceinline__ float2 add<float>(float2 a, float2 b) { return __fadd2_rn(a, b); }
+template <> __device__ __forceinline__ float2 sub<float>(float2 a, float2 b) {
+  return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+}
 template <typename T> __device__ __forceinline__ cpx<T> mul(cpx<T> a, cpx<T> b) {
   return mk<T>(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
@@ -37,9 +46,32 @@ template <typename T> __device__ __forceinline__ cpx<T> cmulc(cpx<T> a, cpx<T> b
   return mk<T>(fma(a.x, b.x, a.y * b.y), fma(a.x, b.y, -a.y * b.x));
 }
 template <typename T> __device__ __forceinline__ cpx<T> scale(cpx<T> a, T s) { return mk<T>(a.x * s, a.y * s); }
+template <> __device__ __forceinline__ float2 scale<float>(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }
 // i^S * a  for S = +-1
 template <typename T, int S> __device__ __forceinline__ cpx<T> mul_i(cpx<T> a) {
   return S > 0 ? mk<T>(-a.y, a.x) : mk<T>(a.y, -a.x);
+}
+
+// Whether an FP32 line of length n packs its rotations and twiddles too: all but
+// 32 and its quarters.  Pair y,x pass and z pass in us a pair, all scalar / sums
+// packed / all packed: 32^3 (N_G 2120) 0.0589, 0.0138 / 0.0530, 0.0112 / 0.0554,
+// 0.0117; 48^3 (7180) 0.2193, 0.0414 / 0.2123, 0.0376 / 0.2071, 0.0371; 40^3 (3911)
+// 0.1294, 0.0282 / 0.1314, 0.0292 / 0.1268, 0.0273; 64^3 (8765) 0.483, 0.0645 /
+// 0.478, 0.0745 / 0.480, 0.0553.  The passes wait for loads more than for issue
+// slots (48^3: 0.71 of the instructions, 0.94 of the time).
+__host__ __device__ constexpr bool pack_all(int n) { return !(n == 8 || n == 32); }
+
+// Packed forms, FP32: a + i S b, s a + b for a real s, and a b
+template <int S> __device__ __forceinline__ float2 pk_add_i(float2 a, float2 b) {
+  return __ffma2_rn(make_float2(b.y, b.x), make_float2(S > 0 ? -1.f : 1.f, S > 0 ? 1.f : -1.f), a);
+}
+__device__ __forceinline__ float2 pk_fma(float s, float2 a, float2 b) { return __ffma2_rn(a, make_float2(s, s), b); }
+__device__ __forceinline__ float2 pk_mul(float2 a, float2 b) {
+  return __ffma2_rn(a, make_float2(b.x, b.x), __fmul2_rn(make_float2(a.y, a.x), make_float2(-b.y, b.y)));
+}
+template <typename T, bool PK> __device__ __forceinline__ cpx<T> mul_tw(cpx<T> a, cpx<T> b) {
+  if constexpr (PK) return pk_mul(a, b);
+  else return mul<T>(a, b);
 }
 
 // Supported line lengths and their offsets in the twiddle table.
@@ -67,11 +99,38 @@ __host__ __device__ constexpr int first_radix(int n) {
 #define BGW_S51 0.95105651629515357212
 #define BGW_S52 0.58778525229247312917
 
-template <typename T, int R, int S>
+template <typename T, int R, int S, bool PK>
 __device__ __forceinline__ void dft_small(const cpx<T> (&a)[R], cpx<T> (&b)[R]) {
   if constexpr (R == 2) {
     b[0] = add<T>(a[0], a[1]);
     b[1] = sub<T>(a[0], a[1]);
+  } else if constexpr (R == 4 && PK) {
+    const float2 s02 = add<T>(a[0], a[2]), d02 = sub<T>(a[0], a[2]);
+    const float2 s13 = add<T>(a[1], a[3]), d13 = sub<T>(a[1], a[3]);
+    b[0] = add<T>(s02, s13);
+    b[2] = sub<T>(s02, s13);
+    b[1] = pk_add_i<S>(d02, d13);
+    b[3] = pk_add_i<-S>(d02, d13);
+  } else if constexpr (R == 3 && sizeof(T) == 4) {
+    const float s = float(S) * float(BGW_S3);
+    const float2 sum = add<T>(a[1], a[2]), dif = sub<T>(a[1], a[2]);
+    const float2 t = pk_fma(-0.5f, sum, a[0]);
+    b[0] = add<T>(a[0], sum);
+    const float2 rot = make_float2(dif.y, dif.x);
+    b[1] = __ffma2_rn(rot, make_float2(-s, s), t);   // t +- i s (a1 - a2)
+    b[2] = __ffma2_rn(rot, make_float2(s, -s), t);
+  } else if constexpr (R == 5 && PK) {
+    const T c1 = T(BGW_C51), c2 = T(BGW_C52);
+    const T s1 = T(S) * T(BGW_S51), s2 = T(S) * T(BGW_S52);
+    const float2 p14 = add<T>(a[1], a[4]), m14 = sub<T>(a[1], a[4]);
+    const float2 p23 = add<T>(a[2], a[3]), m23 = sub<T>(a[2], a[3]);
+    b[0] = add<T>(a[0], add<T>(p14, p23));
+    const float2 t1 = pk_fma(c1, p14, pk_fma(c2, p23, a[0])), t2 = pk_fma(c2, p14, pk_fma(c1, p23, a[0]));
+    const float2 u1 = pk_fma(s1, m14, scale<T>(m23, s2)), u2 = pk_fma(s2, m14, scale<T>(m23, -s1));
+    b[1] = pk_add_i<1>(t1, u1);
+    b[4] = pk_add_i<-1>(t1, u1);
+    b[2] = pk_add_i<1>(t2, u2);
+    b[3] = pk_add_i<-1>(t2, u2);
   } else if constexpr (R == 4) {
     cpx<T> s02 = add<T>(a[0], a[2]), d02 = sub<T>(a[0], a[2]);
     cpx<T> s13 = add<T>(a[1], a[3]), d13 = mul_i<T, S>(sub<T>(a[1], a[3]));
@@ -129,6 +188,7 @@ template <typename T, int N, int n, int st, int S>
 __device__ __forceinline__ void fft_stage(cpx<T> (&x)[N], cpx<T> (&y)[N]) {
   constexpr int r = first_radix(n);
   constexpr int m = n / r;
+  constexpr bool PK = sizeof(T) == 4 && pack_all(N);
 #pragma unroll
   for (int p = 0; p < m; ++p) {
 #pragma unroll
@@ -136,7 +196,7 @@ __device__ __forceinline__ void fft_stage(cpx<T> (&x)[N], cpx<T> (&y)[N]) {
       cpx<T> a[r], b[r];
 #pragma unroll
       for (int j = 0; j < r; ++j) a[j] = x[q + st * (p + j * m)];
-      dft_small<T, r, S>(a, b);
+      dft_small<T, r, S, PK>(a, b);
       y[q + st * (r * p)] = b[0];
 #pragma unroll
       for (int k = 1; k < r; ++k) {
@@ -145,7 +205,7 @@ __device__ __forceinline__ void fft_stage(cpx<T> (&x)[N], cpx<T> (&y)[N]) {
         } else if (p == 0) {
           y[q + st * (r * p + k)] = b[k];
         } else {
-          y[q + st * (r * p + k)] = mul<T>(b[k], twiddle<T, N, S>((p * k * (N / n)) % N));
+          y[q + st * (r * p + k)] = mul_tw<T, PK>(b[k], twiddle<T, N, S>((p * k * (N / n)) % N));
         }
       }
     }
@@ -180,6 +240,7 @@ __device__ __forceinline__ void fft_line(cpx<T> (&a)[N]) {
 template <typename T, int N, typename Load>
 __device__ __forceinline__ void fft_quarters(Load load, cpx<T> (&lo)[N / 4], cpx<T> (&hi)[N / 4]) {
   constexpr int M = N / 4;
+  constexpr bool PK = sizeof(T) == 4 && pack_all(N);
   static_assert(N % 4 == 0, "fft_quarters needs N divisible by 4");
 #pragma unroll
   for (int n1 = 0; n1 < 4; ++n1) {
@@ -189,14 +250,17 @@ __device__ __forceinline__ void fft_quarters(Load load, cpx<T> (&lo)[N / 4], cpx
     fft_line<T, M, 1>(y);
 #pragma unroll
     for (int k2 = 0; k2 < M; ++k2) {
-      const cpx<T> t = (n1 == 0 || k2 == 0) ? y[k2] : mul<T>(y[k2], twiddle<T, N, 1>(n1 * k2));
-      const cpx<T> u = n1 == 0 ? t : n1 == 1 ? mk<T>(t.y, -t.x) : n1 == 2 ? mk<T>(-t.x, -t.y) : mk<T>(-t.y, t.x);
+      const cpx<T> t = (n1 == 0 || k2 == 0) ? y[k2] : mul_tw<T, PK>(y[k2], twiddle<T, N, 1>(n1 * k2));
       if (n1 == 0) {
         lo[k2] = t;
-        hi[k2] = u;
+        hi[k2] = t;
+        continue;
+      }
+      lo[k2] = add<T>(lo[k2], t);
+      if constexpr (PK) {
+        hi[k2] = n1 == 1 ? pk_add_i<-1>(hi[k2], t) : n1 == 2 ? sub<T>(hi[k2], t) : pk_add_i<1>(hi[k2], t);
       } else {
-        lo[k2] = add<T>(lo[k2], t);
-        hi[k2] = add<T>(hi[k2], u);
+        hi[k2] = add<T>(hi[k2], n1 == 1 ? mk<T>(t.y, -t.x) : n1 == 2 ? mk<T>(-t.x, -t.y) : mk<T>(-t.y, t.x));
       }
     }
   }
