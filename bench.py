@@ -192,7 +192,9 @@ def mtxel_flops(s):
     pruned product transform, 5 n log2 n per 1D line over n^2 + (2 g_x + 1) n
     + (2 g_x + 1)(2 g_y + 1) lines (g_x, g_y: the epsilon sphere's largest
     |G_x|, |G_y|), plus 6 n^3 for the product; per band the band transform,
-    counted as three full passes of n^2 lines (an upper bound)."""
+    counted as three full passes of n^2 lines (an upper bound).  n is the
+    caller's grid: the transform runs on the smallest grid that gives the same
+    coefficients, so the flops issued are fewer."""
     n = s.fft
     gx, gy = int(np.abs(s.geps[:, 0]).max()), int(np.abs(s.geps[:, 1]).max())
     line = 5.0 * n * math.log2(n)
@@ -356,7 +358,8 @@ def _roofline(s, kt, step_ms, peaks, peak_src, size_tag="c2"):
                 "achieved": fl["mtxel"] / (sum(kt[k][1] for k in ("pair_yxpass", "pair_zgather", "band_transform")
                                                if k in kt) / 1e3) / 1e12,
                 "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "algorithmic": "pruned FFT flops of all matrix-element passes per step (5 n log2 n per line)",
+                "algorithmic": "pruned FFT flops of all matrix-element passes per step on the caller's grid "
+                               "(5 n log2 n per line; the transform runs on a smaller alias-free one)",
                 "peak_source": "derived: 152 SM x 128 FP32 lanes x 2 x 2.07 GHz",
                 "launch_ms": t_launch * 1e3, "traffic_tag": dom}
     elif dom == "chi_f64":

@@ -219,7 +219,8 @@ int bgw_graph_stats(bgw_ctx* ctx, uint64_t* graphs, uint64_t* replays);
  *    of 2 tiles.  Every tile's arithmetic is the same: the results are
  *    bit-identical, only the speed changes.                                */
 /*  BGW_OPT_WAIT_LIMIT_NS: how long (nanoseconds, 0 .. 10^10; default 10^9)
- *    a wait of the tensor-core chi kernels on its pipeline (a copy landing,
+ *    a wait of the tensor-core chi kernels (mixed precision and FP64) on its
+ *    pipeline (a copy landing,
  *    an MMA stage finishing, tensor memory being drained) may last before
  *    the kernel gives up: it then lets its copies and MMAs in flight finish
  *    (within 1 s), frees its tensor memory, returns, and the next bgw_sync

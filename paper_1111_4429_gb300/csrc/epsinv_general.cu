@@ -240,7 +240,8 @@ __device__ void factor_block(double2* __restrict__ lu, int kb, double2 (*Lb)[kPB
 // four solved rows at a time and rounds once for them: with one FMA after the
 // other on the row itself the step takes 88 us but the inverse's error is 6 %
 // larger than with a product rounded apart from the row, this way 5 % smaller.
-// Five matrices of N_G 2064: 106 us a step (82 us of FP64 operations alone),
+// Five matrices of N_G 1643: 106 us a step (the FP64 pipe 88 % busy, 60 us of it
+// the operations without the idle lanes and the last wave),
 // CTAs of one warp for the last wave's sake (of two: 17 us more); 209 us with
 // 16 columns by 16 row groups, shared memory and three barriers a row pair.
 constexpr int kCopyRows = 32;
