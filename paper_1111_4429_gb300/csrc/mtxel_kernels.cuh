@@ -272,6 +272,87 @@ __global__ void __launch_bounds__(32 * kPairWarps, sizeof(T) == 4 ? 4 : 2)
   for (int c = lane; c < ncol; c += 32) Tp[c] = Yw[c];
 }
 
+// Line lengths whose columns leave lanes of the y pass idle that a second pair
+// can use: two pairs' 2 N columns take fewer rounds of 32 lanes than N twice.
+__host__ __device__ constexpr bool two_pairs(int n) { return n > 32 && n <= 48; }
+
+// The same with two consecutive pairs a warp, three rounds of the y pass for
+// four (N = 36, 40, 48): the first pair's columns 0 .. 31; its others and the
+// second pair's first HB columns; the second pair's others.  After the second
+// round the first pair's x pass runs and its rows are free for the third.
+// grid (ceil(npb / (2 kPairWarps)), N), block 32 kPairWarps.
+// smem: (Y[nys][N+1] | B[nys][HB+1])[kPairWarps] | colmap[N*nys] | yslot[N].
+// Waits for the band planes bound both forms, a round's worth each.  48^3, N_G
+// 7180, FP32: 0.207 -> 0.184 us a pair; 40^3, 3911: 0.132 -> 0.118; FP64 (pipe
+// bound) 48^3: 7.59 -> 6.38.
+template <typename T, int N>
+__global__ void __launch_bounds__(32 * kPairWarps, sizeof(T) == 4 ? 4 : 2)
+    pair_yxpass_warp2(const cpx<T>* __restrict__ uv, const cpx<T>* __restrict__ uc, int nc, int pbase, int npb,
+                      int nys, int ncol, const int* __restrict__ g_colmap, const int* __restrict__ g_yslot,
+                      cpx<T>* __restrict__ Tbuf) {
+  static_assert(two_pairs(N), "three rounds hold two pairs' columns");
+  constexpr int LD = N + 1, Q = N / 4, HB = 64 - N, LB = HB + 1;   // HB + (N - 32) lanes in the second round
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cpx<T>* Y = reinterpret_cast<cpx<T>*>(smem_raw);
+  int* colmap = reinterpret_cast<int*>(Y + (size_t)kPairWarps * nys * (LD + LB));
+  int* yslot = colmap + N * nys;
+  const int z = blockIdx.y, tid = threadIdx.x;
+  for (int i = tid; i < N * nys; i += blockDim.x) colmap[i] = g_colmap[i];
+  for (int i = tid; i < N; i += blockDim.x) yslot[i] = g_yslot[i];
+  __syncthreads();
+  const int warp = tid >> 5, lane = tid & 31;
+  const int pl0 = 2 * (blockIdx.x * kPairWarps + warp);
+  if (pl0 >= npb) return;
+  const bool second = pl0 + 1 < npb;
+  const size_t plane = (size_t)N * N;
+  cpx<T>* Ya = Y + (size_t)warp * nys * (LD + LB);
+  cpx<T>* Yb = Ya + (size_t)nys * LD;
+#pragma unroll 1
+  for (int r = 0; r < 3; ++r) {
+    const int k = r == 2 || (r == 1 && lane >= N - 32);   // the lane's pair and column
+    const int x = r == 0 ? lane : r == 2 ? HB + lane : k ? lane - (N - 32) : 32 + lane;
+    if (x < N && (k == 0 || second)) {
+      const int p = pbase + pl0 + k, v = p / nc, c = p - v * nc;
+      const cpx<T>* pv = uv + ((size_t)v * N + z) * plane + x;
+      const cpx<T>* pc = uc + ((size_t)c * N + z) * plane + x;
+      cpx<T> lo[Q], hi[Q];
+      fft_quarters<T, N>([&](int y) { return cmulc<T>(pv[(size_t)y * N], pc[(size_t)y * N]); }, lo, hi);
+      cpx<T>* dst = k && r == 1 ? Yb + x : Ya + x;
+      const int ld = k && r == 1 ? LB : LD;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int s0 = yslot[q], s3 = yslot[q + 3 * Q];
+        if (s0 >= 0) dst[s0 * ld] = lo[q];
+        if (s3 >= 0) dst[s3 * ld] = hi[q];
+      }
+    }
+    if (r == 0) continue;
+    if (r == 2 && !second) break;
+    __syncwarp();
+    // x pass of pair r - 1, as above
+    const int pl = pl0 + r - 1, s = lane;
+    cpx<T>* Tp = Tbuf + ((size_t)pl * N + z) * ncol;
+    cpx<T> lo[Q], hi[Q];
+    if (s < nys) {
+      const cpx<T>* row = Ya + (size_t)s * LD;
+      const cpx<T>* head = r == 2 ? Yb + (size_t)s * LB : row;   // columns below HB
+      fft_quarters<T, N>([&](int xx) { return xx < HB ? head[xx] : row[xx]; }, lo, hi);
+    }
+    __syncwarp();
+    if (s < nys) {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int c0 = colmap[q * nys + s], c3 = colmap[(q + 3 * Q) * nys + s];
+        if (c0 >= 0) Ya[c0] = lo[q];
+        if (c3 >= 0) Ya[c3] = hi[q];
+      }
+    }
+    __syncwarp();
+    for (int c = lane; c < ncol; c += 32) Tp[c] = Ya[c];
+    __syncwarp();
+  }
+}
+
 // ---------------------------------------------------------------- pair z
 // grid (npb), block 256.  smem Mrow[ng], or none with direct != 0 (a list
 // too long for shared memory: the outputs go straight to M, complex only).
@@ -336,6 +417,38 @@ static void pair_block_shape(int ppb, int nys, int ncol, int* threads, size_t* s
   *threads = t > 256 ? 256 : t;
 }
 
+// Launch of the warp-per-pair form, with two pairs a warp where that saves a
+// round and a launch with one pair a warp would fill the SMs often enough: in
+// FP32 16 times (48^3: 400 pairs, 8 times, 106 against 108 us with two; 640, 13
+// times, 162 against 166; 800, 16 times, 191 against 188; 17,280 pairs 0.89 of the
+// time), as three rounds and two x passes make a longer last turn; in FP64, with half the warps resident and the
+// pipe busy in every turn, 8 (208 pairs: 1623 against 1450 us).
+template <typename T, int N>
+static cudaError_t launch_warp(const MtxelExec& x, const cpx<T>* uv, const cpx<T>* uc, int pbase, int npb,
+                               cpx<T>* Tb) {
+  const PairPlan* pp = x.pp;
+  const size_t maps = (size_t)(N * pp->nys + N) * sizeof(int);
+  cudaError_t e;
+  if constexpr (two_pairs(N)) {
+    constexpr long long warps = sizeof(T) == 4 ? 16 * 16 : 8 * 8;   // an SM's, over its turns
+    if ((long long)npb * N >= warps * sm_count(x.ctx)) {
+      const size_t sm = (size_t)kPairWarps * pp->nys * (N + 1 + 64 - N + 1) * sizeof(cpx<T>) + maps;
+      if (sm <= 200 * 1024) {
+        if ((e = set_smem(pair_yxpass_warp2<T, N>, sm)) != cudaSuccess) return e;
+        const int per = 2 * kPairWarps;
+        pair_yxpass_warp2<T, N><<<dim3((npb + per - 1) / per, N), 32 * kPairWarps, sm, x.st>>>(
+            uv, uc, x.nc, pbase, npb, pp->nys, pp->ncol, pp->d_colmap, pp->d_yslot_of_k, Tb);
+        return cudaGetLastError();
+      }
+    }
+  }
+  const size_t sm = (size_t)kPairWarps * pp->nys * (N + 1) * sizeof(cpx<T>) + maps;
+  if ((e = set_smem(pair_yxpass_warp<T, N>, sm)) != cudaSuccess) return e;
+  pair_yxpass_warp<T, N><<<dim3((npb + kPairWarps - 1) / kPairWarps, N), 32 * kPairWarps, sm, x.st>>>(
+      uv, uc, x.nc, pbase, npb, pp->nys, pp->ncol, pp->d_colmap, pp->d_yslot_of_k, Tb);
+  return cudaGetLastError();
+}
+
 // Autotuner of the pairs per pair_yxpass block: each candidate runs twice on
 // the first pairs of the call (the second run is timed with CUDA events on
 // the call's stream) and the fastest is kept for this (grid, precision,
@@ -382,21 +495,17 @@ static int tune_pairs_per_block(const MtxelExec& x, const cpx<T>* uv, const cpx<
   if constexpr (LB) {   // the warp-per-pair kernel as one more candidate
     const size_t sm = (size_t)kPairWarps * pp->nys * (N + 1) * sizeof(cpx<T>) + (size_t)(N * pp->nys + N) * sizeof(int);
     float ms = 0.f;
-    if (sm <= 200 * 1024 && set_smem(pair_yxpass_warp<T, N>, sm) == cudaSuccess) {
-      for (int rep = 0; rep < 2; ++rep) {
-        cudaEventRecord(e0, x.st);
-        pair_yxpass_warp<T, N><<<dim3((npb + kPairWarps - 1) / kPairWarps, N), 32 * kPairWarps, sm, x.st>>>(
-            uv, uc, x.nc, 0, npb, pp->nys, pp->ncol, pp->d_colmap, pp->d_yslot_of_k, Tb);
-        cudaEventRecord(e1, x.st);
-      }
-      if (cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) {
-        *x.launches += 2;
-        if (ms < best_ms) {
-          best_ms = ms;
-          best = kWarpPerPair;
-        }
-      } else {
-        cudaGetLastError();
+    bool ok = sm <= 200 * 1024;
+    for (int rep = 0; rep < 2 && ok; ++rep) {
+      cudaEventRecord(e0, x.st);
+      ok = launch_warp<T, N>(x, uv, uc, 0, npb, Tb) == cudaSuccess;
+      cudaEventRecord(e1, x.st);
+    }
+    if (ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) {
+      *x.launches += 2;
+      if (ms < best_ms) {
+        best_ms = ms;
+        best = kWarpPerPair;
       }
     } else {
       cudaGetLastError();
@@ -447,14 +556,8 @@ static cudaError_t mtxel_exec_lb(const MtxelExec& x) {
   // choice) falls back to the block kernel with the default pairs per block
   const bool warp_kernel = LB && ppb == kWarpPerPair;
   if (ppb >= kWarpPerPair && !warp_kernel) ppb = 256 / N > 0 ? 256 / N : 1;
-  int threads = 32 * kPairWarps;
+  int threads = 0;
   size_t sm = 0;
-  if constexpr (LB) {
-    if (warp_kernel) {
-      sm = (size_t)kPairWarps * pp->nys * (N + 1) * sizeof(C) + (size_t)(N * pp->nys + N) * sizeof(int);
-      if ((e = set_smem(pair_yxpass_warp<T, N>, sm)) != cudaSuccess) return e;
-    }
-  }
   if (!warp_kernel) {
     pair_block_shape<T, N>(ppb, pp->nys, pp->ncol, &threads, &sm);
     if ((e = set_smem(pair_yxpass<T, N, LB>, sm)) != cudaSuccess) return e;
@@ -469,9 +572,7 @@ static cudaError_t mtxel_exec_lb(const MtxelExec& x) {
     {
       TimedScope ts(x.ctx, kTPairYX, x.st);
       if constexpr (LB) {
-        if (warp_kernel)
-          pair_yxpass_warp<T, N><<<dim3((npb + kPairWarps - 1) / kPairWarps, N), threads, sm, x.st>>>(
-              uv, uc, x.nc, (int)p0, npb, pp->nys, pp->ncol, pp->d_colmap, pp->d_yslot_of_k, Tb);
+        if (warp_kernel && (e = launch_warp<T, N>(x, uv, uc, (int)p0, npb, Tb)) != cudaSuccess) return e;
       }
       if (!warp_kernel)
         pair_yxpass<T, N, LB><<<dim3((npb + ppb - 1) / ppb, N), threads, sm, x.st>>>(
