@@ -993,12 +993,23 @@ int oz_update(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, int mode, cudaSt
   const int nsm = sm_count(c);
   int wide = plan->slices < 7 ? 3 : kJPI;
   {
-    const int nI = (ngmax + BM - 1) / BM, nJ = (ngmax + BN - 1) / BN, k1 = k0 + NB;
-    grid = pipe_items(mode, wide, nI, nJ, k1 / BM, k1 < ngmax);
+    // the most items of a matrix that has not finished: a smaller one at its
+    // last step has items (no next row tile to leave out) where the largest
+    // may have none
+    auto most_items = [&](int w) {
+      int n = 0;
+      for (int m = 0; m < plan->nmat; ++m) {
+        const int ng = plan->batch.m[m].ng, k1 = k0 + NB;
+        if (k0 < ng && (mode != 1 || k1 < ng))
+          n = std::max(n, pipe_items(mode, w, (ng + BM - 1) / BM, (ng + BN - 1) / BN, k1 / BM, k1 < ng));
+      }
+      return n;
+    };
+    grid = most_items(wide);
     const bool narrow = plan->bulk_narrow >= 0 ? plan->bulk_narrow == 1 : (long long)grid * plan->nmat <= nsm;
     if (mode != 1 && narrow) {
       wide = 2;
-      grid = pipe_items(mode, wide, nI, nJ, k1 / BM, k1 < ngmax);
+      grid = most_items(wide);
     }
   }
   if (grid <= 0) return BGW_OK;
