@@ -53,6 +53,15 @@ __device__ __forceinline__ double2 cmul2(double2 a, double2 b) {
   return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
 
+// z - a b, four FP64 FMAs
+__device__ __forceinline__ double2 cfnma2(double2 a, double2 b, double2 z) {
+  z.x = fma(-a.x, b.x, z.x);
+  z.y = fma(-a.x, b.y, z.y);
+  z.x = fma(a.y, b.y, z.x);
+  z.y = fma(-a.y, b.x, z.y);
+  return z;
+}
+
 // z - a b with one rounding of z
 __device__ __forceinline__ double2 csub2(double2 z, double2 a, double2 b) {
   const double2 t = cmul2(a, b);
@@ -177,9 +186,11 @@ __device__ __forceinline__ void stash_block(const double2* __restrict__ A, int n
 // 1/U_ss.  Lane = row, warp w holds columns w, w + 8, ... in registers; the
 // row of U comes by shuffle, the column of L through shared memory, written
 // for the next column by its warp ahead of that warp's other columns (one
-// barrier a column).  50 us, bounded by that chain (its FP64 operations queue
-// behind the other warps') and by the pipe (25 us with idle lanes); it runs
-// beside the swaps (about 10 us).
+// barrier a column).  41 us, bounded by that chain (its FP64 operations queue
+// behind the other warps') and by the pipe (17 us with idle lanes); it runs
+// beside the swaps (about 10 us).  With each product rounded apart from its
+// element, 50 us; the inverse's error is below the older kernels' either way
+// (by 2 to 30 % at N_G 37 to 900).
 __device__ void factor_block(double2* __restrict__ lu, int kb, double2 (*Lb)[kPB], int* __restrict__ status) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double2 x[4];
@@ -205,7 +216,7 @@ __device__ void factor_block(double2* __restrict__ lu, int kb, double2 (*Lb)[kPB
       const double2 l = Lb[s & 1][lane];
       auto upd = [&](double2& v) {
         const double2 u = shfl2(v, s);
-        if (lane > s) v = csub2(v, l, u);
+        if (lane > s) v = cfnma2(l, u, v);
       };
       if (q < 7) {
         if (warp == q + 1 && s + 1 < kb) {
@@ -292,6 +303,7 @@ __global__ void __launch_bounds__(kSolveThreads) solve_panels_kernel(const __gri
   double2 y[4];
 #pragma unroll
   for (int h = 0; h < 8; ++h) {   // unit lower factor
+    if (4 * h >= kb) break;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       y[q] = shfl2(x[h], q, 4);
@@ -302,6 +314,7 @@ __global__ void __launch_bounds__(kSolveThreads) solve_panels_kernel(const __gri
   }
 #pragma unroll
   for (int h = 7; h >= 0; --h) {   // upper factor
+    if (4 * h >= kb) continue;
 #pragma unroll
     for (int q = 3; q >= 0; --q) {
       if (l == q) x[h] = cmul2(x[h], rinv[4 * h + q]);
