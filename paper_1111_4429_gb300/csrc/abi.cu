@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "runtime.h"
+#include "transform_grid.h"
 
 using namespace bgw;
 
@@ -54,8 +55,9 @@ int check_cell(Ctx* c, const bgw_cell* cell, int* n) {
   return BGW_OK;
 }
 
-// G components in [-n/2, n/2), no duplicates; returns max |G_d| per axis.
-int check_glist(Ctx* c, const char* name, int cnt, const int32_t* g, int n, int gmax[3]) {
+// G components in [-n/2, n/2), no duplicates; returns max |G_d| per axis and
+// widens the transform's box to the list.
+int check_glist(Ctx* c, const char* name, int cnt, const int32_t* g, int n, int gmax[3], GridNeed* need) {
   if (cnt <= 0) return fail(c, BGW_EINVAL, "%s: count must be >= 1", name);
   if (!g) return fail(c, BGW_EINVAL, "%s is NULL", name);
   const int lo = -(n / 2), hi = n - n / 2;  // [lo, hi)
@@ -67,6 +69,8 @@ int check_glist(Ctx* c, const char* name, int cnt, const int32_t* g, int n, int 
       if (v < lo || v >= hi)
         return fail(c, BGW_EINVAL, "%s[%d] component %d = %d outside [-n/2, n/2) for n = %d", name, i, d, v, n);
       gmax[d] = std::max(gmax[d], std::abs(v));
+      need->lo = std::min(need->lo, v);
+      need->hi = std::max(need->hi, v);
     }
     keys[i] = ((int64_t)(g[3 * i] - lo) * n + (g[3 * i + 1] - lo)) * n + (g[3 * i + 2] - lo);
   }
@@ -136,7 +140,8 @@ int max_ng(int prec) { return (int)((227 * 1024) / (prec == BGW_PREC_FP64 ? 16 :
 int validate_mtxel(Ctx* c, const bgw_cell* cell, int nv, int npw_v, const int32_t* gv, const void* cv, int nc,
                    int npw_c, const int32_t* gc, const void* cc, int ng, const int32_t* geps, int prec, void* M,
                    int* n_out) {
-  int n, rc, need = 0;
+  int n, rc;
+  GridNeed need;
   if ((rc = check_cell(c, cell, &n)) != BGW_OK) return rc;
   if ((rc = check_prec(c, prec)) != BGW_OK) return rc;
   if (nv <= 0 || nc <= 0) return fail(c, BGW_EINVAL, "nv and nc must be >= 1");
@@ -145,15 +150,15 @@ int validate_mtxel(Ctx* c, const bgw_cell* cell, int nv, int npw_v, const int32_
   if (!cv || !cc || !M) return fail(c, BGW_EINVAL, "coefficient or output pointer is NULL");
   if (ng > max_ng(prec)) return fail(c, BGW_EUNSUPPORTED, "ng = %d exceeds %d for this precision", ng, max_ng(prec));
   int mv[3], mc[3], me[3];
-  if ((rc = check_glist(c, "gv", npw_v, gv, n, mv)) != BGW_OK) return rc;
-  if ((rc = check_glist(c, "gc", npw_c, gc, n, mc)) != BGW_OK) return rc;
-  if ((rc = check_glist(c, "geps", ng, geps, n, me)) != BGW_OK) return rc;
+  if ((rc = check_glist(c, "gv", npw_v, gv, n, mv, &need)) != BGW_OK) return rc;
+  if ((rc = check_glist(c, "gc", npw_c, gc, n, mc, &need)) != BGW_OK) return rc;
+  if ((rc = check_glist(c, "geps", ng, geps, n, me, &need)) != BGW_OK) return rc;
   for (int d = 0; d < 3; ++d) {
     if (n <= mv[d] + mc[d] + me[d])
       return fail(c, BGW_EINVAL,
                   "FFT grid %d aliases on axis %d: need n > max|Gv| + max|Gc| + max|Geps| = %d + %d + %d", n, d,
                   mv[d], mc[d], me[d]);
-    need = std::max(need, mv[d] + mc[d] + me[d] + 1);
+    need.points = std::max(need.points, mv[d] + mc[d] + me[d] + 1);
   }
   *n_out = transform_grid(n, need, ng, geps);
   return BGW_OK;
@@ -1031,14 +1036,14 @@ int bgw_sigma_cohsex(bgw_ctx* ctx, const bgw_cell* cell, int no, int npw_o, cons
     return fail(c, BGW_EINVAL, "co, ci and epsinv must be device arrays");
   if (ng > max_ng(BGW_PREC_FP64)) return fail(c, BGW_EUNSUPPORTED, "ng = %d exceeds %d", ng, max_ng(BGW_PREC_FP64));
   int mo[3], mi[3], me[3];
-  if ((rc = check_glist(c, "go", npw_o, go, n, mo)) != BGW_OK) return rc;
-  if ((rc = check_glist(c, "gi", npw_i, gi, n, mi)) != BGW_OK) return rc;
-  if ((rc = check_glist(c, "geps", ng, geps, n, me)) != BGW_OK) return rc;
-  int need = 0;
+  GridNeed need;
+  if ((rc = check_glist(c, "go", npw_o, go, n, mo, &need)) != BGW_OK) return rc;
+  if ((rc = check_glist(c, "gi", npw_i, gi, n, mi, &need)) != BGW_OK) return rc;
+  if ((rc = check_glist(c, "geps", ng, geps, n, me, &need)) != BGW_OK) return rc;
   for (int d = 0; d < 3; ++d) {
     if (n <= mo[d] + mi[d] + me[d])
       return fail(c, BGW_EINVAL, "FFT grid %d aliases on axis %d: need n > max|Gi| + max|Go| + max|Geps|", n, d);
-    need = std::max(need, mo[d] + mi[d] + me[d] + 1);
+    need.points = std::max(need.points, mo[d] + mi[d] + me[d] + 1);
   }
   if ((rc = check_q(c, cell, ng, geps)) != BGW_OK) return rc;
   DeviceGuard g(c->device);
@@ -1048,7 +1053,7 @@ int bgw_sigma_cohsex(bgw_ctx* ctx, const bgw_cell* cell, int no, int npw_o, cons
   for (size_t i = 0; i < neg.size(); ++i) neg[i] = -geps[i];
   {   // -G must stay inside [-n/2, n/2) as well
     int tmp[3];
-    if ((rc = check_glist(c, "-geps", ng, neg.data(), n, tmp)) != BGW_OK) return rc;
+    if ((rc = check_glist(c, "-geps", ng, neg.data(), n, tmp, &need)) != BGW_OK) return rc;
   }
   n = transform_grid(n, need, ng, neg.data());
   const BandPlan *bpo, *bpi;

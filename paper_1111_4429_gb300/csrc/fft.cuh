@@ -24,6 +24,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "transform_grid.h"
+
 namespace bgw {
 
 template <typename T> struct cpx_t;
@@ -74,7 +76,7 @@ template <typename T, bool PK> __device__ __forceinline__ cpx<T> mul_tw(cpx<T> a
   else return mul<T>(a, b);
 }
 
-// Supported line lengths and their offsets in the twiddle table.
+// Line lengths (kSupportedN) and their offsets in the twiddle table.
 // Lengths 6, 9 and 15 serve only as the quarter-length sub-transforms of
 // 24, 36 and 60 (fft_quarters).
 __host__ __device__ constexpr int twiddle_offset(int n) {
@@ -83,7 +85,6 @@ __host__ __device__ constexpr int twiddle_offset(int n) {
        : n == 50 ? 276 : n == 60 ? 326 : n == 64 ? 386 : n == 9 ? 450 : n == 15 ? 459 : n == 6 ? 474 : -1;
 }
 constexpr int kTwiddleTotal = 480;
-constexpr int kSupportedN[] = {8, 10, 12, 16, 20, 24, 30, 32, 36, 40, 48, 50, 60, 64};
 
 // First radix of a sub-length: 4 while it divides, then 2, 3, 5.
 __host__ __device__ constexpr int first_radix(int n) {

@@ -16,31 +16,6 @@ bool fft_size_supported(int n) {
   return false;
 }
 
-// Grid of the product transform: with n > max|Gv| + max|Gc| + max|Geps| on
-// every axis the kept coefficients are those of the product itself, whatever
-// n is, so the transforms run on the smallest such supported grid instead of
-// the caller's (often a density grid, near twice the size needed).  Measured
-// per pair (y,x passes + z pass, us): spheres that need 30 points, FP32 40^3
-// 0.139, 32^3 0.080; FP64 3.70 and 1.71; spheres that need 44, FP32 60^3 0.553,
-// 48^3 0.266.  The smallest is the fastest but for 30, where 32 allows the
-// low-band lines (every kept frequency in [-8, 8)): FP32 0.096 against 0.080,
-// FP64 1.93 against 1.71.  Lines of 36 and 50 points without the low band
-// still beat low-band lines of 40 and 60.
-int transform_grid(int n, int need, int ng, const int32_t* geps) {
-  int m = n;
-  for (int s : kSupportedN)
-    if (s >= need) {
-      m = std::min(m, s);
-      break;
-    }
-  if (m == 30 && n >= 32) {
-    for (int i = 0; i < 3 * ng; ++i)
-      if (geps[i] < -8 || geps[i] >= 8) return m;
-    m = 32;
-  }
-  return m;
-}
-
 static inline int wrap(int g, int n) { return ((g % n) + n) % n; }
 
 template <typename V>

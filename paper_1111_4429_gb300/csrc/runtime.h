@@ -195,10 +195,6 @@ int upload_cached(Ctx* c, const void* host, size_t bytes, cudaStream_t st, const
 int get_band_plan(Ctx* c, int n, int npw, const int32_t* g, cudaStream_t st, const BandPlan** out);
 int get_pair_plan(Ctx* c, int n, int ng, const int32_t* geps, cudaStream_t st, const PairPlan** out);
 bool fft_size_supported(int n);
-// Grid the product transform runs on: the smallest supported one of at least
-// `need` points (max|Gv| + max|Gc| + max|Geps| + 1 over the axes, at most the
-// caller's n), on which no kept coefficient aliases.
-int transform_grid(int n, int need, int ng, const int32_t* geps);
 
 // One matrix-element evaluation with its scratch (see mtxel_kernels.cuh).
 // Codes of the pair transform's y,x kernel in the tuned-shape table: a
