@@ -164,11 +164,19 @@ int validate_mtxel(Ctx* c, const bgw_cell* cell, int nv, int npw_v, const int32_
   return BGW_OK;
 }
 
+// The ways of a call's direct run, kept for the capture that may follow it.
+struct RouteScope {
+  Ctx* c;
+  explicit RouteScope(Ctx* c) : c(c) { c->routes.record(); }
+  ~RouteScope() { c->routes.off(); }
+};
+
 // Runs body (launches on st and streams forked from it) directly the first
 // time a key is seen -- plans, tuning and pool blocks are made then -- and
 // captures a second, unexecuted pass into a CUDA graph; later calls with the
 // key replay the graph.  Pool blocks handed out during the capture stay
-// pinned for the graph's life.  With BGW_OPT_TIMING on, or on the legacy
+// pinned for the graph's life; a block that is missing ends the capture, and the
+// next call runs directly again.  With BGW_OPT_TIMING on, or on the legacy
 // default stream (not capturable), every call runs directly.
 int run_graphed(Ctx* c, uint64_t key, cudaStream_t st, const std::function<int()>& body) {
   if (!c->use_graphs || c->timing.on || st == nullptr || st == cudaStreamLegacy) return body();
@@ -179,6 +187,7 @@ int run_graphed(Ctx* c, uint64_t key, cudaStream_t st, const std::function<int()
     c->graph_replays += 1;
     return BGW_OK;
   }
+  RouteScope routes(c);
   int rc = body();
   if (rc != BGW_OK) return rc;
   if (c->graphs.size() >= kMaxGraphs) return BGW_OK;   // no more pinned scratch: run directly
@@ -187,6 +196,7 @@ int run_graphed(Ctx* c, uint64_t key, cudaStream_t st, const std::function<int()
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
+    c->routes.repeat();
     rc = body();
     e = cudaStreamEndCapture(st, &graph);
   }
@@ -747,6 +757,7 @@ extern "C" int bgw_epsilon_batch(bgw_ctx* ctx, int nq, const bgw_problem* proble
     if ((rc = upload_cached(c, p.ec, p.nc * sizeof(double), st, &dev_ec[q])) != BGW_OK) return rc;
     if ((rc = upload_cached(c, p.geps, (size_t)p.ng * 12, st, &dev_geps[q])) != BGW_OK) return rc;
   }
+  RouteScope routes(c);
   // Direct run: produces this call's results, creates the plans, tunes and
   // fills the pool with the blocks the capture below will reuse.
   if ((rc = run_batch(c, nq, problems, grids, nfreq, static_cast<const double*>(dev_om), prec, epsinv, dev_ev, dev_ec,
@@ -761,6 +772,7 @@ extern "C" int bgw_epsilon_batch(bgw_ctx* ctx, int nq, const bgw_problem* proble
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
+    c->routes.repeat();
     rc = run_batch(c, nq, problems, grids, nfreq, static_cast<const double*>(dev_om), prec, epsinv, dev_ev, dev_ec,
                    dev_geps, st);
     e = cudaStreamEndCapture(st, &graph);

@@ -202,12 +202,21 @@ static int chi_f64_on_tensor_cores(Ctx* c, long long K, int ng, const void* M, c
                                    int nrow, double scale, int accumulate, void* chi, bool real, Scratch* flags,
                                    cudaStream_t st) {
   if (real && K <= kFmaRealPairs) return BGW_OK;
+  long long chunk = 0;
+  if (c->routes.given(&chunk) && chunk == 0) return BGW_OK;
   void* p = nullptr;
-  if (c->pool.alloc((size_t)nrow * sizeof(int), &p) != BGW_OK) return BGW_OK;
-  const int rc = chi_oz_run(c, K, ng, M, wr, wc, nrow, scale, accumulate, chi, real, static_cast<int*>(p), st);
-  if (rc != BGW_OK) c->pool.release(p);
-  else flags->ptr = p;
-  return rc == BGW_ENOMEM ? BGW_OK : rc;
+  int rc = c->pool.alloc((size_t)nrow * sizeof(int), &p);
+  if (rc == BGW_OK)
+    rc = chi_oz_run(c, K, ng, M, wr, wc, nrow, scale, accumulate, chi, real, static_cast<int*>(p), &chunk, st);
+  if (rc == BGW_OK) {
+    flags->ptr = p;
+  } else if (p) {
+    c->pool.release(p);
+  }
+  if (rc != BGW_OK && rc != BGW_ENOMEM) return rc;
+  c->routes.note(rc == BGW_OK ? chunk : 0);
+  c->err.clear();
+  return BGW_OK;
 }
 
 int chi_mixed_run(Ctx* c, int prec, long long K, int ng, const void* M, const double* w, int nrow,

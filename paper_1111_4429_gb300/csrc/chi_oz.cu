@@ -630,9 +630,11 @@ int oz_launch(Ctx* c, const OzGemm& g, long long nstages, const OzSplit& s, int 
 // weights (Hermitian product; real: real M and chi), wc: complex weights (the
 // real axis: every element).  *flags [nrow] (device, zeroed here): set where
 // an operand is not finite, the rows the caller's FMA kernel must do.
-// Returns BGW_ENOMEM when the scratch does not fit (nothing was launched).
+// *chunk: pairs per chunk as a run before took them, or 0 to size it here; the
+// size taken is left there.  Returns BGW_ENOMEM when the scratch does not fit
+// (nothing was launched).
 int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, const double2* wc, int nrow, double scale,
-               int accumulate, void* chi, bool real, int* flags, cudaStream_t st) {
+               int accumulate, void* chi, bool real, int* flags, long long* chunk, cudaStream_t st) {
   using namespace oz64;
   const bool general = wc != nullptr;
   const int nsm = sm_count(c);
@@ -653,17 +655,19 @@ int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, con
   long long kc = std::min<long long>((long long)(kOzChunkBytes / per_pair) / seg_pairs * seg_pairs,
                                      (K + spp - 1) / spp * spp);
   kc = std::max<long long>(kc, std::min<long long>(seg_pairs, (K + spp - 1) / spp * spp));
-  if ((rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &meta.ptr)) != BGW_OK) return BGW_ENOMEM;
-  if (!general && (rc = c->pool.alloc((size_t)K * sizeof(double), &fac.ptr)) != BGW_OK) return BGW_ENOMEM;
+  if (*chunk > 0) kc = *chunk;
+  if ((rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &meta.ptr)) != BGW_OK) return rc;
+  if (!general && (rc = c->pool.alloc((size_t)K * sizeof(double), &fac.ptr)) != BGW_OK) return rc;
   for (;;) {
     g.kpad = (kc + spp - 1) / spp * spp;
     const long long last = K - (K - 1) / kc * kc;
     rc = oz_alloc(c, &g, general, ntiles, nsm, last, real);
     if (rc == BGW_OK) break;
     oz_release(c, &g);
-    if (kc <= kMinChunk || rc == BGW_ECUDA) return rc == BGW_ECUDA ? rc : BGW_ENOMEM;
+    if (kc <= kMinChunk || rc != BGW_ENOMEM) return rc;
     kc = std::max<long long>(kc / 2 / seg_pairs * seg_pairs, seg_pairs);
   }
+  *chunk = kc;
   const void* d_tiles;
   if ((rc = upload_cached(c, tl.data(), tl.size() * sizeof(int2), st, &d_tiles)) != BGW_OK) return rc;
   const int2* tiles = static_cast<const int2*>(d_tiles);
@@ -760,13 +764,13 @@ int sigma_oz_forms(Ctx* c, long long K, int ng, const void* M, const void* W, co
   long long rows = std::min<long long>((K + BM - 1) / BM * BM,
                                        std::max<long long>(BM, (long long)(kOzChunkBytes / 2 / row_bytes) / BM * BM));
   int rc;
-  if ((rc = c->pool.alloc((size_t)(rows + g.vrows) * sizeof(int), &meta.ptr)) != BGW_OK) return BGW_ENOMEM;
+  if ((rc = c->pool.alloc((size_t)(rows + g.vrows) * sizeof(int), &meta.ptr)) != BGW_OK) return rc;
   for (;;) {
     g.urows = (int)rows;
     rc = oz_alloc(c, &g, true, (int)(rows / BM) * nJ, nsm, g.kpad, false);
     if (rc == BGW_OK) break;
     oz_release(c, &g);
-    if (rc == BGW_ECUDA || rows == BM) return rc == BGW_ECUDA ? rc : BGW_ENOMEM;
+    if (rc != BGW_ENOMEM || rows == BM) return rc;
     rows = std::max<long long>(BM, rows / 2 / BM * BM);
   }
   std::vector<int2> tl;

@@ -485,9 +485,14 @@ __global__ void sw_finish_kernel(const __grid_constant__ SweepBatch b) {
 static bool plain_default(Ctx* c) { return c->inverse_mode == -1 && !c->run_ff_chain; }
 static bool one_step(Ctx* c, int ngmax) { return plain_default(c) && ngmax <= NB; }
 bool fma_fallback(Ctx* c, int rc) {
-  if (!plain_default(c) || (rc != BGW_ENOMEM && rc != BGW_EBUSY)) return false;
-  c->err.clear();
-  return true;
+  const bool fma = plain_default(c) && rc == BGW_ENOMEM;
+  if (fma) c->err.clear();
+  if (fma || rc == BGW_OK) c->routes.note(fma ? 0 : 1);
+  return fma;
+}
+bool fma_before(Ctx* c) {
+  long long way = 1;
+  return c->routes.given(&way) && way == 0;
 }
 
 // eps~ formation for every matrix of the batch, then the batched sweep.
@@ -541,7 +546,7 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
     const size_t upd_smem = sizeof(double2) * 2 * TU * (NB + 1);
     BGW_CUDA(c, cudaFuncSetAttribute(sw_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)upd_smem));
     std::unique_ptr<OzPlan, void (*)(OzPlan*)> oz(nullptr, oz_plan_delete);
-    if (tc_update && !one_step(c, ngmax)) {
+    if (tc_update && !one_step(c, ngmax) && !fma_before(c)) {
       oz.reset(oz_plan_new());
       std::vector<int> ngs(nb);
       std::vector<double2*> As(nb);
@@ -556,12 +561,12 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
       }
       rc = oz_prepare(c, nb, ngs.data(), As.data(), Cs.data(), Ps.data(), Ds.data(), oz.get(), false, real_values,
                       c->run_slices, c->run_ff_chain);
-      if (rc == BGW_OK)
-        oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
-      else if (fma_fallback(c, rc))
+      if (fma_fallback(c, rc))
         oz.reset();
-      else
+      else if (rc != BGW_OK)
         return rc;
+      else
+        oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
     }
     if (!oz) {
       for (int k0 = 0; k0 < ngmax; k0 += NB) {

@@ -534,7 +534,7 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
     }
     TimedScope ts(c, kTInverse, st);
     std::unique_ptr<OzPlan, void (*)(OzPlan*)> oz(nullptr, oz_plan_delete);
-    if (tc_update) {
+    if (tc_update && !fma_before(c)) {
       oz.reset(oz_plan_new());
       std::vector<int> ngs(nb, n);
       std::vector<double2*> As(nb);
@@ -546,12 +546,12 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
       }
       rc = oz_prepare(c, nb, ngs.data(), As.data(), Rs.data(), Cs.data(), nullptr, oz.get(), true, false,
                       c->run_slices, c->run_ff_chain);
-      if (rc == BGW_OK)
-        oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
-      else if (fma_fallback(c, rc))
+      if (fma_fallback(c, rc))
         oz.reset();
-      else
+      else if (rc != BGW_OK)
         return rc;
+      else
+        oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
     }
     int* piv = ipiv.as<int>();
     int* src = piv + (size_t)kGB * ngmax;

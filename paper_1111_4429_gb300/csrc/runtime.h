@@ -121,11 +121,36 @@ struct BatchGraph {
   uint64_t kernels = 0;   // kernel launches the graph holds (added to the launch count per replay)
 };
 
+// The ways a direct run took where free scratch decides (pairs per chunk of
+// digits, tensor cores or FMA sweep), in order.  The capture that follows it
+// takes the same ways: there the pool has no new memory to offer, and a way
+// chosen for that reason would stay in the graph.  A block that is missing then
+// ends the capture.
+class Routes {
+ public:
+  void record() { mode_ = kRecord; taken_.clear(); }
+  void repeat() { mode_ = kRepeat; next_ = 0; }
+  void off() { mode_ = kOff; taken_.clear(); }
+  // The way the direct run took here; false where the caller decides.
+  bool given(long long* way) {
+    if (mode_ != kRepeat || next_ >= taken_.size()) return false;
+    *way = taken_[next_++];
+    return true;
+  }
+  void note(long long way) { if (mode_ == kRecord) taken_.push_back(way); }
+
+ private:
+  enum Mode { kOff, kRecord, kRepeat } mode_ = kOff;
+  std::vector<long long> taken_;
+  size_t next_ = 0;
+};
+
 struct Ctx {
   int device = 0;
   Timing timing;
   std::unordered_map<uint64_t, BatchGraph> graphs;
   uint64_t graph_replays = 0;
+  Routes routes;
   bool use_graphs = true;          // false in the server's slot contexts (one-shot buffers per request)
   std::map<std::tuple<int, int, int, int>, int> tuned_ppb;  // (n, prec, nys, ncol) -> pairs per CTA
   bool autotune = true;
@@ -254,9 +279,10 @@ int chi_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const doubl
             bool real = false);
 // FP64 chi on the tensor cores (chi_oz.cu): BGW_ENOMEM when its scratch does
 // not fit (nothing launched), flags[f] set on the device where the FP64 FMA
-// kernel must do frequency f (operands that are not finite).
+// kernel must do frequency f (operands that are not finite).  *chunk: pairs
+// per chunk of digits, 0 to size it here (the size taken is returned).
 int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, const double2* wc, int nrow,
-               double scale, int accumulate, void* chi, bool real, int* flags, cudaStream_t st);
+               double scale, int accumulate, void* chi, bool real, int* flags, long long* chunk, cudaStream_t st);
 // The FP64 Sigma forms of K pairs (M [K][ng], W [ng][ng], sv = v^1/2) on the
 // tensor cores; *flag and the return value as chi_oz_run's.
 int sigma_oz_forms(Ctx* c, long long K, int ng, const void* M, const void* W, const double* sv, double* qW, double* qV,
@@ -270,8 +296,10 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
                      const int32_t* const* d_geps, const void* const* chi, void* const* eps, void* const* epsinv,
                      cudaStream_t st, bool tc_update, bool real_values = false);
 // Whether the FMA sweep takes over an FP64 inverse whose tensor-core buffers
-// could not be had (rc from oz_prepare): under the default option only.
+// do not fit (rc from oz_prepare): under the default option only.  Notes the
+// way taken; fma_before: the direct run before this capture took the FMA sweep.
 bool fma_fallback(Ctx* c, int rc);
+bool fma_before(Ctx* c);
 // eps~ = I - sv chi sv of one matrix into A (and eps when non-NULL), sv from
 // the cell's Coulomb model (epsinv.cu).
 int eps_form_run(Ctx* c, const bgw_cell* cell, const int32_t* d_geps, int ng, const void* chi, double* sv,

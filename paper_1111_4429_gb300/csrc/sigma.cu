@@ -347,12 +347,9 @@ int sigma_run(Ctx* c, const bgw_cell* cell, int n, int no, const BandPlan* bpo, 
       // (behind the device flag) an operand is not finite
       Scratch flag;
       flag.pool = &c->pool;
-      if (c->pool.alloc(sizeof(int), &flag.ptr) == BGW_OK) {
+      if ((rc = c->pool.alloc(sizeof(int), &flag.ptr)) == BGW_OK)
         rc = sigma_oz_forms(c, K, ng, sM.ptr, sW.ptr, sv.as<double>(), qW, qV, flag.as<int>(), st);
-        if (rc != BGW_OK && rc != BGW_ENOMEM) return rc;
-      } else {
-        rc = BGW_ENOMEM;
-      }
+      if (rc != BGW_OK && rc != BGW_ENOMEM) return rc;
       const int* guard = rc == BGW_OK ? flag.as<int>() : nullptr;
       sigma_quad_kernel<<<dim3((unsigned)((K + TQ - 1) / TQ), ntg), 256, 0, st>>>(
           sM.as<double2>(), K, ng, sW.as<double2>(), guard, part.as<double2>());
