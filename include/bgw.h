@@ -196,7 +196,8 @@ int bgw_graph_stats(bgw_ctx* ctx, uint64_t* graphs, uint64_t* replays);
  *    (default) and 7: error near 2^-48 of the update's scale (FP64-level
  *    inverse); 5: near 2^-34 with 15 slice products per tile instead of 28
  *    (implies BGW_OPT_DOUBLE_FP32).  For inputs whose own errors are far
- *    larger and ε̃ that is well conditioned.                                 */
+ *    larger and ε̃ that is well conditioned.  FP64 inputs (BGW_PREC_FP64,
+ *    bgw_epsinv*) take five only under BGW_OPT_INVERSE = 1.                 */
 /*  BGW_OPT_DOUBLE_FP32: the tensor-core sweep's critical chain -- the next
  *    32 x 32 diagonal block's sweep and the panel product P = C D^-1 -- in
  *    double-FP32 arithmetic (value = hi + lo, about 2^-46 per operation,
@@ -204,7 +205,7 @@ int bgw_graph_stats(bgw_ctx* ctx, uint64_t* graphs, uint64_t* replays);
  *    on GB300 issues 64 times the FP64 pipe's operations.  -1 (default): on
  *    in bgw_epsilon, bgw_epsilon_real, bgw_epsilon_batch and the server for
  *    the mixed precisions, off for FP64 inputs and for bgw_epsinv*; 0: off;
- *    1: on.                                                                */
+ *    1: on (FP64 inputs and bgw_epsinv*: only under BGW_OPT_INVERSE = 1).   */
 /*  BGW_OPT_PAIR_KERNEL: which kernel runs the pair transform's y and x
  *    passes.  -1 (default): the autotuner's choice (or the fixed default
  *    while BGW_OPT_AUTOTUNE is 0); 0: one (pair block, plane) per CTA with

@@ -227,15 +227,18 @@ int run_graphed(Ctx* c, uint64_t key, cudaStream_t st, const std::function<int()
 // BGW_OPT_INVERSE asks for FP64 FMA.
 bool use_tc_inverse(Ctx* c) { return c->inverse_mode != 0; }
 
-// Precision of the tensor-core inverse for a call of precision prec: seven
-// slices unless the option asks for five (near 2^-34); the mixed precisions
-// take the level sums (near 2^-48), the next diagonal block and the panel
-// product in double FP32 (about 2^-46), FP64 inputs join the level sums in
-// integers (below the roundings of the FMA sweep) and stay FP64 elsewhere.
+// Precision of the tensor-core inverse for a call of precision prec.  The mixed
+// precisions: seven slices unless the option asks for five (near 2^-34), the
+// level sums (near 2^-48), the next diagonal block and the panel product in
+// double FP32 (about 2^-46) unless the option says FP64.  FP64 inputs keep seven
+// slices, level sums joined in integers and the FP64 chain whatever those
+// options say, unless BGW_OPT_INVERSE asks for the tensor cores by itself.
 // Recorded in the context for the inverse that follows.
 void set_run_slices(Ctx* c, int prec) {
-  c->run_slices = c->update_slices ? c->update_slices : 7;
-  c->run_ff_chain = c->double_fp32 == 1 || (c->double_fp32 == -1 && prec != BGW_PREC_FP64) || c->run_slices < 7;
+  const bool plain = prec == BGW_PREC_FP64 && c->inverse_mode != 1;
+  c->run_slices = !plain && c->update_slices ? c->update_slices : 7;
+  c->run_ff_chain = !plain && (c->double_fp32 == 1 || (c->double_fp32 == -1 && prec != BGW_PREC_FP64) ||
+                               c->run_slices < 7);
 }
 
 int init_device(Ctx* c) {

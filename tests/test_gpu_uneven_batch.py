@@ -37,6 +37,7 @@ def test_uneven(sizes, items, chain, cu):
         chis.append(torch.from_numpy(chi).cuda())
         eps.append(np.eye(n) - sv[:, None] * chi * sv[None, :])
     invs = [torch.zeros_like(c) for c in chis]
+    ctx.set_option(bgw.BGW_OPT_INVERSE, 1 if chain else -1)   # FP64 inputs take the double-FP32 chain by request only
     ctx.set_option(bgw.BGW_OPT_DOUBLE_FP32, chain)
     ctx.set_option(bgw.BGW_OPT_UPDATE_ITEMS, items)
     ctx.epsinv(cells, lists, chis, None, invs)
