@@ -92,18 +92,23 @@ __device__ __forceinline__ double2 operand(const void* __restrict__ M, const dou
   }
 }
 
-__device__ __forceinline__ int exp_field(double x) {
-  return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7FFu);
+// Size of a value as an integer that orders as its binary exponent: 0 for zero,
+// 1 below the normal range, then the exponent field + 1; kNotFinite for an
+// infinity or NaN.
+constexpr int kNotFinite = 0x800;
+__device__ __forceinline__ int size_of(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7FFFFFFFu;
+  return (hi | (unsigned)__double2loint(x)) ? (int)(hi >> 20) + 1 : 0;
 }
-// Scale exponent of a column from its largest exponent field: |x| 2^-e < 1.
-__device__ __forceinline__ int scale_of(int field) { return field ? field - 1022 : 0; }
+// Scale exponent of a column from its largest size: |x| 2^-e < 1.
+__device__ __forceinline__ int scale_of(int size) { return size ? size - 1023 : 0; }
 
 __global__ void sqrt_weights_kernel(const double* __restrict__ w, long long K, double* __restrict__ out) {
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < K) out[p] = sqrt(fabs(w[p]));
 }
 
-// field[g] = largest exponent field over the pairs; *flag = 1 where a value is
+// field[g] = largest size over the pairs; *flag = 1 where a value is
 // not finite.  One pass over M (HBM bound).  grid (ceil(ng/64), strips of
 // pairs), block 256 = 64 columns x 4 pairs.
 template <int OP>
@@ -117,14 +122,14 @@ __global__ void __launch_bounds__(256) colmax_kernel(const void* __restrict__ M,
   if (g < ng)
     for (long long p = (long long)blockIdx.y * 4 + ty; p < K; p += 4LL * gridDim.y) {
       const double2 v = operand<OP>(M, fac, wc, p, g, ng);
-      m = max(m, max(exp_field(v.x), exp_field(v.y)));
+      m = max(m, max(size_of(v.x), size_of(v.y)));
     }
   red[ty][tx] = m;
   __syncthreads();
   if (ty == 0 && g < ng) {
     m = max(max(red[0][tx], red[1][tx]), max(red[2][tx], red[3][tx]));
     if (m) atomicMax(field + g, m);
-    if (m == 0x7FF) atomicExch(flag, 1);
+    if (m == kNotFinite) atomicExch(flag, 1);
   }
 }
 
@@ -207,14 +212,14 @@ __global__ void __launch_bounds__(256) row_digits_kernel(const double2* __restri
   if (r < R)
     for (int k = lane; k < K; k += 32) {
       const double2 v = src[(size_t)r * K + k];
-      m = max(m, max(exp_field(v.x), exp_field(v.y)));
+      m = max(m, max(size_of(v.x), size_of(v.y)));
     }
   m = __reduce_max_sync(0xffffffffu, m);
   if (lane == 0) {
     field[r] = m;
-    if (m == 0x7FF) atomicExch(flag, 1);
+    if (m == kNotFinite) atomicExch(flag, 1);
   }
-  if (m == 0x7FF) m = 0;   // the product is not used
+  if (m == kNotFinite) m = 0;   // the product is not used
   const int e = scale_of(m);
   const size_t plane = (size_t)rows * rowlen;
   for (size_t x = 0; x < rowlen; x += 64) {

@@ -108,3 +108,25 @@ def test_sigma_forms_at_tile_edges(no, ni, nocc):
         for k, key in enumerate(("X", "SX", "CH")):
             want = np.real(ref[key])
             assert np.abs(got[k] - want).max() <= 1e-12 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("real", [False, True])
+def test_columns_below_the_normal_range(real):
+    """A column of subnormals against one near 1e290: their element of chi is an ordinary number.  Rounding an operand
+    near 1e-309 to the subnormals' spacing of 5e-324 costs 5e-15 of it."""
+    from paper_1111_4429_gb300 import bgw
+    ctx, cell = bgw.Context(0), bgw.make_cell(*CELL)
+    ng, nv, nc = 3, 2, 40
+    r = np.random.default_rng(8)
+    m = r.standard_normal((nv * nc, ng)) + (0 if real else 1j * r.standard_normal((nv * nc, ng)))
+    m[:, 1] = m[:, 0] * np.exp(0.2j if not real else 0.0) + 0.1 * m[:, 1]
+    big, small = m * 1.0, m[:, 0] * 1e-309
+    m = np.stack([small, m[:, 1] * 1e290, m[:, 2]], 1)
+    ev, ec = np.sort(r.uniform(-0.5, 0.0, nv)), np.sort(r.uniform(0.04, 1.5, nc))
+    chi = torch.zeros((1, ng, ng), dtype=torch.float64 if real else torch.complex128, device="cuda")
+    ctx.chi_sum(cell, nv, nc, ng, torch.from_numpy(m).cuda(), ev, ec, None, bgw.BGW_FLAVOR_REAL if real else 0, False,
+                chi)
+    ctx.sync()
+    w = 1.0 / np.subtract.outer(ev, ec).ravel()
+    want = np.sum(big[:, 0].conj() * w * (m[:, 1] * 1e-290)) * 1e-19 * (4.0 / CELL[1])
+    assert abs(chi[0, 0, 1].item() - want) <= 1e-13 * abs(want)
