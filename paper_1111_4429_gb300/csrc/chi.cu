@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(256) chi_f64_real_kernel(const double* __restr
 
 // The FP64 product on the tensor cores where it is the faster one: *flags
 // then holds one device word per frequency, set where the FMA kernel must do
-// it after all (operands that are not finite).  Real products of a few pairs,
+// it after all (operands that are not finite, or pairs of very different sizes).  Real products of a few pairs,
 // and calls whose scratch does not fit, leave *flags empty: the FMA kernels do
 // them.
 static int chi_f64_on_tensor_cores(Ctx* c, long long K, int ng, const void* M, const double* wr, const double2* wc,

@@ -18,7 +18,9 @@
 // converted to FP64 once per CTA.  What is lost are the bits of X below
 // 2^(e - 56) and the levels past 7: an error near 2^-58 sqrt(6 K) 2^(e_G + e_G'),
 // against 2^-53 0.3 sqrt(K) |chi| of a running FP64 sum (chi_f64_kernel); the
-// running sum's error grows with K, this one's relative size does not.
+// running sum's error grows with K, this one's relative size does not.  The
+// bound is relative to (chi_GG chi_G'G')^1/2; for it to hold for every block of
+// chi as well, the pairs' sizes may not spread too far (kSpreadBits).
 //
 // Why: the SM's FP64 pipe (2 FMA per clock) bounds chi_f64_kernel at
 // 1.12 TFLOP/s; 36 exact FP16 products per FP64 one on the tensor cores are
@@ -35,9 +37,9 @@
 // diagonal: 6.6e-16 / 2.0e-16 at K 25600 (FMA kernel 4.1e-15 / 3.0e-15),
 // 1.6e-16 / 1.0e-16 at K 2400 (7.7e-16 / 1.9e-15).
 //
-// A column with an infinity or NaN cannot be scaled: the maximum pass then
-// sets a device flag, the kernels here return and chi_f64_kernel, launched
-// behind the same flag, does the call.
+// A column with an infinity or NaN cannot be scaled, and pairs of very different
+// sizes lose bits: the maximum pass then sets a device flag, the kernels here
+// return and chi_f64_kernel, launched behind the same flag, does the call.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -69,9 +71,10 @@ static_assert(kSmem <= 227 * 1024, "shared memory of one CTA");
 constexpr int kTileElems = BM * BN;
 
 // Operand values of pair p and column g, as the maximum and digit passes read
-// them.  kHerm: M sqrt|w| (complex), kReal: the same with real M, kPlain: M,
-// kWeighted: w M with complex w.
-enum Operand { kHerm = 0, kReal = 1, kPlain = 2, kWeighted = 3 };
+// them.  kHerm: M sqrt|w| (complex), kReal: the same with real M, kWeighted:
+// M w / sqrt|w| with complex w (against kHerm: a resonance's weight is shared
+// by both operands, so that neither spreads over the pairs more than its root).
+enum Operand { kHerm = 0, kReal = 1, kWeighted = 2 };
 
 template <int OP>
 __device__ __forceinline__ double2 operand(const void* __restrict__ M, const double* __restrict__ fac,
@@ -83,11 +86,9 @@ __device__ __forceinline__ double2 operand(const void* __restrict__ M, const dou
     if constexpr (OP == kHerm) {
       const double s = fac[p];
       return make_double2(m.x * s, m.y * s);
-    } else if constexpr (OP == kWeighted) {
+    } else {
       const double2 w = wc[p];
       return make_double2(fma(w.x, m.x, -w.y * m.y), fma(w.x, m.y, w.y * m.x));
-    } else {
-      return m;
     }
   }
 }
@@ -103,34 +104,96 @@ __device__ __forceinline__ int size_of(double x) {
 // Scale exponent of a column from its largest size: |x| 2^-e < 1.
 __device__ __forceinline__ int scale_of(int size) { return size ? size - 1023 : 0; }
 
-__global__ void sqrt_weights_kernel(const double* __restrict__ w, long long K, double* __restrict__ out) {
+// A column's scale is set by its largest entry over all pairs, so a pair 2^s
+// smaller than the largest one keeps s bits less of its operands.  Norm-wise
+// nothing is lost, but blocks of chi that only the smaller pairs make are.
+// Sizes of the pairs (their largest operand) further apart than 2^kSpreadBits
+// leave the call to the FMA kernels.  Blocks made by pairs 2^s below the largest
+// one, relative error here / in running sums: K 240, s 6 / 8 / 12 / 20: 4.9e-16,
+// 1.7e-15, 2.8e-14, 6.6e-12 / 5.5e-16; K 2400: 5e-16, 1.6e-15, 2.1e-14, 7.5e-12 /
+// 1.7e-15.  Pairs of one band structure lie within 2^7: sqrt|w| over gaps of 0.04
+// to 2 Ha 2^2.8, on the real axis (broadening 0.02 and more) 2^5, elements 2^2.
+constexpr int kSpreadBits = 8;
+
+// sqrt|w|, and for complex weights w / sqrt|w|.
+__global__ void sqrt_weights_kernel(const double* __restrict__ w, const double2* __restrict__ wc, long long K,
+                                    double* __restrict__ out, double2* __restrict__ outc) {
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < K) out[p] = sqrt(fabs(w[p]));
+  if (p >= K) return;
+  if (!wc) {
+    out[p] = sqrt(fabs(w[p]));
+    return;
+  }
+  const double2 z = wc[p];
+  const double s = sqrt(hypot(z.x, z.y));
+  out[p] = s;
+  outc[p] = s > 0.0 ? make_double2(z.x / s, z.y / s) : z;
 }
 
-// field[g] = largest size over the pairs; *flag = 1 where a value is
-// not finite.  One pass over M (HBM bound).  grid (ceil(ng/64), strips of
-// pairs), block 256 = 64 columns x 4 pairs.
+// Sizes of one operand, zeroed before the pass that fills them: of each
+// column, of each pair, and how many CTAs are done.
+struct Sizes {
+  int* col;
+  int* pair;
+  int* done;
+};
+
+// sz.col[g] = largest size over the pairs, sz.pair[p] = largest size over the
+// columns; *flag = 1 where a value is not finite or, found by the last CTA, the
+// pairs' sizes spread by more than kSpreadBits.  One pass over M (HBM bound).
+// grid (ceil(ng/64), strips of pairs), block 256 = 64 columns x 4 pairs.
 template <int OP>
 __global__ void __launch_bounds__(256) colmax_kernel(const void* __restrict__ M, const double* __restrict__ fac,
                                                      const double2* __restrict__ wc, long long K, int ng,
-                                                     int* __restrict__ field, int* __restrict__ flag) {
+                                                     const Sizes sz, int* __restrict__ flag) {
   __shared__ int red[4][64];
+  __shared__ int lohi[2], last;
   const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
   const int g = blockIdx.x * 64 + tx;
   int m = 0;
-  if (g < ng)
-    for (long long p = (long long)blockIdx.y * 4 + ty; p < K; p += 4LL * gridDim.y) {
+#pragma unroll 4
+  for (long long p = (long long)blockIdx.y * 4 + ty; p < K; p += 4LL * gridDim.y) {   // a warp has one pair
+    int k = 0;
+    if (g < ng) {
       const double2 v = operand<OP>(M, fac, wc, p, g, ng);
-      m = max(m, max(size_of(v.x), size_of(v.y)));
+      k = max(size_of(v.x), size_of(v.y));
     }
+    m = max(m, k);
+    const int row = __reduce_max_sync(0xffffffffu, k);
+    if ((tx & 31) == 0 && row) atomicMax(sz.pair + p, row);
+  }
   red[ty][tx] = m;
   __syncthreads();
   if (ty == 0 && g < ng) {
     m = max(max(red[0][tx], red[1][tx]), max(red[2][tx], red[3][tx]));
-    if (m) atomicMax(field + g, m);
+    if (m) atomicMax(sz.col + g, m);
     if (m == kNotFinite) atomicExch(flag, 1);
   }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(sz.done, 1) == (int)(gridDim.x * gridDim.y) - 1;
+    lohi[0] = kNotFinite;
+    lohi[1] = 0;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  int lo = kNotFinite, hi = 0;   // over the pairs that are not zero
+#pragma unroll 8
+  for (long long p = threadIdx.x; p < K; p += 256) {
+    const int k = __ldcg(sz.pair + p);
+    if (k) lo = min(lo, k);
+    hi = max(hi, k);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&lohi[0], lo);
+    atomicMax(&lohi[1], hi);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && lohi[1] - lohi[0] > kSpreadBits) atomicExch(flag, 1);
 }
 
 // Digit a of two adjacent values (X0, X1: rint(x 2^(56 - e))) as a half2:
@@ -542,11 +605,11 @@ constexpr size_t kOzChunkBytes = size_t(1) << 30;
 constexpr long long kMinChunk = 512;
 
 template <int OP>
-void launch_colmax(Ctx* c, const void* M, const double* fac, const double2* wc, long long K, int ng, int* field,
-                   int* flag, cudaStream_t st) {
+void launch_colmax(Ctx* c, const void* M, const double* fac, const double2* wc, long long K, int ng,
+                   const oz64::Sizes& sz, int* flag, cudaStream_t st) {
   const int gx = (ng + 63) / 64;
   const int gy = (int)std::min<long long>((K + 3) / 4, std::max(1, sm_count(c) * 8 / gx));
-  oz64::colmax_kernel<OP><<<dim3(gx, gy), 256, 0, st>>>(M, fac, wc, K, ng, field, flag);
+  oz64::colmax_kernel<OP><<<dim3(gx, gy), 256, 0, st>>>(M, fac, wc, K, ng, sz, flag);
 }
 }  // namespace
 
@@ -634,7 +697,8 @@ int oz_launch(Ctx* c, const OzGemm& g, long long nstages, const OzSplit& s, int 
 // The FP64 polarizability of nrow frequencies on the tensor cores.  wr: real
 // weights (Hermitian product; real: real M and chi), wc: complex weights (the
 // real axis: every element).  *flags [nrow] (device, zeroed here): set where
-// an operand is not finite, the rows the caller's FMA kernel must do.
+// an operand is not finite or the pairs spread too far (kSpreadBits), the rows
+// the caller's FMA kernel must do.
 // *chunk: pairs per chunk as a run before took them, or 0 to size it here; the
 // size taken is left there.  Returns BGW_ENOMEM when the scratch does not fit
 // (nothing was launched).
@@ -654,6 +718,9 @@ int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, con
   OzGemm g(&c->pool);
   Scratch meta, fac;
   meta.pool = fac.pool = &c->pool;
+  // sizes of the operands (two where the columns' differ from the rows'), and the pairs' factors
+  const int nop = general ? 2 : 1;
+  const size_t meta_bytes = (size_t)nop * (rows + K + 1) * sizeof(int);
   g.urows = g.vrows = rows;
   // chunk of pairs, whole segments
   const long long seg_pairs = kSegStages * spp, per_pair = (long long)S * rows * (real ? 2 : 4) * (general ? 2 : 1);
@@ -661,8 +728,8 @@ int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, con
                                      (K + spp - 1) / spp * spp);
   kc = std::max<long long>(kc, std::min<long long>(seg_pairs, (K + spp - 1) / spp * spp));
   if (*chunk > 0) kc = *chunk;
-  if ((rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &meta.ptr)) != BGW_OK) return rc;
-  if (!general && (rc = c->pool.alloc((size_t)K * sizeof(double), &fac.ptr)) != BGW_OK) return rc;
+  if ((rc = c->pool.alloc(meta_bytes, &meta.ptr)) != BGW_OK) return rc;
+  if ((rc = c->pool.alloc((size_t)K * (general ? 3 : 1) * sizeof(double), &fac.ptr)) != BGW_OK) return rc;
   for (;;) {
     g.kpad = (kc + spp - 1) / spp * spp;
     const long long last = K - (K - 1) / kc * kc;
@@ -677,28 +744,29 @@ int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, con
   if ((rc = upload_cached(c, tl.data(), tl.size() * sizeof(int2), st, &d_tiles)) != BGW_OK) return rc;
   const int2* tiles = static_cast<const int2*>(d_tiles);
   if ((rc = oz_maps(c, &g)) != BGW_OK) return rc;
-  int* field = meta.as<int>();
-  int* yfield = general ? field + rows : field;
+  Sizes sz[2];
+  for (int k = 0; k < nop; ++k) {
+    sz[k].col = meta.as<int>() + (size_t)k * (rows + K + 1);
+    sz[k].pair = sz[k].col + rows;
+    sz[k].done = sz[k].pair + K;
+  }
+  const int *field = sz[0].col, *yfield = sz[nop - 1].col;
+  double2* wf = general ? fac.as<double2>() : nullptr;   // 16-byte aligned: before the roots
+  double* fp = general ? fac.as<double>() + 2 * K : fac.as<double>();
   BGW_CUDA(c, cudaMemsetAsync(flags, 0, nrow * sizeof(int), st));
   for (int f = 0; f < nrow; ++f) {
-    const double* w = general ? nullptr : wr + (size_t)f * K;
-    const double2* w2 = general ? wc + (size_t)f * K : nullptr;
-    const double* fp = fac.as<double>();
     int* flag = flags + f;
     {
       TimedScope ts(c, kTChiSplit, st);
-      BGW_CUDA(c, cudaMemsetAsync(meta.ptr, 0, (size_t)2 * rows * sizeof(int), st));
-      if (!general) {
-        sqrt_weights_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(w, K, fac.as<double>());
-        if (real)
-          launch_colmax<kReal>(c, M, fp, nullptr, K, ng, field, flag, st);
-        else
-          launch_colmax<kHerm>(c, M, fp, nullptr, K, ng, field, flag, st);
-      } else {
-        launch_colmax<kPlain>(c, M, nullptr, nullptr, K, ng, field, flag, st);
-        launch_colmax<kWeighted>(c, M, nullptr, w2, K, ng, yfield, flag, st);
-      }
-      c->launches += 2;
+      BGW_CUDA(c, cudaMemsetAsync(meta.ptr, 0, meta_bytes, st));
+      sqrt_weights_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(
+          general ? nullptr : wr + (size_t)f * K, general ? wc + (size_t)f * K : nullptr, K, fp, wf);
+      if (real)
+        launch_colmax<kReal>(c, M, fp, nullptr, K, ng, sz[0], flag, st);
+      else
+        launch_colmax<kHerm>(c, M, fp, nullptr, K, ng, sz[0], flag, st);
+      if (general) launch_colmax<kWeighted>(c, M, nullptr, wf, K, ng, sz[1], flag, st);
+      c->launches += 1 + nop;
     }
     for (long long p0 = 0; p0 < K; p0 += kc) {
       const long long kn = std::min(kc, K - p0), nst = (kn + spp - 1) / spp;
@@ -708,14 +776,13 @@ int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, con
         // rows of the planes are rowlen long; a shorter last chunk fills the
         // first nst stages of each row and the product reads no further
         __half* up = g.u.as<__half>();
-        if (real) {
+        if (real)
           digits_kernel<kReal><<<grid, 256, 0, st>>>(M, fp, nullptr, p0, kn, ng, rows, g.rowlen, field, flag, up);
-        } else if (!general) {
+        else
           digits_kernel<kHerm><<<grid, 256, 0, st>>>(M, fp, nullptr, p0, kn, ng, rows, g.rowlen, field, flag, up);
-        } else {
-          digits_kernel<kPlain><<<grid, 256, 0, st>>>(M, nullptr, nullptr, p0, kn, ng, rows, g.rowlen, field, flag, up);
+        if (general) {
           digits_kernel<kWeighted>
-              <<<grid, 256, 0, st>>>(M, nullptr, w2, p0, kn, ng, rows, g.rowlen, yfield, flag, g.v.as<__half>());
+              <<<grid, 256, 0, st>>>(M, nullptr, wf, p0, kn, ng, rows, g.rowlen, yfield, flag, g.v.as<__half>());
           c->launches += 1;
         }
         BGW_CUDA(c, cudaGetLastError());

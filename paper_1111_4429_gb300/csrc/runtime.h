@@ -279,7 +279,8 @@ int chi_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const doubl
             bool real = false);
 // FP64 chi on the tensor cores (chi_oz.cu): BGW_ENOMEM when its scratch does
 // not fit (nothing launched), flags[f] set on the device where the FP64 FMA
-// kernel must do frequency f (operands that are not finite).  *chunk: pairs
+// kernel must do frequency f (operands that are not finite, or pairs of very
+// different sizes).  *chunk: pairs
 // per chunk of digits, 0 to size it here (the size taken is returned).
 int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, const double2* wc, int nrow,
                double scale, int accumulate, void* chi, bool real, int* flags, long long* chunk, cudaStream_t st);

@@ -130,3 +130,56 @@ def test_columns_below_the_normal_range(real):
     w = 1.0 / np.subtract.outer(ev, ec).ravel()
     want = np.sum(big[:, 0].conj() * w * (m[:, 1] * 1e-290)) * 1e-19 * (4.0 / CELL[1])
     assert abs(chi[0, 0, 1].item() - want) <= 1e-13 * abs(want)
+
+
+def _exact_product(x, y):
+    """sum_p conj(x_p) y_p of [K][a] and [K][b] in extended precision."""
+    q = np.clongdouble
+    return np.einsum("pa,pb->ab", x.conj().astype(q), y.astype(q))
+
+
+# Pairs at most 2^9 apart (sizes up to 8 apart) keep operands to 2^(10 - 57) of their own largest entry, about 3
+# standard deviations: 2^-45 of a block's norm.  Pairs further apart take running FP64 sums, K^1/2 2^-53.
+@pytest.mark.parametrize("real", [False, True])
+@pytest.mark.parametrize("spread", [0, 6, 9, 13, 20, 27, 40])
+def test_blocks_made_by_the_smaller_pairs(spread, real):
+    """One pair 2^spread larger than the others in some columns and zero in the rest: the block between the two groups
+    of columns is made by the smaller pairs alone."""
+    from paper_1111_4429_gb300 import bgw
+    ctx, cell = bgw.Context(0), bgw.make_cell(*CELL)
+    ng, nv, nc = 40, 4, 60
+    r = np.random.default_rng(spread)
+    m = r.standard_normal((nv * nc, ng)) + (0 if real else 1j * r.standard_normal((nv * nc, ng)))
+    m[7, :15] *= 2.0 ** spread
+    m[7, 15:] = 0.0
+    ev, ec = np.sort(r.uniform(-0.5, 0.0, nv)), np.sort(r.uniform(0.5, 1.5, nc))
+    chi = torch.zeros((1, ng, ng), dtype=torch.float64 if real else torch.complex128, device="cuda")
+    ctx.chi_sum(cell, nv, nc, ng, torch.from_numpy(m).cuda(), ev, ec, None, bgw.BGW_FLAVOR_REAL if real else 0, False,
+                chi)
+    ctx.sync()
+    w = 1.0 / np.subtract.outer(ev, ec).ravel()
+    want = (_exact_product(m[:, :15], m[:, 15:] * w[:, None]) * (4.0 / CELL[1])).astype(complex)
+    got = chi[0].cpu().numpy()[:15, 15:]
+    assert np.linalg.norm(got - want) <= 2.0 ** -45 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("delta", [0.05, 1e-4, 1e-8])
+def test_resonance_on_the_real_axis(delta):
+    """One pair in resonance, its elements zero in the second group of columns."""
+    from paper_1111_4429_gb300 import bgw
+    ctx, cell = bgw.Context(0), bgw.make_cell(*CELL)
+    ng, nv, nc = 40, 4, 60
+    r = np.random.default_rng(4)
+    m = r.standard_normal((nv * nc, ng)) + 1j * r.standard_normal((nv * nc, ng))
+    m[7, 15:] = 0.0
+    ev, ec = np.sort(r.uniform(-0.5, 0.0, nv)), np.sort(r.uniform(0.5, 1.5, nc))
+    d = np.subtract.outer(ev, ec).ravel()
+    e = np.array([-d[7]])
+    x = torch.zeros((1, ng, ng), dtype=torch.complex128, device="cuda")
+    ctx.chi_sum_real(cell, nv, nc, ng, torch.from_numpy(m).cuda(), ev, ec, e, delta, False, 0, False, x)
+    ctx.sync()
+    w = 0.5 * (1 / (d - e[0] - 1j * delta) + 1 / (d + e[0] + 1j * delta))
+    got = x[0].cpu().numpy()
+    for rows, cols in ((slice(0, 15), slice(15, ng)), (slice(15, ng), slice(0, 15))):
+        want = (_exact_product(m[:, rows], m[:, cols] * w[:, None]) * (4.0 / CELL[1])).astype(complex)
+        assert np.linalg.norm(got[rows, cols] - want) <= 2.0 ** -45 * np.linalg.norm(want)
