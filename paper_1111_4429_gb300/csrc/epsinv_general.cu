@@ -255,14 +255,18 @@ __device__ void factor_block(double2* __restrict__ lu, int kb, double2 (*Lb)[kPB
 // the operations without the idle lanes and the last wave),
 // CTAs of one warp for the last wave's sake (of two: 17 us more); 209 us with
 // 16 columns by 16 row groups, shared memory and three barriers a row pair.
+// SIZES (FP64 inputs): sizes[m][0 / 1][k], the largest exponent fields of
+// row k of R and of column k of Cp outside the block's rows.
 constexpr int kCopyRows = 32;
 constexpr int kSolveThreads = 32, kSolveCols = kSolveThreads / 4;
 
+template <bool SIZES>
 __global__ void __launch_bounds__(kSolveThreads) solve_panels_kernel(const __grid_constant__ GenPtrs P, int ng,
                                                                      int k0, int kb,
                                                                      const double2* __restrict__ lu_all,
                                                                      double2* __restrict__ R_all,
-                                                                     double2* __restrict__ C_all) {
+                                                                     double2* __restrict__ C_all,
+                                                                     int* __restrict__ sizes) {
   const int tid = threadIdx.x;
   const int m = blockIdx.y;
   const double2* __restrict__ A = P.A[m];
@@ -272,9 +276,15 @@ __global__ void __launch_bounds__(kSolveThreads) solve_panels_kernel(const __gri
   const int ncol = (ng + kSolveCols - 1) / kSolveCols;
   if ((int)blockIdx.x >= ncol) {   // kCopyRows rows of the column panel
     const int r0 = (blockIdx.x - ncol) * kCopyRows, s = tid & 31;
+    int top = 0;
 #pragma unroll 8
     for (int r = tid >> 5; r < kCopyRows; r += kSolveThreads / 32)
-      if (s < kb && r0 + r < ng) C[(size_t)(r0 + r) * kPB + s] = A[(size_t)(r0 + r) * ng + k0 + s];
+      if (s < kb && r0 + r < ng) {
+        const double2 v = A[(size_t)(r0 + r) * ng + k0 + s];
+        C[(size_t)(r0 + r) * kPB + s] = v;
+        if (SIZES && (r0 + r < k0 || r0 + r >= k0 + kb)) top = max(top, max(exponent_field(v.x), exponent_field(v.y)));
+      }
+    if (SIZES && top) atomicMax(sizes + (m * 2 + 1) * kPB + s, top);
     return;
   }
   __shared__ double2 D[kPB][kPB];   // by columns
@@ -328,6 +338,13 @@ __global__ void __launch_bounds__(kSolveThreads) solve_panels_kernel(const __gri
   for (int h = 0; h < 8; ++h) {
     const int r = l + 4 * h;
     if (r < kb && j < ng) R[(size_t)r * ng + j] = x[h];
+  }
+  if constexpr (!SIZES) return;
+#pragma unroll
+  for (int h = 0; h < 8; ++h) {   // largest of the warp's columns in rows l + 4 h
+    int top = max(exponent_field(x[h].x), exponent_field(x[h].y));
+    for (int o = 4; o < 32; o <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    if (tid < 4 && top) atomicMax(sizes + m * 2 * kPB + l + 4 * h, top);
   }
 }
 
@@ -399,10 +416,11 @@ __global__ void __launch_bounds__(kTRows) pivot_merge_kernel(const __grid_consta
 __global__ void __launch_bounds__(256) pivot_swap_kernel(const __grid_constant__ GenPtrs Pm, int ng, int k0, int kb,
                                                          const int* __restrict__ sel_all, int cstride,
                                                          int* __restrict__ ipiv_all, double2* __restrict__ lu_all,
-                                                         int* __restrict__ status) {
+                                                         int* __restrict__ sizes, int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int m = blockIdx.y;
   if (blockIdx.x == gridDim.x - 1) {
+    if (sizes && threadIdx.x < 2 * kPB) sizes[m * 2 * kPB + threadIdx.x] = 0;   // solve_panels_kernel fills them
     factor_block(lu_all + (size_t)m * kPB * (kPB + 1), kb, reinterpret_cast<double2 (*)[kPB]>(smem_raw), status);
     return;
   }
@@ -500,9 +518,10 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
   const int cstride = nleaf_max * (kPB + 1);   // candidates then counts, per matrix
   Scratch sv, lu, R, Cp, cand, ipiv;
   sv.pool = lu.pool = R.pool = Cp.pool = cand.pool = ipiv.pool = &c->pool;
+  const size_t lu_bytes = (size_t)kGB * kPB * (kPB + 1) * sizeof(double2);   // the operands' sizes follow
   int rc;
   if ((rc = c->pool.alloc((size_t)ngmax * sizeof(double), &sv.ptr)) != BGW_OK ||
-      (rc = c->pool.alloc((size_t)kGB * kPB * (kPB + 1) * sizeof(double2), &lu.ptr)) != BGW_OK ||
+      (rc = c->pool.alloc(lu_bytes + (size_t)kGB * 2 * kPB * sizeof(int), &lu.ptr)) != BGW_OK ||
       (rc = c->pool.alloc((size_t)kGB * kPB * ngmax * sizeof(double2), &R.ptr)) != BGW_OK ||
       (rc = c->pool.alloc((size_t)kGB * kPB * ngmax * sizeof(double2), &Cp.ptr)) != BGW_OK ||
       (rc = c->pool.alloc((size_t)2 * kGB * cstride * sizeof(int), &cand.ptr)) != BGW_OK ||
@@ -553,6 +572,7 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
       else
         oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
     }
+    int* sizes = oz && !c->run_ff_chain ? reinterpret_cast<int*>(static_cast<char*>(lu.ptr) + lu_bytes) : nullptr;
     int* piv = ipiv.as<int>();
     int* src = piv + (size_t)kGB * ngmax;
     for (int k0 = 0; k0 < n; k0 += kPB) {
@@ -572,15 +592,19 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
           groups = next;
         }
         pivot_swap_kernel<<<dim3((n + kSwapCols - 1) / kSwapCols + 1, nb), 256, ssmem, st>>>(
-            P, n, k0, kb, cbuf[cur], cstride, piv, lu.as<double2>(), c->d_status);
+            P, n, k0, kb, cbuf[cur], cstride, piv, lu.as<double2>(), sizes, c->d_status);
         c->launches += 1;
         BGW_CUDA(c, cudaGetLastError());
       }
       {
         TimedScope tg(c, kTSweepChain, st);
-        solve_panels_kernel<<<dim3((n + kSolveCols - 1) / kSolveCols + (n + kCopyRows - 1) / kCopyRows, nb),
-                              kSolveThreads, 0, st>>>(
-            P, n, k0, kb, lu.as<double2>(), R.as<double2>(), Cp.as<double2>());
+        const dim3 g((n + kSolveCols - 1) / kSolveCols + (n + kCopyRows - 1) / kCopyRows, nb);
+        if (sizes)
+          solve_panels_kernel<true><<<g, kSolveThreads, 0, st>>>(P, n, k0, kb, lu.as<double2>(), R.as<double2>(),
+                                                                 Cp.as<double2>(), sizes);
+        else
+          solve_panels_kernel<false><<<g, kSolveThreads, 0, st>>>(P, n, k0, kb, lu.as<double2>(), R.as<double2>(),
+                                                                  Cp.as<double2>(), nullptr);
         c->launches += 1;
         BGW_CUDA(c, cudaGetLastError());
       }
@@ -591,7 +615,7 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
             return rc;
       } else {
         TimedScope tu(c, kTOzUpdate, st);
-        if ((rc = oz_slice(c, oz.get(), k0, n, 0, st)) != BGW_OK || (rc = oz_update(c, oz.get(), k0, n, 0, 0, st)) != BGW_OK)
+        if ((rc = oz_slice(c, oz.get(), k0, n, 0, sizes, st)) != BGW_OK || (rc = oz_update(c, oz.get(), k0, n, 0, 0, st)) != BGW_OK)
           return rc;
         c->launches += 3;
       }

@@ -364,7 +364,7 @@ int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2
                double2* const* D, OzPlan* plan, bool general, bool real_values, int slices, bool ff_chain);
 // epsinv_batch_run with real_values: the matrices are real (imaginary parts zero).
 // Slices of one pivoted Gauss-Jordan step (general plans).
-int oz_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, cudaStream_t st);
+int oz_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, const int* sizes, cudaStream_t st);
 // The Hermitian sweep's panel (C, P = C D^-1, A_RK <- P) and its slices in one launch.
 int oz_panel_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, cudaStream_t st);
 int oz_update(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, int mode, cudaStream_t st);

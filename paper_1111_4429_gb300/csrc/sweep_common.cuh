@@ -16,6 +16,8 @@ __device__ __forceinline__ double neg_bits(double x) {
   return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);
 }
 
+__device__ __forceinline__ int exponent_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+
 constexpr int kSwNB = 32;
 constexpr int kDiagThreads = 17 * 32;   // a thread per lower element, and the pivot's warp
 

@@ -196,18 +196,20 @@ __device__ __forceinline__ void digits7(long long X, __half* out, size_t stride)
 // all lanes call it.  VROW false: a row of U, re | im.  VROW true: the two
 // rows a column of the product reads (vrow): re | im for the real part of
 // P C^H and -im | re for the imaginary part, so that one MMA makes both.
-// *exp_out: the row's exponent; mark: a row that holds an infinity or NaN
-// gets kBadExp, which makes NaN of every element it updates.
-template <bool VROW>
+// *exp_out: the row's exponent.  FP64 (FP64 inputs): the lane's value counts as
+// value 2^t, and a row that holds an infinity or NaN gets kBadExp, which makes
+// NaN of every element it updates.
+template <bool VROW, bool FP64>
 __device__ __forceinline__ void slice_row(double re, double im, int lane, __half* base, size_t stride, int* exp_out,
-                                          bool mark) {
+                                          int t = 0) {
   // e = frexp exponent of the row's largest magnitude, from the biased
   // exponent fields (integer max over the warp; 0 for a zero row, and rows
   // of subnormals alone are cut to zero)
-  const unsigned er = ((unsigned)__double2hiint(re) >> 20) & 0x7FFu, ei = ((unsigned)__double2hiint(im) >> 20) & 0x7FFu;
-  const unsigned emax = __reduce_max_sync(0xffffffffu, er > ei ? er : ei);
-  const int e = emax ? (int)emax - 1022 : 0;   // |value| 2^-e < 1
-  const long long Xr = fixed56(re, e), Xi = fixed56(im, e);
+  int top = max(exponent_field(re), exponent_field(im));
+  if constexpr (FP64) top = top == 0x7FF ? kBadExp : top ? max(top + t, 1) : 0;
+  const int emax = __reduce_max_sync(0xffffffffu, top);
+  const int e = emax ? emax - 1022 : 0;   // |value| 2^(t - e) < 1
+  const long long Xr = fixed56(re, e - t), Xi = fixed56(im, e - t);
   digits7(Xr, base + lane, stride);
   digits7(Xi, base + lane + 32, stride);
   if constexpr (VROW) {
@@ -215,7 +217,7 @@ __device__ __forceinline__ void slice_row(double re, double im, int lane, __half
     digits7(-Xi, second + lane, stride);
     digits7(Xr, second + lane + 32, stride);
   }
-  if (lane == 0) *exp_out = (mark && emax == 0x7FFu) ? kBadExp : e;
+  if (lane == 0) *exp_out = FP64 && emax == kBadExp ? kBadExp : e;
 }
 
 // Row of V planes that holds column j's real-part row (its imaginary-part row
@@ -228,6 +230,11 @@ __device__ __forceinline__ size_t vrow(size_t j) { return (j >> 4) * 32 + (j & 1
 // P_i = C_i D^-1, the panel buffers and A_iK <- P_i written as the panel
 // kernel of the FP64 sweep does, then P_i and C_i cut into their slices.
 // Rows of K and padding rows get zero slices.  grid (ngpad/8, nmat).
+// FP64 inputs: P_ik 2^t_k and C_jk 2^-t_k are cut, 2^t_k near (D^-1)_kk^-1/2.
+// A row's entries are held to 2^-57 of its largest, and where the diagonal of
+// eps~ is graded (a macroscopic constant of 1e6 or 1e8 in the head) P_ik falls
+// and C_jk grows with the k-th diagonal entry: unscaled, the inverse of such a
+// matrix was off by 2e-15 and 2e-14 against 5e-16.
 // FF: P_i = C_i D^-1 in double FP32 (the five-slice update, whose target
 // precision, near 2^-34, is far above the pair arithmetic's 2^-43): the
 // products as exact pairs, their high words two-summed and the errors
@@ -322,24 +329,31 @@ __global__ void __launch_bounds__(256) panel_slice_kernel(const __grid_constant_
     }
   }
   if (lane >= kb) pv = cv = make_double2(0.0, 0.0);
+  const int t = FF ? 0 : (1023 - exponent_field(Ds[lane][lane].x)) >> 1;
   const size_t row = (size_t)M.row_off + i;
-  slice_row<false>(pv.x, pv.y, lane, U + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
-                   sig + (size_t)buf * rows_total + row, !FF);
+  slice_row<false, !FF>(pv.x, pv.y, lane, U + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
+                        sig + (size_t)buf * rows_total + row, t);
   if (vpair)
-    slice_row<true>(cv.x, cv.y, lane, V + ((size_t)buf * S * 2 * rows_total + vrow(row)) * KR,
-                    (size_t)2 * rows_total * KR, tau + (size_t)buf * rows_total + row, !FF);
+    slice_row<true, !FF>(cv.x, cv.y, lane, V + ((size_t)buf * S * 2 * rows_total + vrow(row)) * KR,
+                         (size_t)2 * rows_total * KR, tau + (size_t)buf * rows_total + row, -t);
   else   // real values: the real part's rows alone
-    slice_row<false>(cv.x, cv.y, lane, V + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
-                     tau + (size_t)buf * rows_total + row, !FF);
+    slice_row<false, !FF>(cv.x, cv.y, lane, V + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
+                          tau + (size_t)buf * rows_total + row, -t);
 }
 
 // Slices for the general (Gauss-Jordan) update A -= Cp R of the pivoted
 // inverse: z = 0 slices the column panel Cp [ng][NB] (rows of the block K
 // zero: they are overwritten with R afterwards), z = 1 slices R^H, read
 // transposed from R [NB][ng] (every row live: the block's columns receive
-// -Cp D^-1).  M.P holds Cp, M.C holds R.
+// -Cp D^-1).  M.P holds Cp, M.C holds R.  FP64 inputs (sizes): Cp_ik 2^t_k and
+// R_kj 2^-t_k, which brings both operands' largest entries of inner index k to
+// the same size, as in the Hermitian panel (head 1e6 / 1e8: 1e-14 / 1e-13 without
+// it, 4e-16 by FP64 FMA); sizes[m][0 / 1][k] are the exponent fields of the
+// largest entries of row k of R and of column k of Cp.
+template <bool FP64>
 __global__ void __launch_bounds__(256) slice_general_kernel(const __grid_constant__ OzBatch b, int k0,
-                                                            int rows_total, int buf, int mark,
+                                                            int rows_total, int buf,
+                                                            const int* __restrict__ sizes,
                                                             __half* __restrict__ U, __half* __restrict__ V,
                                                             int* __restrict__ sig, int* __restrict__ tau) {
   const OzMat& M = b.m[blockIdx.y];
@@ -360,13 +374,18 @@ __global__ void __launch_bounds__(256) slice_general_kernel(const __grid_constan
     re = v.x;
     im = -v.y;
   }
+  int t = 0;
+  if constexpr (FP64) {
+    const int r = sizes[blockIdx.y * 2 * NB + lane], q = sizes[blockIdx.y * 2 * NB + NB + lane];
+    if (r && q) t = (r - q) >> 1;
+  }
   const size_t row = (size_t)M.row_off + i;
   if (blockIdx.z == 0)
-    slice_row<false>(re, im, lane, U + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
-                     sig + (size_t)buf * rows_total + row, mark != 0);
+    slice_row<false, FP64>(re, im, lane, U + ((size_t)buf * S * rows_total + row) * KR, (size_t)rows_total * KR,
+                           sig + (size_t)buf * rows_total + row, t);
   else
-    slice_row<true>(re, im, lane, V + ((size_t)buf * S * 2 * rows_total + vrow(row)) * KR,
-                    (size_t)2 * rows_total * KR, tau + (size_t)buf * rows_total + row, mark != 0);
+    slice_row<true, FP64>(re, im, lane, V + ((size_t)buf * S * 2 * rows_total + vrow(row)) * KR,
+                          (size_t)2 * rows_total * KR, tau + (size_t)buf * rows_total + row, -t);
 }
 
 // Rows of the block K after the general update: A[k0 + r][j] = R[r][j].
@@ -938,14 +957,17 @@ int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2
 }
 
 // Slices of one pivoted Gauss-Jordan step (column panel and R^H of every matrix) into buffer buf.
-int oz_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, cudaStream_t st) {
+int oz_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, const int* sizes, cudaStream_t st) {
   using namespace oz;
   const int rpad = (ngmax + BM - 1) / BM * BM;
   if (!plan->general) return fail(c, BGW_EINVAL, "oz_slice: the Hermitian sweep slices in oz_panel_slice");
-  slice_general_kernel<<<dim3(rpad / 8, plan->nmat, 2), 256, 0, st>>>(plan->batch, k0, plan->rows_total, buf,
-                                                                      plan->ff_chain ? 0 : 1, plan->U.as<__half>(),
-                                                                      plan->V.as<__half>(), plan->sig.as<int>(),
-                                                                      plan->tau.as<int>());
+  const dim3 g(rpad / 8, plan->nmat, 2);
+  __half *U = plan->U.as<__half>(), *V = plan->V.as<__half>();
+  int *sig = plan->sig.as<int>(), *tau = plan->tau.as<int>();
+  if (plan->ff_chain)
+    slice_general_kernel<false><<<g, 256, 0, st>>>(plan->batch, k0, plan->rows_total, buf, nullptr, U, V, sig, tau);
+  else
+    slice_general_kernel<true><<<g, 256, 0, st>>>(plan->batch, k0, plan->rows_total, buf, sizes, U, V, sig, tau);
   BGW_CUDA(c, cudaGetLastError());
   return BGW_OK;
 }
