@@ -470,7 +470,11 @@ int bgw_epsilon_batch(bgw_ctx* ctx, int nq, const bgw_problem* problems,
  *   opts.hbm_budget_bytes  bound on the sum of the estimates of admitted
  *                          requests (0 = 90 % of the free device memory at
  *                          open); a request whose estimate exceeds it alone
- *                          completes with BGW_ENOMEM
+ *                          completes with BGW_ENOMEM.  BGW_PREC_FP64
+ *                          requests also take what the bound has left, up
+ *                          to their tensor-core polarizability's scratch
+ *                          (about 1 GiB and its partial sums); it runs in
+ *                          smaller chunks, or by FP64 FMA, with less
  *   opts.max_slots         1..64 requests in flight
  *   request.problem        one q-point; cv, cc are HOST arrays here
  *   request.epsinv_out     host c128 [ng][ng]; written before the request

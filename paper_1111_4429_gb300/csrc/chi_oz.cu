@@ -640,17 +640,32 @@ OzSplit oz_split(long long nstages, int ntiles, int nsm) {
   return s;
 }
 
-int oz_alloc(Ctx* c, OzGemm* g, bool two, int ntiles, int nsm, long long last, bool real) {
+// Sizes of the planes (bytes) and partial sums for chunks of g->kpad inner
+// values, the last of `last`.
+struct OzBytes {
+  size_t u, v, work;
+  size_t total() const { return u + v + work; }
+};
+OzBytes oz_bytes(OzGemm* g, bool two, int ntiles, int nsm, long long last, bool real) {
   using namespace oz64;
   const long long spp = real ? SK : SK / 2;   // pairs per stage
   g->rowlen = (size_t)(g->kpad / spp) * SK;
-  const size_t ub = (size_t)S * g->urows * g->rowlen * 2, vb = (size_t)S * g->vrows * g->rowlen * 2;
   const int ga = oz_split(g->kpad / spp, ntiles, nsm).groups, gb = oz_split((last + spp - 1) / spp, ntiles, nsm).groups;
   g->ngroups_max = std::max(ga, gb);
+  OzBytes b;
+  b.u = (size_t)S * g->urows * g->rowlen * 2;
+  b.v = two ? (size_t)S * g->vrows * g->rowlen * 2 : 0;
+  b.work = (size_t)g->ngroups_max * ntiles * kTileElems * sizeof(double2);
+  return b;
+}
+
+int oz_alloc(Ctx* c, OzGemm* g, bool two, int ntiles, int nsm, long long last, bool real) {
+  const OzBytes b = oz_bytes(g, two, ntiles, nsm, last, real);
+  if (b.total() > c->digit_room) return BGW_ENOMEM;
   int rc;
-  if ((rc = c->pool.alloc(ub, &g->u.ptr)) != BGW_OK) return rc;
-  if (two && (rc = c->pool.alloc(vb, &g->v.ptr)) != BGW_OK) return rc;
-  return c->pool.alloc((size_t)g->ngroups_max * ntiles * kTileElems * sizeof(double2), &g->work.ptr);
+  if ((rc = c->pool.alloc(b.u, &g->u.ptr)) != BGW_OK) return rc;
+  if (two && (rc = c->pool.alloc(b.v, &g->v.ptr)) != BGW_OK) return rc;
+  return c->pool.alloc(b.work, &g->work.ptr);
 }
 
 void oz_release(Ctx* c, OzGemm* g) {
@@ -694,6 +709,38 @@ int oz_launch(Ctx* c, const OzGemm& g, long long nstages, const OzSplit& s, int 
 }
 }  // namespace
 
+namespace {
+// Tiles of the product (lower ones alone for the Hermitian one).
+std::vector<int2> oz_tiles(int ng, bool general) {
+  using namespace oz64;
+  const int nI = (ng + BM - 1) / BM, nJ = (ng + BN - 1) / BN;
+  std::vector<int2> tl;
+  for (int I = 0; I < nI; ++I)
+    for (int J = 0; J < nJ; ++J)
+      if (general || J * BN <= I * BM + BM - 1) tl.push_back(make_int2(I, J));
+  return tl;
+}
+
+// Pairs per chunk: whole segments within kOzChunkBytes of digits.
+long long oz_chunk(long long K, int rows, bool general, bool real) {
+  using namespace oz64;
+  const long long spp = real ? SK : SK / 2, whole = (K + spp - 1) / spp * spp;
+  const long long seg_pairs = kSegStages * spp, per_pair = (long long)S * rows * (real ? 2 : 4) * (general ? 2 : 1);
+  const long long kc = std::min<long long>((long long)(kOzChunkBytes / per_pair) / seg_pairs * seg_pairs, whole);
+  return std::max<long long>(kc, std::min<long long>(seg_pairs, whole));
+}
+}  // namespace
+
+size_t chi_oz_bytes(Ctx* c, long long K, int ng) {
+  using namespace oz64;
+  OzGemm g(&c->pool);
+  g.urows = g.vrows = (ng + BM - 1) / BM * BM;
+  const long long kc = oz_chunk(K, g.urows, false, false);
+  g.kpad = kc;
+  const size_t b = oz_bytes(&g, false, (int)oz_tiles(ng, false).size(), sm_count(c), K - (K - 1) / kc * kc, false).total();
+  return b + (size_t(4) << 20);   // the pool rounds each block up to 2 MiB
+}
+
 // The FP64 polarizability of nrow frequencies on the tensor cores.  wr: real
 // weights (Hermitian product; real: real M and chi), wc: complex weights (the
 // real axis: every element).  *flags [nrow] (device, zeroed here): set where
@@ -707,12 +754,9 @@ int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, con
   using namespace oz64;
   const bool general = wc != nullptr;
   const int nsm = sm_count(c);
-  const int nI = (ng + BM - 1) / BM, nJ = (ng + BN - 1) / BN, rows = nI * BM;
-  const long long spp = real ? SK : SK / 2;
-  std::vector<int2> tl;
-  for (int I = 0; I < nI; ++I)
-    for (int J = 0; J < nJ; ++J)
-      if (general || J * BN <= I * BM + BM - 1) tl.push_back(make_int2(I, J));
+  const int rows = (ng + BM - 1) / BM * BM;
+  const long long spp = real ? SK : SK / 2, seg_pairs = kSegStages * spp;
+  const std::vector<int2> tl = oz_tiles(ng, general);
   const int ntiles = (int)tl.size();
   int rc;
   OzGemm g(&c->pool);
@@ -722,11 +766,7 @@ int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, con
   const int nop = general ? 2 : 1;
   const size_t meta_bytes = (size_t)nop * (rows + K + 1) * sizeof(int);
   g.urows = g.vrows = rows;
-  // chunk of pairs, whole segments
-  const long long seg_pairs = kSegStages * spp, per_pair = (long long)S * rows * (real ? 2 : 4) * (general ? 2 : 1);
-  long long kc = std::min<long long>((long long)(kOzChunkBytes / per_pair) / seg_pairs * seg_pairs,
-                                     (K + spp - 1) / spp * spp);
-  kc = std::max<long long>(kc, std::min<long long>(seg_pairs, (K + spp - 1) / spp * spp));
+  long long kc = oz_chunk(K, rows, general, real);
   if (*chunk > 0) kc = *chunk;
   if ((rc = c->pool.alloc(meta_bytes, &meta.ptr)) != BGW_OK) return rc;
   if ((rc = c->pool.alloc((size_t)K * (general ? 3 : 1) * sizeof(double), &fac.ptr)) != BGW_OK) return rc;

@@ -175,6 +175,7 @@ struct Ctx {
   bool chi_tc_ready = false;
   uint64_t launches = 0;     // kernels launched by this context
   int chi_segment_pairs = 0; // mixed chi: pairs per FP32 accumulation segment (0 = default)
+  size_t digit_room = SIZE_MAX;  // FP64 chi: bytes its digit planes and partial sums may take (the server's admission)
   int chi_chunk_pairs = 0;   // mixed chi: pairs per chunk of operand planes (0 = sized to 4 GiB)
   unsigned long long wait_ns = 1000000000ull;  // limit of the tensor-core chi kernels' pipeline waits
   // Content-keyed caches (hash_bytes over the bytes plus sizes).
@@ -284,6 +285,8 @@ int chi_run(Ctx* c, int prec, int nv, int nc, int ng, const void* M, const doubl
 // per chunk of digits, 0 to size it here (the size taken is returned).
 int chi_oz_run(Ctx* c, long long K, int ng, const void* M, const double* wr, const double2* wc, int nrow,
                double scale, int accumulate, void* chi, bool real, int* flags, long long* chunk, cudaStream_t st);
+// Bytes of digit planes and partial sums a Hermitian product of K pairs takes where nothing limits it.
+size_t chi_oz_bytes(Ctx* c, long long K, int ng);
 // The FP64 Sigma forms of K pairs (M [K][ng], W [ng][ng], sv = v^1/2) on the
 // tensor cores; *flag and the return value as chi_oz_run's.
 int sigma_oz_forms(Ctx* c, long long K, int ng, const void* M, const void* W, const double* sv, double* qW, double* qV,

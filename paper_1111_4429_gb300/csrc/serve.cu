@@ -45,6 +45,8 @@ struct Req {
   void* user_out = nullptr;   // caller's host eps~^-1 [ng][ng]
   bool user_pinned = false;
   uint64_t est = 0;           // admission estimate (bytes)
+  uint64_t extra = 0;         // FP64: what the tensor-core polarizability takes beyond it
+  uint64_t room = 0;          // the part of extra granted at admission
   enum State { kQueued, kRunning, kDone } state = kQueued;
   bgw_result res{};
   Clock::time_point t_submit, t_admit;
@@ -117,7 +119,10 @@ namespace {
 
 // Device bytes one request needs at most: coefficients, band grids and the
 // band z-pass intermediate, the pair intermediate, M, the chi operand planes,
-// workspace and weights, chi and eps~^-1 and the inverse's panels.
+// workspace and weights, chi and eps~^-1 and the inverse's panels.  FP64
+// requests run their polarizability on the tensor cores where the budget has
+// room for its digits (Req::extra) as well, in smaller chunks or by FP64 FMA
+// where it has not.
 size_t count_columns(const std::vector<int32_t>& g, int n) {
   std::set<int> cols;
   for (size_t i = 0; i + 2 < g.size(); i += 3) cols.insert((((g[i + 1] % n) + n) % n) * n + (((g[i] % n) + n) % n));
@@ -159,7 +164,7 @@ void finish(Server* s, Slot& sl, int status) {
   r->res.queue_ms = std::chrono::duration<double, std::milli>(r->t_admit - r->t_submit).count();
   r->res.hbm_bytes = r->est;
   r->state = Req::kDone;
-  s->in_use -= r->est;
+  s->in_use -= r->est + r->room;
   s->pinned_put(r->h_coef);
   s->pinned_put(r->h_out);
   r->h_coef = r->h_out = nullptr;
@@ -173,6 +178,7 @@ void finish(Server* s, Slot& sl, int status) {
 int launch(Server* s, Slot& sl) {
   Req& r = *sl.req;
   Ctx* c = &sl.ctx->impl;
+  c->digit_room = r.room;
   const size_t bcv = (size_t)r.nv * r.npw_v * 16, bcc = (size_t)r.nc * r.npw_c * 16;
   const size_t bout = (size_t)r.ng * r.ng * 16;
   int rc;
@@ -231,8 +237,15 @@ void worker_main(Server* s) {
       s->queue.pop_front();
       r->state = Req::kRunning;
       r->t_admit = Clock::now();
-      s->in_use += r->est;
       free_slot->req = r;
+      s->in_use += r->est;
+      // room for FP64 digits: what is left when the waiting requests that have a slot are in
+      uint64_t left = s->budget - s->in_use;
+      size_t idle = 0;
+      for (auto& sl : s->slots) idle += sl.req ? 0 : 1;
+      for (size_t k = 0; k < idle && k < s->queue.size(); ++k) left -= std::min(left, s->queue[k]->est);
+      r->room = std::min(r->extra, left);
+      s->in_use += r->room;
       lk.unlock();
       int rc = launch(s, *free_slot);
       if (rc != BGW_OK) {
@@ -321,6 +334,8 @@ int bgw_serve_submit(bgw_server* srv, const bgw_request* req, uint64_t* ticket) 
     }
   }
   r->est = bgw::estimate_bytes(*r, s->opts.prec);
+  if (s->opts.prec == BGW_PREC_FP64 && s->slots[0].ctx)
+    r->extra = bgw::chi_oz_bytes(&s->slots[0].ctx->impl, (long long)p.nv * p.nc, p.ng);
   r->t_submit = bgw::Clock::now();
   std::lock_guard<std::mutex> lk(s->mu);
   r->ticket = s->next_ticket++;

@@ -92,3 +92,33 @@ def test_over_budget_request_is_refused_and_queue_cancel():
         assert done[ts[-1]]["status"] == bgw.BGW_ECANCELED
     ref = _alone(small, bgw.BGW_PREC_MIX_FP16)
     assert _rel(outs[1], ref) <= 1e-6
+
+
+def test_fp64_requests_stay_within_the_budget():
+    """The device memory an FP64 server takes stays within its budget when the request's estimate leaves no room for the
+    tensor-core polarizability's digit planes (0.7 GB here), and the results are the same to FP64 accuracy."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1111_4429_gb300 import bgw
+    s = synth.make_system("b", a=17.0, fft=20, ecut_wfn=8.0, ecut_eps=4.4, nv=24, nc=1200, seed=77)
+    alone = _alone(s, bgw.BGW_PREC_FP64)   # also loads every kernel
+
+    def serve(budget):
+        torch.cuda.synchronize()
+        free0 = torch.cuda.mem_get_info()[0]
+        srv = bgw.Server(bgw.Context(0), hbm_budget_bytes=budget, max_slots=1, prec=bgw.BGW_PREC_FP64)
+        out = np.zeros((s.ng, s.ng), dtype=np.complex128)
+        t, r, free = srv.submit(s, out), None, free0
+        while r is None:   # the slot may give its scratch back when the request completes
+            free = min(free, torch.cuda.mem_get_info()[0])
+            r = srv.poll(t, timeout_ms=0)
+        srv.close()
+        used = free0 - free
+        return r, used, out
+
+    est = serve(1 << 20)[0]["hbm_bytes"]              # refused: reports the estimate
+    for budget in (est, est + (128 << 20), est + (4 << 30)):
+        r, used, out = serve(budget)
+        assert r["status"] == 0
+        assert used <= budget, (used, budget)
+        assert _rel(out, alone) <= 1e-12
