@@ -485,14 +485,9 @@ __global__ void sw_finish_kernel(const __grid_constant__ SweepBatch b) {
 static bool plain_default(Ctx* c) { return c->inverse_mode == -1 && !c->run_ff_chain; }
 static bool one_step(Ctx* c, int ngmax) { return plain_default(c) && ngmax <= NB; }
 bool fma_fallback(Ctx* c, int rc) {
-  const bool fma = plain_default(c) && rc == BGW_ENOMEM;
-  if (fma) c->err.clear();
-  if (fma || rc == BGW_OK) c->routes.note(fma ? 0 : 1);
-  return fma;
-}
-bool fma_before(Ctx* c) {
-  long long way = 1;
-  return c->routes.given(&way) && way == 0;
+  if (!plain_default(c) || rc != BGW_ENOMEM) return false;
+  c->err.clear();
+  return true;
 }
 
 // eps~ formation for every matrix of the batch, then the batched sweep.
@@ -546,7 +541,10 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
     const size_t upd_smem = sizeof(double2) * 2 * TU * (NB + 1);
     BGW_CUDA(c, cudaFuncSetAttribute(sw_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)upd_smem));
     std::unique_ptr<OzPlan, void (*)(OzPlan*)> oz(nullptr, oz_plan_delete);
-    if (tc_update && !one_step(c, ngmax) && !fma_before(c)) {
+    const bool tc = tc_update && !one_step(c, ngmax);
+    long long way = -1;   // sets of slices; 0: the FMA sweep
+    if (tc) c->routes.given(&way);
+    if (tc && way != 0) {
       oz.reset(oz_plan_new());
       std::vector<int> ngs(nb);
       std::vector<double2*> As(nb);
@@ -560,13 +558,14 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
         Ds[k] = sb.m[k].Dinv;
       }
       rc = oz_prepare(c, nb, ngs.data(), As.data(), Cs.data(), Ps.data(), Ds.data(), oz.get(), false, real_values,
-                      c->run_slices, c->run_ff_chain);
+                      c->run_slices, c->run_ff_chain, (int)way);
       if (fma_fallback(c, rc))
         oz.reset();
       else if (rc != BGW_OK)
         return rc;
       else
         oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
+      c->routes.note(oz ? oz_buffers(oz.get()) : 0);
     }
     if (!oz) {
       for (int k0 = 0; k0 < ngmax; k0 += NB) {
@@ -583,7 +582,8 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
       // runs on a high-priority side stream, while the main stream updates the
       // other tiles of the current step.  Dependencies:
       //   step k's chain waits for the main-stream update of step k-2 (same
-      //     slice buffer; tiles of block k may still be pending there);
+      //     slice buffer; tiles of block k may still be pending there), or of
+      //     step k-1 where there is one set of slices;
       //   step k's next-block update waits for the main-stream update of k-1;
       //   step k's main-stream update waits for step k's slices.
       if (!c->side) {
@@ -597,10 +597,12 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
       cudaEvent_t ev_rest[2] = {c->la_ev[2], c->la_ev[3]};
       BGW_CUDA(c, cudaEventRecord(ev_fork, st));
       BGW_CUDA(c, cudaStreamWaitEvent(s2, ev_fork, 0));
+      const bool one_set = oz_buffers(oz.get()) == 1;
       int k = 0;
       for (int k0 = 0; k0 < ngmax; k0 += NB, ++k) {
-        const int buf = k & 1;
-        if (k >= 2) BGW_CUDA(c, cudaStreamWaitEvent(s2, ev_rest[buf], 0));
+        const int par = k & 1, buf = one_set ? 0 : par;
+        if (k >= 2) BGW_CUDA(c, cudaStreamWaitEvent(s2, ev_rest[par], 0));
+        if (k >= 1 && one_set) BGW_CUDA(c, cudaStreamWaitEvent(s2, ev_rest[par ^ 1], 0));
         {
           TimedScope ts(c, kTSweepChain, s2);
           // the diagonal block of step k >= 1 was swept by step k-1's
@@ -609,7 +611,7 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
           if ((rc = oz_panel_slice(c, oz.get(), k0, ngmax, buf, s2)) != BGW_OK) return rc;
         }
         BGW_CUDA(c, cudaEventRecord(ev_slice, s2));
-        if (k >= 1) BGW_CUDA(c, cudaStreamWaitEvent(s2, ev_rest[buf ^ 1], 0));
+        if (k >= 1) BGW_CUDA(c, cudaStreamWaitEvent(s2, ev_rest[par ^ 1], 0));
         {
           TimedScope ts(c, kTOzAhead, s2);
           if ((rc = oz_update(c, oz.get(), k0, ngmax, buf, 1, s2)) != BGW_OK) return rc;
@@ -619,7 +621,7 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
           TimedScope ts(c, kTOzUpdate, st);
           if ((rc = oz_update(c, oz.get(), k0, ngmax, buf, 2, st)) != BGW_OK) return rc;
         }
-        BGW_CUDA(c, cudaEventRecord(ev_rest[buf], st));
+        BGW_CUDA(c, cudaEventRecord(ev_rest[par], st));
         BGW_CUDA(c, cudaGetLastError());
         c->launches += 4;
       }

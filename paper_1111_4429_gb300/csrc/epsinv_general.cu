@@ -553,7 +553,9 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
     }
     TimedScope ts(c, kTInverse, st);
     std::unique_ptr<OzPlan, void (*)(OzPlan*)> oz(nullptr, oz_plan_delete);
-    if (tc_update && !fma_before(c)) {
+    long long way = -1;   // sets of slices; 0: the FMA sweep
+    if (tc_update) c->routes.given(&way);
+    if (tc_update && way != 0) {
       oz.reset(oz_plan_new());
       std::vector<int> ngs(nb, n);
       std::vector<double2*> As(nb);
@@ -564,13 +566,14 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
         Cs[k] = Cp.as<double2>() + (size_t)k * kPB * n;
       }
       rc = oz_prepare(c, nb, ngs.data(), As.data(), Rs.data(), Cs.data(), nullptr, oz.get(), true, false,
-                      c->run_slices, c->run_ff_chain);
+                      c->run_slices, c->run_ff_chain, (int)way);
       if (fma_fallback(c, rc))
         oz.reset();
       else if (rc != BGW_OK)
         return rc;
       else
         oz_set_bulk_items(oz.get(), c->update_items);   // the option's width, else the SM-count rule
+      c->routes.note(oz ? oz_buffers(oz.get()) : 0);
     }
     int* sizes = oz && !c->run_ff_chain ? reinterpret_cast<int*>(static_cast<char*>(lu.ptr) + lu_bytes) : nullptr;
     int* piv = ipiv.as<int>();

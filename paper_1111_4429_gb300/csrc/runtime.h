@@ -300,10 +300,8 @@ int epsinv_batch_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* cel
                      const int32_t* const* d_geps, const void* const* chi, void* const* eps, void* const* epsinv,
                      cudaStream_t st, bool tc_update, bool real_values = false);
 // Whether the FMA sweep takes over an FP64 inverse whose tensor-core buffers
-// do not fit (rc from oz_prepare): under the default option only.  Notes the
-// way taken; fma_before: the direct run before this capture took the FMA sweep.
+// do not fit (rc from oz_prepare): under the default option only.
 bool fma_fallback(Ctx* c, int rc);
-bool fma_before(Ctx* c);
 // eps~ = I - sv chi sv of one matrix into A (and eps when non-NULL), sv from
 // the cell's Coulomb model (epsinv.cu).
 int eps_form_run(Ctx* c, const bgw_cell* cell, const int32_t* d_geps, int ng, const void* chi, double* sv,
@@ -363,8 +361,12 @@ void oz_plan_delete(OzPlan* p);
 // ff_chain: the next diagonal block and the panel product in double FP32
 // (about 2^-46), the FP64-level class of the seven-slice update, on the
 // FP32 pipe (GB300's FP64 pipe is 64 times slower); five slices imply it.
+// buffers: sets of slices as a run before took them (oz_buffers), or -1: two for
+// the Hermitian sweep, so that a step may slice while the update before it still
+// reads its own, one where two do not fit; one for the pivoted form.
 int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2* const* C, const double2* const* P,
-               double2* const* D, OzPlan* plan, bool general, bool real_values, int slices, bool ff_chain);
+               double2* const* D, OzPlan* plan, bool general, bool real_values, int slices, bool ff_chain, int buffers);
+int oz_buffers(const OzPlan* plan);
 // epsinv_batch_run with real_values: the matrices are real (imaginary parts zero).
 // Slices of one pivoted Gauss-Jordan step (general plans).
 int oz_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, const int* sizes, cudaStream_t st);

@@ -871,6 +871,7 @@ struct OzPlan {
   bool real_values = false;  // every matrix real (real flavor): only the real-part MMAs
   int bulk_narrow = -1;   // bulk items: -1 SM-count rule, 0 wide, 1 two column tiles
   int nmat = 0;
+  int buffers = 2;        // sets of slices
   int rows_total = 0;
   int max_tiles = 0;
   oz::OzBatch batch;
@@ -879,7 +880,7 @@ struct OzPlan {
 };
 
 int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2* const* C, const double2* const* P,
-               double2* const* D, OzPlan* plan, bool general, bool real_values, int slices, bool ff_chain) {
+               double2* const* D, OzPlan* plan, bool general, bool real_values, int slices, bool ff_chain, int buffers) {
   using namespace oz;
   if (slices != 5 && slices != 7) return fail(c, BGW_EINVAL, "tensor-core inverse: 5 or 7 slices");
   plan->slices = slices;
@@ -912,22 +913,31 @@ int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2
   plan->max_tiles = tiles;
   plan->U.pool = plan->V.pool = plan->sig.pool = plan->tau.pool = plan->dff.pool = &c->pool;
   int rc;
-  // two slice buffers: a step may slice while the previous step's update
-  // still reads its own
-  const size_t sb = (size_t)2 * S * rows * KR * sizeof(__half);
-  if ((rc = c->pool.alloc(sb, &plan->U.ptr)) != BGW_OK || (rc = c->pool.alloc(real_values ? sb : 2 * sb, &plan->V.ptr)) != BGW_OK ||
-      (rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &plan->sig.ptr)) != BGW_OK ||
-      (rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &plan->tau.ptr)) != BGW_OK ||
-      (rc = c->pool.alloc((size_t)nmat * NB * NB * sizeof(float4), &plan->dff.ptr)) != BGW_OK)
-    return fail(c, rc, "tensor-core inverse: slice buffers (%zu B) could not be allocated", 3 * sb);
+  // two sets of slices: a step may slice while the previous step's update still
+  // reads its own
+  for (plan->buffers = buffers > 0 ? buffers : general ? 1 : 2;; plan->buffers = 1) {
+    const size_t sb = (size_t)plan->buffers * S * rows * KR * sizeof(__half);
+    if ((rc = c->pool.alloc(sb, &plan->U.ptr)) == BGW_OK &&
+        (rc = c->pool.alloc(real_values ? sb : 2 * sb, &plan->V.ptr)) == BGW_OK &&
+        (rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &plan->sig.ptr)) == BGW_OK &&
+        (rc = c->pool.alloc((size_t)2 * rows * sizeof(int), &plan->tau.ptr)) == BGW_OK &&
+        (rc = c->pool.alloc((size_t)nmat * NB * NB * sizeof(float4), &plan->dff.ptr)) == BGW_OK)
+      break;
+    for (Scratch* x : {&plan->U, &plan->V, &plan->sig, &plan->tau, &plan->dff}) {
+      if (x->ptr) c->pool.release(x->ptr);
+      x->ptr = nullptr;
+    }
+    if (rc != BGW_ENOMEM || plan->buffers == 1)
+      return fail(c, rc, "tensor-core inverse: slice buffers (%zu B) could not be allocated", real_values ? 2 * sb : 3 * sb);
+  }
   for (int m = 0; m < nmat; ++m) plan->batch.m[m].Dff = plan->dff.as<float4>() + (size_t)m * NB * NB;
-  cuuint64_t gdim[2] = {(cuuint64_t)KR, (cuuint64_t)2 * S * rows};
+  cuuint64_t gdim[2] = {(cuuint64_t)KR, (cuuint64_t)plan->buffers * S * rows};
   cuuint64_t gstride[1] = {(cuuint64_t)KR * sizeof(__half)};
   cuuint32_t estr[2] = {1, 1};
   cuuint32_t ubox[2] = {(cuuint32_t)KR, (cuuint32_t)BM};
   // 16 columns of two rows each (vrow); real values: 32 of one
   cuuint32_t vbox[2] = {(cuuint32_t)KR, (cuuint32_t)BN};
-  cuuint64_t vdim[2] = {(cuuint64_t)KR, (cuuint64_t)(real_values ? 2 : 4) * S * rows};
+  cuuint64_t vdim[2] = {(cuuint64_t)KR, (cuuint64_t)(real_values ? 1 : 2) * plan->buffers * S * rows};
   if (encode(&plan->umap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plan->U.ptr, gdim, gstride, ubox, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
@@ -1083,6 +1093,8 @@ int oz_update(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, int mode, cudaSt
   BGW_CUDA(c, cudaGetLastError());
   return BGW_OK;
 }
+
+int oz_buffers(const OzPlan* plan) { return plan->buffers; }
 
 void oz_set_bulk_items(OzPlan* plan, int narrow) { plan->bulk_narrow = narrow < 0 ? -1 : (narrow ? 1 : 0); }
 
