@@ -160,7 +160,7 @@ int validate_mtxel(Ctx* c, const bgw_cell* cell, int nv, int npw_v, const int32_
                   mv[d], mc[d], me[d]);
     need.points = std::max(need.points, mv[d] + mc[d] + me[d] + 1);
   }
-  *n_out = transform_grid(n, need, ng, geps);
+  *n_out = transform_grid(n, need, ng, geps, prec != BGW_PREC_FP64);
   return BGW_OK;
 }
 
@@ -1070,7 +1070,7 @@ int bgw_sigma_cohsex(bgw_ctx* ctx, const bgw_cell* cell, int no, int npw_o, cons
     int tmp[3];
     if ((rc = check_glist(c, "-geps", ng, neg.data(), n, tmp, &need)) != BGW_OK) return rc;
   }
-  n = transform_grid(n, need, ng, neg.data());
+  n = transform_grid(n, need, ng, neg.data(), prec != BGW_PREC_FP64);
   const BandPlan *bpo, *bpi;
   const PairPlan* pp;
   if ((rc = get_band_plan(c, n, npw_o, go, st, &bpo)) != BGW_OK) return rc;

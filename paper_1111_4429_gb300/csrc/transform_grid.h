@@ -24,27 +24,35 @@ struct GridNeed {
 // wider than the other's, even though nothing kept aliases).
 inline bool grid_serves(int s, const GridNeed& g) { return s >= g.points && g.lo >= -(s / 2) && g.hi < s - s / 2; }
 
+// Whether the pair transform's low-band lines run on a grid of s points: every
+// kept frequency in the outer quarters, [-s/4, s/4).
+inline bool grid_lowband(int s, int ng, const int32_t* geps) {
+  if (s % 4) return false;
+  for (int i = 0; i < 3 * ng; ++i)
+    if (geps[i] < -(s / 4) || geps[i] >= s / 4) return false;
+  return true;
+}
+
 // Any grid that serves gives the coefficients of the product itself, so the
 // transforms run on the smallest such supported grid instead of the caller's
-// (often a density grid, near twice the size needed).  Measured per pair
-// (y,x passes + z pass, us): spheres that need 30 points, FP32 40^3 0.139,
-// 32^3 0.080; FP64 3.70 and 1.71; spheres that need 44, FP32 60^3 0.553,
-// 48^3 0.266.  The smallest is the fastest but for 30, where 32 allows the
-// low-band lines (every kept frequency in [-8, 8)): FP32 0.096 against 0.080,
-// FP64 1.93 against 1.71.  Lines of 36 and 50 points without the low band
-// still beat low-band lines of 40 and 60.
-inline int transform_grid(int n, const GridNeed& g, int ng, const int32_t* geps) {
+// (often a density grid, near twice the size needed).  4096 pairs, us a call in
+// FP32 / FP64 (FP64 from 38 points on: 1024 pairs), spheres that need 8 points, 8^3
+// 39 / 142, 16^3 67 / 716; need 14, 16^3 79 / 803, 20^3 117 / 1902; need 22, 24^3 203
+// / 3379, 32^3 318 / 6905; need 31, 32^3 491 / 8535, 36^3 563 / 12793; need 38, 40^3
+// 762 / 4856, 48^3 1024 / 7360; need 45, 48^3 2053 / 9159, 60^3 2161 / 17336.  A grid
+// without the low-band lines is still the faster one (12 against 16, 20 against
+// 24, 24 against 32, 36 against 40, 48 against 60) but for three: 30 (441 / 8387; 32:
+// 361 / 7388), 50 in FP32 (need 49, N_G 2109 2071, 7153 2470; 60: 1902, 2231; FP64
+// 11254 against 15557), and 60 where 64 has them (3895 / 19736 against 3037 / 18224).
+inline int transform_grid(int n, const GridNeed& g, int ng, const int32_t* geps, bool fp32) {
   int m = n;
   for (int s : kSupportedN)
     if (grid_serves(s, g)) {
       m = std::min(m, s);
       break;
     }
-  if (m == 30 && n >= 32) {
-    for (int i = 0; i < 3 * ng; ++i)
-      if (geps[i] < -8 || geps[i] >= 8) return m;
-    m = 32;
-  }
+  const int up = m == 30 ? 32 : m == 50 && fp32 ? 60 : m == 60 ? 64 : m;
+  if (up > m && up <= n && !grid_lowband(m, ng, geps) && grid_lowband(up, ng, geps)) m = up;
   return m;
 }
 

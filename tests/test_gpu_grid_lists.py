@@ -41,6 +41,27 @@ def test_elements(v, c, e, n, prec, tol):
     assert np.array_equal(runs[0], runs[1])
 
 
+# the grids that the next one with low-band lines replaces: 50 by 60 (FP32), 60 by 64
+@pytest.mark.parametrize("w,e,n", [(18, 12, 60), (18, 12, 50), (21, 15, 64), (21, 15, 60), (20, 14, 64)])
+@pytest.mark.parametrize("prec,tol", [(0, 1e-12), (1, 1e-5)])
+def test_low_band_neighbours(w, e, n, prec, tol):
+    from paper_1111_4429_gb300 import bgw
+    rng = np.random.default_rng(w + e)
+
+    def some(r, keep):
+        g = rng.integers(-r, r + 1, (keep, 3))
+        return np.unique(np.concatenate([g, [[r, -r, 0], [-r, r, r], [0, 0, -r]]]), axis=0).astype(np.int32)
+    gv, gc, ge = some(w, 300), some(w, 300), some(e, 200)
+    cv, cc = _bands(rng, 5, gv), _bands(rng, 4, gc)
+    ctx = bgw.Context(0)
+    M = torch.full((20, len(ge)), float("nan"), dtype=torch.complex128 if prec == 0 else torch.complex64, device="cuda")
+    ctx.mtxel(bgw.make_cell(np.eye(3) * 0.3, 8641.0, (0.1, 0.0, 0.0), n), gv, torch.from_numpy(cv).cuda(), gc,
+              torch.from_numpy(cc).cuda(), ge, prec, M)
+    ctx.sync()
+    ref = oracle.mtxel_direct(gv, cv, gc, cc, ge)
+    assert np.linalg.norm(M.cpu().numpy().reshape(ref.shape) - ref) <= tol * np.linalg.norm(ref)
+
+
 @pytest.mark.parametrize("o,i,e,n", [((-1, 1), (-1, 1), (-4, 4), 20), ((-1, 1), (-6, 6), (-2, 2), 20)])
 def test_sigma(o, i, e, n):
     from paper_1111_4429_gb300 import bgw

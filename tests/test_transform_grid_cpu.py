@@ -15,12 +15,12 @@ SIZES = (8, 10, 12, 16, 20, 24, 30, 32, 36, 40, 48, 50, 60, 64)
 
 SHIM = r'''
 #include "transform_grid.h"
-extern "C" int pick(int n, int points, int lo, int hi, int ng, const int32_t* geps) {
+extern "C" int pick(int n, int points, int lo, int hi, int ng, const int32_t* geps, int fp32) {
   bgw::GridNeed g;
   g.points = points;
   g.lo = lo;
   g.hi = hi;
-  return bgw::transform_grid(n, g, ng, geps);
+  return bgw::transform_grid(n, g, ng, geps, fp32 != 0);
 }
 '''
 
@@ -37,12 +37,12 @@ def pick(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     lib = ctypes.CDLL(str(d / "shim.so"))
 
-    def call(n, gv, gc, ge):
+    def call(n, gv, gc, ge, fp32=0):
         points = int((np.abs(gv).max(0) + np.abs(gc).max(0) + np.abs(ge).max(0)).max()) + 1
         every = np.concatenate([gv, gc, ge])
         buf = np.ascontiguousarray(ge, dtype=np.int32)
         return lib.pick(n, points, min(0, int(every.min())), max(0, int(every.max())), len(ge),
-                        buf.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)))
+                        buf.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), fp32)
     return call
 
 
@@ -76,7 +76,18 @@ def _check(m, n, lists):
 def test_wide_lists(pick, bands, other, eps, n):
     lists = [_list([r[0]] * 3, [r[1]] * 3) for r in (bands, other, eps)]
     assert _accepted(n, *lists)
-    _check(pick(n, *lists), n, lists)
+    for fp32 in (0, 1):
+        _check(pick(n, *lists, fp32), n, lists)
+
+
+# the next grid has the low-band lines and the smallest one has not
+@pytest.mark.parametrize("w,e,n,fp64,fp32", [(11, 7, 40, 32, 32), (11, 7, 30, 30, 30), (10, 8, 40, 30, 30),
+                                             (18, 12, 60, 50, 60), (18, 12, 50, 50, 50), (17, 15, 64, 50, 50),
+                                             (20, 14, 64, 60, 60), (21, 15, 64, 64, 64), (21, 15, 60, 60, 60),
+                                             (13, 9, 64, 36, 36), (16, 12, 64, 48, 48)])
+def test_low_band_neighbours(pick, w, e, n, fp64, fp32):
+    lists = [_list([-r] * 3, [r] * 3) for r in (w, w, e)]
+    assert (pick(n, *lists, 0), pick(n, *lists, 1)) == (fp64, fp32)
 
 
 def test_random_boxes(pick):
@@ -91,4 +102,4 @@ def test_random_boxes(pick):
         if not _accepted(n, *lists):
             continue
         done += 1
-        _check(pick(n, *lists), n, lists)
+        _check(pick(n, *lists, done & 1), n, lists)
