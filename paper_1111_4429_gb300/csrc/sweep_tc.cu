@@ -45,41 +45,14 @@ constexpr int KR = 64;           // real inner length (32 complex)
 constexpr int NB = 32;           // sweep block width
 constexpr int kUTile = BM * KR * 2;    // 16 KiB
 constexpr int kVTile = BN * KR * 2;    // 4 KiB
-constexpr unsigned long long kWaitNs = 1000000000ull;
+using tc::globaltimer;
+using tc::kWaitNs;
+using tc::mbar_try_wait;
+using tc::mbar_wait;
+using tc::mma;
+using tc::smem_u32;
+using tc::tma_load_2d;
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  while (!mbar_try_wait(bar, parity))
-    if (globaltimer() - t0 > kWaitNs) return false;
-  return true;
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::
-          "r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
-      : "memory");
-}
 // K-major operand, 128-byte swizzle: rows of 128 bytes, 8-row groups 1024
 // bytes apart.
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
@@ -91,21 +64,8 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   d |= (uint64_t)2u << 61;  // SWIZZLE_128B
   return d;
 }
-__host__ __device__ constexpr uint32_t idesc(bool neg_a, int n = BN) {
-  return (1u << 4) | ((neg_a ? 1u : 0u) << 13) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-}
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(id), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(taddr));
+__host__ __device__ constexpr uint32_t idesc(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 // 16 lanes x 256 bits: register pair (0, 1) holds lane base + l / 4, columns
 // 2 (l % 4) and 2 (l % 4) + 1; pair (2, 3) the same columns of lane base + 8 + l / 4.
@@ -113,18 +73,6 @@ __device__ __forceinline__ void tmem_ld16x256(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
 }
 
 // Per-matrix description of one batched sweep (device pointers).
@@ -428,18 +376,6 @@ constexpr int kPipeThreads = (kPipeEpiWarps + 1) * 32;
 static_assert(kPipeThreads == kDiagThreads, "the look-ahead CTA sweeps the next diagonal block");
 constexpr int kVRing = 2;              // V units in flight
 
-
-// Bounded wait that also gives up when the CTA aborts.
-__device__ __forceinline__ bool mbar_wait_ab(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  while (!mbar_try_wait(bar, parity)) {
-    if (*abort_flag) return false;
-    if (globaltimer() - t0 > kWaitNs) return false;
-  }
-  return true;
-}
-
 // A segment's seven level sums (integers below 2^23.2 in FP32) joined in units
 // of 2^-55: adjacent levels in 32 bits, the rest in 64.
 __device__ __forceinline__ long long join_levels(const uint32_t (&x)[7][4], int q) {
@@ -561,7 +497,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
       if (lane == 0 && nt > 0 && !*abort_flag) {
         // U slices of the row tile, once the previous item's MMAs have read
         // the last ones (its epilogue may still run: items are independent)
-        bool ok = u_loads == 0 || mbar_wait_ab(u_empty, (u_loads - 1) & 1, abort_flag);
+        bool ok = u_loads == 0 || mbar_wait(u_empty, (u_loads - 1) & 1, abort_flag);
         const int u_phase = u_loads & 1;
         if (ok) {
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(u_full)),
@@ -575,7 +511,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
         const int uu0 = UN * t, uu1 = UN * (t + nt);
         auto issue_v = [&](int uu) {
           const int bq = uu % kVRing;
-          if (uu >= kVRing && !mbar_wait_ab(&v_empty[bq], (uu / kVRing - 1) & 1, abort_flag)) return false;
+          if (uu >= kVRing && !mbar_wait(&v_empty[bq], (uu / kVRing - 1) & 1, abort_flag)) return false;
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(v_full + bq)),
                        "r"((uint32_t)(SL * kVTile))
                        : "memory");
@@ -594,9 +530,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
           }
           const int tt = uu / UN, bq = uu % kVRing;
           const int acc = realv ? tt & 1 : uu & 1, use = realv ? tt >> 1 : tt;   // accumulators, and how often used before
-          if ((uu == uu0 && !mbar_wait_ab(u_full, u_phase, abort_flag)) ||
-              !mbar_wait_ab(&v_full[bq], (uu / kVRing) & 1, abort_flag) ||
-              (use > 0 && !mbar_wait_ab(&t_empty[acc], (use - 1) & 1, abort_flag))) {
+          if ((uu == uu0 && !mbar_wait(u_full, u_phase, abort_flag)) ||
+              !mbar_wait(&v_full[bq], (uu / kVRing) & 1, abort_flag) ||
+              (use > 0 && !mbar_wait(&t_empty[acc], (use - 1) & 1, abort_flag))) {
             ok = false;
             break;
           }
@@ -615,7 +551,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
           for (int a = 0; a < SL; ++a) {
             const uint32_t d = tmem + (acc * SL + a) * 32;
             const uint64_t ua = du + (uint64_t)((a * kUTile) >> 4);
-            const uint32_t id = idesc(false, 32 * (SL - a));
+            const uint32_t id = idesc(32 * (SL - a));
             // byte offsets 32 q along K: +2 q in the descriptor; real values fill the first half of the row
 #pragma unroll
             for (int q = 0; q < (realv ? 2 : 4); ++q) mma(d, ua + 2 * q, dv + 2 * q, id, a == 0 && q == 0 ? 0u : 1u);
@@ -743,7 +679,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)   // 17 warps: at most 5 per 
         // the next tile's column exponents, used after this tile
         int tnext[2];
         if constexpr (!realv) load_tau(k + 1, c0, tnext);
-        have = mbar_wait_ab(&t_full[group], (realv ? tt >> 1 : tt) & 1, abort_flag);
+        have = mbar_wait(&t_full[group], (realv ? tt >> 1 : tt) & 1, abort_flag);
         have = __all_sync(0xffffffffu, have) != 0;
         if (have) {
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -873,7 +809,6 @@ struct OzPlan {
   int nmat = 0;
   int buffers = 2;        // sets of slices
   int rows_total = 0;
-  int max_tiles = 0;
   oz::OzBatch batch;
   CUtensorMap umap, vmap;
   Scratch U, V, sig, tau, dff;
@@ -892,7 +827,7 @@ int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2
   plan->general = general;
   plan->real_values = real_values;
   plan->batch.n = nmat;
-  int rows = 0, tiles = 0;
+  int rows = 0;
   for (int m = 0; m < nmat; ++m) {
     plan->batch.m[m].A = A[m];
     plan->batch.m[m].C = C[m];
@@ -901,16 +836,8 @@ int oz_prepare(Ctx* c, int nmat, const int* ng, double2* const* A, const double2
     plan->batch.m[m].ng = ng[m];
     plan->batch.m[m].row_off = rows;
     rows += (ng[m] + BM - 1) / BM * BM;
-    const int nI = (ng[m] + BM - 1) / BM, nJ = (ng[m] + BN - 1) / BN;
-    int t = 0;
-    if (general)
-      t = nI * nJ;
-    else
-      for (int I = 0; I < nI; ++I) t += std::min(4 * I + 4, nJ);
-    tiles = std::max(tiles, t);
   }
   plan->rows_total = rows;
-  plan->max_tiles = tiles;
   plan->U.pool = plan->V.pool = plan->sig.pool = plan->tau.pool = plan->dff.pool = &c->pool;
   int rc;
   // two sets of slices: a step may slice while the previous step's update still
@@ -1009,13 +936,7 @@ int oz_panel_slice(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, cudaStream_
 // runs mode 3 (every tile) and then writes R into the block's rows.
 int oz_update(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, int mode, cudaStream_t st) {
   using namespace oz;
-  int grid = plan->max_tiles;
-  if (mode == 1) {
-    const int k1 = k0 + NB;
-    if (k1 >= ngmax) return BGW_OK;
-    const int nI = (ngmax + BM - 1) / BM, nJ = (ngmax + BN - 1) / BN, In = k1 / BM;
-    grid = std::min(4 * In + 4, nJ) + std::max(0, nI - In - 1);
-  }
+  if (mode == 1 && k0 + NB >= ngmax) return BGW_OK;
   if (plan->general) mode = 3;
   // Column tiles per bulk work item: 4 with seven slices, 3 with five; 2
   // where those items would not exceed the SMs (each CTA then pipelines two
@@ -1023,7 +944,7 @@ int oz_update(Ctx* c, OzPlan* plan, int k0, int ngmax, int buf, int mode, cudaSt
   // 3.10 -> 2.95 ms per inverse, while at 7180 items of 4 stay best), unless
   // the plan fixes the width (the context's timed choice or its option).
   const int nsm = sm_count(c);
-  int wide = plan->slices < 7 ? 3 : kJPI;
+  int wide = plan->slices < 7 ? 3 : kJPI, grid;
   {
     // the most items of a matrix that has not finished: a smaller one at its
     // last step has items (no next row tile to leave out) where the largest
