@@ -215,12 +215,14 @@ def flops_of(s):
 
 def _set_inverse_options(ctx, prec):
     from paper_1111_4429_gb300 import bgw
-    # the mixed precisions invert with the tensor-core trailing update (seven
-    # slices, the sweep's critical chain in double FP32), the plain path with
-    # FP64 FMA, as bgw_epsilon does
-    ctx.set_option(bgw.BGW_OPT_INVERSE, 0 if prec == bgw.BGW_PREC_FP64 else 1)
-    ctx.set_option(bgw.BGW_OPT_UPDATE_SLICES, 0 if prec == bgw.BGW_PREC_FP64 else UPDATE_SLICES_MIXED)
-    ctx.set_option(bgw.BGW_OPT_DOUBLE_FP32, 0 if prec == bgw.BGW_PREC_FP64 else 1)
+    # as bgw_epsilon does: the mixed precisions invert with the tensor-core
+    # trailing update (seven slices, the sweep's critical chain in double
+    # FP32), the plain path with the defaults (the update's level sums joined
+    # in integers, the chain in FP64)
+    plain = prec == bgw.BGW_PREC_FP64
+    ctx.set_option(bgw.BGW_OPT_INVERSE, -1 if plain else 1)
+    ctx.set_option(bgw.BGW_OPT_UPDATE_SLICES, 0 if plain else UPDATE_SLICES_MIXED)
+    ctx.set_option(bgw.BGW_OPT_DOUBLE_FP32, -1 if plain else 1)
 
 
 def _reset_inverse_options(ctx):
@@ -300,10 +302,10 @@ def _solve_steps(ctx, s, prec, steps, warmup, flush, timing, nc_chunk=None, timi
     return np.array(stage), kt, chi, inv, launches
 
 
-def _roofline(s, kt, step_ms, peaks, peak_src, size_tag="c2"):
+def _roofline(s, kt, step_ms, peaks, peak_src, size_tag="c2", fp64=False):
     """Roofline of the kernel group with the largest time per step (kt:
     kernel group -> (launches per step, ms per step)); size_tag names the
-    workload in the profiles' traffic records."""
+    workload in the profiles' traffic records; fp64: a plain FP64 solve's."""
     per_step_ms = {k: v[1] for k, v in kt.items() if k != "inverse"}
     if "inverse" in kt and "oz_update" not in kt:
         per_step_ms["inverse"] = kt["inverse"][1]
@@ -312,7 +314,20 @@ def _roofline(s, kt, step_ms, peaks, peak_src, size_tag="c2"):
     bf16 = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
     n_launch, ms = kt[dom]
     t_launch = ms / 1e3 / n_launch
-    if dom == "chi_tc":
+    if dom == "chi_tc" and fp64:
+        # lower tiles of 128x32; per 16 pairs 36 digit products of four real 128x32x16 MMAs each
+        nj = (s.ng + 31) // 32
+        tiles = sum(min(4 * i + 4, nj) for i in range((s.ng + 127) // 128))
+        issued = tiles * 36 * 4 * 2.0 * 128 * 32 * ((s.npairs + 15) // 16 * 16)
+        roof = {"bound": "tensor", "kernel": "oz64::gemm_kernel (tcgen05 kind::f16 M128 N32..256, exact products of "
+                                             "7-bit digits)",
+                "achieved": issued / n_launch / t_launch / 1e12, "peak": bf16, "unit": "TFLOP/s",
+                "algorithmic": "issued tensor flops: 36 digit products of 4 x 2x128x32x16 per lower 128x32 tile and 16 "
+                               f"pairs over {n_launch:.0f} launches per step",
+                "peak_source": f"{peak_src} bf16 sustained",
+                "fp64_equivalent_tflops": fl["chi_herm"] / n_launch / t_launch / 1e12,
+                "launch_ms": t_launch * 1e3, "traffic_tag": "chi_digits"}
+    elif dom == "chi_tc":
         # per launch: one chunk of pairs; algorithmic = the Hermitian product
         # 4 N_G^2 K (complex multiply-adds of the lower triangle, 8 flop per
         # complex multiply-add counted once per G >= G' pair ... as 4 N_G^2 K);
@@ -354,14 +369,15 @@ def _roofline(s, kt, step_ms, peaks, peak_src, size_tag="c2"):
                 "fp64_pipe_peak_tflops": FP64_PEAK_TFLOPS,
                 "launch_ms": t_launch * 1e3, "traffic_tag": "oz_update"}
     elif dom in ("pair_yxpass", "pair_zgather", "band_transform"):
-        roof = {"bound": "alu", "kernel": f"{dom} (FP32 FFT passes of the matrix elements)",
+        roof = {"bound": "alu", "kernel": f"{dom} ({'FP64' if fp64 else 'FP32'} FFT passes of the matrix elements)",
                 "achieved": fl["mtxel"] / (sum(kt[k][1] for k in ("pair_yxpass", "pair_zgather", "band_transform")
                                                if k in kt) / 1e3) / 1e12,
-                "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
+                "peak": FP64_PEAK_TFLOPS if fp64 else FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "algorithmic": "pruned FFT flops of all matrix-element passes per step on the caller's grid "
                                "(5 n log2 n per line; the transform runs on a smaller alias-free one)",
-                "peak_source": "derived: 152 SM x 128 FP32 lanes x 2 x 2.07 GHz",
-                "launch_ms": t_launch * 1e3, "traffic_tag": dom}
+                "peak_source": "derived: 152 SM x 2 FP64 FMA/clk x 2 x 2.07 GHz" if fp64 else
+                               "derived: 152 SM x 128 FP32 lanes x 2 x 2.07 GHz",
+                "launch_ms": t_launch * 1e3, "traffic_tag": None if fp64 else dom}
     elif dom == "chi_f64":
         roof = {"bound": "alu", "kernel": "chi_f64_kernel (FP64 FMA)",
                 "achieved": fl["chi_herm"] / n_launch / t_launch / 1e12, "peak": FP64_PEAK_TFLOPS,
@@ -412,11 +428,11 @@ def run_ours(args):
     _, kt, _, _, _ = _solve_steps(ctx, s, prec, 1, 1, flush, timing=True, nc_chunk=NC_CHUNK,
                                   timing_steps=min(3, args.steps))
     kms = {k: v[1] for k, v in kt.items()}
-    roof = _roofline(s, kt, step_ms, peaks, peak_src)
+    roof = _roofline(s, kt, step_ms, peaks, peak_src, fp64=prec == bgw.BGW_PREC_FP64)
 
     # error against the FP64 oracle: the seeded 256 x 256 principal subblock
     # of chi and eps~^-1 (tests/golden, written by a script that runs only the
-    # oracle) -- the plain FP64 GPU solve of this size takes about a minute
+    # oracle)
     golden = None
     gpath = os.path.join(ROOT, "tests", "golden", "c2_oracle.npz")
     if os.path.exists(gpath) and prec != bgw.BGW_PREC_FP64:
@@ -551,7 +567,9 @@ def run_c1(ctx, prec, flush, args, steps=5, warmup=2):
                            "stage_ms": {"mtxel": m64[0], "chi_sum": m64[1], "epsinv": m64[2]},
                            "chi_tflops_zgemm_eq": fl["chi_zgemm"] / (m64[1] / 1e3) / 1e12,
                            "chi_tflops_hermitian": fl["chi_herm"] / (m64[1] / 1e3) / 1e12,
-                           "kernel_ms_per_step": {k: v[1] for k, v in kt64.items()}},
+                           "kernel_ms_per_step": {k: v[1] for k, v in kt64.items()},
+                           "roofline": _roofline(s, kt64, float(st64.sum(1).mean()), peaks, peak_src, size_tag="c1",
+                                                 fp64=True)},
             "mixed_over_plain_fp64": float(st64.sum(1).mean() / st.sum(1).mean()),
             "epsinv_rel_err_vs_plain_fp64_gpu": err}
 
@@ -1086,9 +1104,7 @@ def run_profile_case(args):
         s = synth.config_system("c1", nc=200) if case == "solve" else synth.config_system("c2", nc=100)
         cell = bgw.system_cell(s)
         prec = bgw.PREC[args.prec]
-        ctx.set_option(bgw.BGW_OPT_INVERSE, 0 if prec == bgw.BGW_PREC_FP64 else 1)
-        ctx.set_option(bgw.BGW_OPT_UPDATE_SLICES, 0 if prec == bgw.BGW_PREC_FP64 else UPDATE_SLICES_MIXED)
-        ctx.set_option(bgw.BGW_OPT_DOUBLE_FP32, 0 if prec == bgw.BGW_PREC_FP64 else 1)
+        _set_inverse_options(ctx, prec)
         cv = torch.from_numpy(s.cv).cuda()
         cc = torch.from_numpy(s.cc).cuda()
         M = torch.empty((s.npairs, s.ng), dtype=torch.complex128 if prec == 0 else torch.complex64, device="cuda")
