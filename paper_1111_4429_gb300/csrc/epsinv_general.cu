@@ -529,13 +529,11 @@ int epsinv_general_run(Ctx* c, int nmat, const int* ng, const bgw_cell* const* c
     return fail(c, rc, "general inverse: scratch allocation failed");
   const size_t psmem = sizeof(float2) * kTRows * (kPB + 1);
   const size_t ssmem = sizeof(double2) * 2 * kPB * kSwapCols;
-  BGW_CUDA(c, cudaFuncSetAttribute(pivot_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
-  BGW_CUDA(c, cudaFuncSetAttribute(pivot_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
-  BGW_CUDA(c, cudaFuncSetAttribute(pivot_swap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
-  BGW_CUDA(c, cudaFuncSetAttribute(colperm_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(2 * sizeof(int) * ngmax)));
-  BGW_CUDA(c, cudaFuncSetAttribute(colperm_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(sizeof(double2) * ngmax)));
+  BGW_CUDA(c, allow_smem(reinterpret_cast<const void*>(pivot_leaf_kernel), psmem));
+  BGW_CUDA(c, allow_smem(reinterpret_cast<const void*>(pivot_merge_kernel), psmem));
+  BGW_CUDA(c, allow_smem(reinterpret_cast<const void*>(pivot_swap_kernel), ssmem));
+  BGW_CUDA(c, allow_smem(reinterpret_cast<const void*>(colperm_build_kernel), 2 * sizeof(int) * ngmax));
+  BGW_CUDA(c, allow_smem(reinterpret_cast<const void*>(colperm_apply_kernel), sizeof(double2) * ngmax));
   int* cbuf[2] = {cand.as<int>(), cand.as<int>() + (size_t)kGB * cstride};
   // Matrices of equal size are stepped together, up to kGB at a time: every
   // launch below serves the whole group.

@@ -404,8 +404,7 @@ __global__ void __launch_bounds__(256) pair_zgather(const cpx<T>* __restrict__ T
 // ------------------------------------------------------------ launchers
 template <typename K>
 static cudaError_t set_smem(K kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return allow_smem(reinterpret_cast<const void*>(kernel), bytes);
 }
 
 // Shared memory and threads of a pair_yxpass block holding ppb pairs.

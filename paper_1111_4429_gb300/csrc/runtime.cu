@@ -4,6 +4,10 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <map>
+#include <mutex>
+#include <utility>
+
 #include "runtime.h"
 
 namespace bgw {
@@ -60,6 +64,21 @@ int cuda_fail(Ctx* c, cudaError_t e, const char* what) {
     return fail(c, BGW_ENOMEM, "%s: %s", what, cudaGetErrorString(e));
   }
   return fail(c, BGW_ECUDA, "%s: %s", what, cudaGetErrorString(e));
+}
+
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> allowed;
+  if (bytes <= 48 * 1024) return cudaSuccess;   // every kernel's own limit
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  size_t& top = allowed[{dev, kernel}];
+  if (bytes <= top) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) top = bytes;
+  return e;
 }
 
 int sm_count(Ctx* c) {

@@ -207,6 +207,11 @@ int fail(Ctx* c, int code, const char* fmt, ...);
 int cuda_fail(Ctx* c, cudaError_t e, const char* what);
 // Streaming multiprocessors of the context's device (152 if the query fails).
 int sm_count(Ctx* c);
+// Lets `kernel` take up to `bytes` of dynamic shared memory on the current
+// device.  The limit is the kernel's, shared by every context and thread, and
+// only ever grows: setting each launch's own size would let one thread lower
+// it between another's setting and launch.
+cudaError_t allow_smem(const void* kernel, size_t bytes);
 #define BGW_CUDA(c, expr)                                    \
   do {                                                       \
     cudaError_t _e = (expr);                                 \
