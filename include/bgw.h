@@ -64,7 +64,13 @@ enum {
 /* Precision of a call.
  *  BGW_PREC_FP64     : every step to FP64 accuracy / complex128 (the plain
  *                      path; chi and the inverse's updates as exact digit
- *                      products on the tensor cores).
+ *                      products on the tensor cores).  chi: an operand
+ *                      M |w|^1/2 is held to 2^-57 of its G column's largest
+ *                      entry; relative to (chi_GG chi_G'G')^1/2 the error is
+ *                      below that of running FP64 sums, and pairs whose
+ *                      largest operands spread by more than 2^8 go to FP64
+ *                      FMA, so a block of chi that small pairs alone make
+ *                      errs by at most about 4e-15 of itself.
  *  BGW_PREC_MIX_FP16 : M in complex64 (FP32 FFTs); chi on the tensor cores
  *                      as split FP16 (hi*hi + hi*lo + lo*hi) products with
  *                      FP32 accumulation, flushed into an FP64 chi per call;
@@ -171,10 +177,15 @@ int bgw_graph_stats(bgw_ctx* ctx, uint64_t* graphs, uint64_t* replays);
  *    into 8-bit slices held exactly in FP16 (seven or five,
  *    BGW_OPT_UPDATE_SLICES) and accumulates every slice product exactly in
  *    FP32.  FP64 inputs (BGW_PREC_FP64, bgw_epsinv*) join the exact sums in
- *    integers and round once, with errors below those of FP64 FMA; the mixed
- *    precisions combine them in double-FP32 (with seven slices near 2^-48 of
- *    the update's scale).  -1 falls back to FP64 FMA for FP64 inputs whose
- *    slice buffers do not fit the budget.                                  */
+ *    integers and round once.  Their entries, the inner indices balanced by
+ *    powers of two, are held to 2^-57 of the largest of their row, and an
+ *    update of (i, j) errs by about 2^-55 of the product of the two rows'
+ *    largest (2^-49 at worst); the inverses measured (flat and graded
+ *    diagonals) are as close to the exact ones as FP64 FMA's.  The mixed
+ *    precisions combine the sums in double-FP32 (with seven slices near 2^-48
+ *    of the update's scale).  Two sets of slices are taken, one where two do
+ *    not fit the budget; -1 falls back to FP64 FMA for FP64 inputs for which
+ *    one does not fit either.                                              */
 /*  BGW_OPT_HEAD: the q0 head of the mixed precisions.  At a small q0 the
  *    head column M_vc(G = 0) is O(|q0|) while v(q0) = 4 pi / |q0|^2, so the
  *    FP32 FFTs' absolute error on it (near 2^-24 |M|) becomes a relative
@@ -209,8 +220,9 @@ int bgw_graph_stats(bgw_ctx* ctx, uint64_t* graphs, uint64_t* replays);
 /*  BGW_OPT_PAIR_KERNEL: which kernel runs the pair transform's y and x
  *    passes.  -1 (default): the autotuner's choice (or the fixed default
  *    while BGW_OPT_AUTOTUNE is 0); 0: one (pair block, plane) per CTA with
- *    the default pairs per block; 1: one warp per pair, where every kept
- *    frequency lies in |k| < N/4 (elsewhere 0 runs).  The results agree to
+ *    the default pairs per block; 1: one warp per pair (or per two pairs, on
+ *    36, 40 and 48 points with enough pairs), where every kept frequency lies
+ *    in |k| < N/4 (elsewhere 0 runs).  The results agree to
  *    rounding; the choice only changes the speed.                          */
 /*  BGW_OPT_UPDATE_ITEMS: column tiles per work item of the tensor-core
  *    sweep's bulk update launches.  -1 (default): the SM-count rule, items

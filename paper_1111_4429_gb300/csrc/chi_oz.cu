@@ -31,6 +31,10 @@
 // Shared memory: a three-deep ring of row-operand stages (64 KB: 8 digits x
 // 128 rows x 16 pairs) and a two-deep one of column-operand stages (16 KB).
 //
+// Bound by the tensor pipe (62 % active at N_G 2120, K 6400, 3.29 ms): one set of
+// level sums fills tensor memory, so between two segments it waits for them to be
+// read and joined (issue slots 9 %, ALU 7 %, L2 hits 83 %).
+//
 // Measured (N_G 2120): K 25600 in 13.8 ms per call (412 ms by chi_f64_kernel),
 // of it 12.7 ms here and 0.9 ms for the maximum and digit passes; K 2400 in
 // 1.5 ms (38.6 ms).  Relative error against quad-precision sums, off-diagonal /
@@ -140,8 +144,10 @@ struct Sizes {
 
 // sz.col[g] = largest size over the pairs, sz.pair[p] = largest size over the
 // columns; *flag = 1 where a value is not finite or, found by the last CTA, the
-// pairs' sizes spread by more than kSpreadBits.  One pass over M (HBM bound).
-// grid (ceil(ng/64), strips of pairs), block 256 = 64 columns x 4 pairs.
+// pairs' sizes spread by more than kSpreadBits.  One pass over M.  grid
+// (ceil(ng/64), strips of pairs), block 256 = 64 columns x 4 pairs.  N_G 2120, 6400
+// pairs: 84 us, 2.6 TB/s, half the warps resident and the FP64 products 60 % of
+// their pipe (the pairs' sizes add 9 us to a call of 2400 pairs, 1453 -> 1461 us).
 template <int OP>
 __global__ void __launch_bounds__(256) colmax_kernel(const void* __restrict__ M, const double* __restrict__ fac,
                                                      const double2* __restrict__ wc, long long K, int ng,
@@ -223,8 +229,9 @@ __device__ __forceinline__ void store_digits(long long X0, long long X1, __half*
 // Digits of the pairs p0 .. p0 + K - 1 (padded with zeros to whole stages) of
 // every column, K-major: planes[a][g][...], a stage's 32 values being 16 real
 // and 16 imaginary parts of 16 pairs (kReal: 32 pairs).  32 x 32 tiles
-// transposed in shared memory; 16 bytes read and 32 written per value (HBM
-// bound).  grid (ceil(kpad/32), rows/32), block 256.
+// transposed in shared memory; 16 bytes read and 32 written per value.  N_G 2120,
+// 6400 pairs: 151 us, 4.0 TB/s, bound by the integer pipe (80 %).  grid
+// (ceil(kpad/32), rows/32), block 256.
 template <int OP>
 __global__ void __launch_bounds__(256) digits_kernel(const void* __restrict__ M, const double* __restrict__ fac,
                                                      const double2* __restrict__ wc, long long p0, long long K,

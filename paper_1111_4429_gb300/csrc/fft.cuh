@@ -59,7 +59,10 @@ template <typename T, int S> __device__ __forceinline__ cpx<T> mul_i(cpx<T> a) {
 // packed / all packed: 32^3 (N_G 2120) 0.0589, 0.0138 / 0.0530, 0.0112 / 0.0554,
 // 0.0117; 48^3 (7180) 0.2193, 0.0414 / 0.2123, 0.0376 / 0.2071, 0.0371; 40^3 (3911)
 // 0.1294, 0.0282 / 0.1314, 0.0292 / 0.1268, 0.0273; 64^3 (8765) 0.483, 0.0645 /
-// 0.478, 0.0745 / 0.480, 0.0553.  The passes wait for loads more than for issue
+// 0.478, 0.0745 / 0.480, 0.0553.  The lengths between, whole calls of 8192 pairs in
+// us: 10 67 / 66 / 66, 16 140 / 133 / 125, 20 307 / 285 / 283, 24 449 / 437 / 434, 30
+// 773 / 746 / 731, 36 1313 / 1264 / 1252, 50 4727 / 4797 / 4630, 60 5623 / 4950 / 4828
+// (8 and 12: within 2 % of each other).  The passes wait for loads more than for issue
 // slots (48^3: 0.71 of the instructions, 0.94 of the time).
 __host__ __device__ constexpr bool pack_all(int n) { return !(n == 8 || n == 32); }
 

@@ -246,7 +246,9 @@ __device__ __forceinline__ float2 ff_dot2(float2 v, float2 a1, float2 b1, float2
 // element at a fixed thread (the pivot's row and column as divergent branches)
 // and the reciprocal by the thread that also updates, 17.3 and 38.7 us; with
 // one barrier a pivot and no shared scaled column, 21 us in double FP32.
-// Element (i, j) of thread q in step s, kb x kb block; live = it owns one.
+//
+// sweep_element: element (i, j) in step s of the thread that holds (x, y) of the
+// smaller triangle.
 __device__ __forceinline__ void sweep_element(int x, int y, int s, int& i, int& j) {
   i = x + (x >= s ? 1 : 0);
   j = y + (y >= s ? 1 : 0);

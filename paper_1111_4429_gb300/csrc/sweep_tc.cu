@@ -22,8 +22,10 @@
 // FP64 inputs (the plain path) join the seven exact level sums in integers
 // instead: a 64-bit integer of unit 2^-55 sigma_i tau_j holds the sum but for
 // its last nine bits, and is rounded to FP64 once.  What is left of the error
-// is the dropped levels' (near 2^-55 sigma_i tau_j), below the roundings of 32
-// complex FMAs and their subtraction.
+// is the dropped levels' and the operands' last bits (near 2^-55 sigma_i tau_j, at
+// worst 2^-49).  An FMA chain errs relative to the sum of |P_ik C_jk|, which is
+// smaller where the large entries of rows i and j lie at different k, so the inner
+// indices are balanced before the cut (panel_slice_kernel, slice_general_kernel).
 #include <cuda.h>
 #include <cuda_fp16.h>
 
