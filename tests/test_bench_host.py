@@ -79,6 +79,31 @@ def test_roofline_record(size, dominant, bound):
         assert roof["peak"] == pytest.approx(bench.FP32_PEAK_TFLOPS)
 
 
+@pytest.mark.parametrize("dominant", ["pair_yxpass", "chi_tc"])
+def test_fp64_roofline_record(dominant):
+    # the plain FP64 solve: transforms against the FP64 pipe on the alias-free grid, chi by its digit products
+    s = _shape("c1")
+    p = synth.CONFIGS["c1"]
+    bvec, _ = synth.cubic_cell(p["a"])
+    s.gv = synth.gsphere(bvec, (0.1, 0.0, 0.0), p["ecut_wfn"])
+    s.gc = synth.gsphere(bvec, (0.0, 0.0, 0.0), p["ecut_wfn"])
+    peaks = {"hbm_gbs": 6775.6, "bf16_tflops": 1939.0, "bf16_tflops_sustained": 1737.8}
+    kt = _kt(dominant)
+    roof = bench._roofline(s, kt, 375.0, peaks, "measured", size_tag="c1", fp64=True)
+    assert roof["frac"] == pytest.approx(roof["achieved"] / roof["peak"])
+    if dominant == "pair_yxpass":
+        assert roof["peak"] == pytest.approx(bench.FP64_PEAK_TFLOPS) and roof["traffic"] is None
+        n = bench.alias_free_points(s)
+        need = int((np.abs(s.gv).max(0) + np.abs(s.gc).max(0) + np.abs(s.geps).max(0)).max()) + 1
+        assert need <= n <= s.fft
+        assert roof["achieved"] == pytest.approx(bench.mtxel_flops(s, n)[0] / ((150.0 + 15.0 + 3.6) / 1e3) / 1e12)
+    else:
+        assert roof["peak"] == peaks["bf16_tflops_sustained"] and roof["traffic"] > 0
+        tiles = sum(1 for i in range((s.ng + 127) // 128) for j in range((s.ng + 31) // 32) if 32 * j <= 128 * i + 127)
+        issued = tiles * 36 * 4 * 2.0 * 128 * 32 * s.npairs   # a multiple of 16 pairs
+        assert s.npairs % 16 == 0 and roof["achieved"] == pytest.approx(issued / 0.15 / 1e12)
+
+
 def test_traffic_records_are_unique():
     # one record per tag, so an edited summary cannot leave a stale twin
     import glob
